@@ -42,7 +42,6 @@ enum : int {
     CTRL_M = 10,         // number of BVH leaves
     CTRL_NCELLS = 11,    // number of dense cells (DenseBox)
     CTRL_WORK_PRE = 12,  // work counters of the persistent traversal kernels
-    CTRL_WORK_MAIN = 13,
     CTRL_KIND_COUNT = 16,  // 3 words: leaves per kind (0 tile, 1 solid tile, 2 dense cell leaf)
     CTRL_KIND_FILL = 19,   // 3 words: fill counters of the per-kind leaf lists
     CTRL_KIND_WORK = 22,   // 3 words: work counters of the per-kind main kernels
@@ -232,7 +231,7 @@ struct ClusterArgs {
     const void* nodes;     // m-1 node records
     const void* nodebox;   // 2m-1 boxes (leaf boxes at m-1+l)
     const int2* leafr;     // m leaf records
-    uint8_t* lsolid;       // m: 1 if all points of the leaf are core and in one set
+    uint8_t* lsolid;       // m: the leaf's flag (nothing to do, all points core and in one set, neither)
     int32_t* klist;        // m: leaf indices grouped by kind
     const uint8_t* pdense; // n or null: dense-cell flags per sorted point (DenseBox)
     const int32_t* dstart; // n or null: first point of each point's dense cell

@@ -5,37 +5,44 @@
 // Work is organised per BVH leaf and per warp: a leaf is either a tile of up
 // to 32 sorted points outside dense cells (one point per lane) or a whole
 // dense cell (Sec. 4.2). A warp takes the next leaf from a global counter
-// (persistent kernels), and its 32 lanes traverse the tree together with one
-// shared stack: at each node every lane tests its own point against both
-// children's boxes (stored in the node record) and the warp descends where
-// any lane hits. At a leaf, pairs are tested either lane-per-query (looping
-// over the leaf's points) or lane-per-leaf-point (looping over the queries
-// that reached the leaf), whichever needs fewer steps.
+// (persistent kernels) and goes through the leaves within eps of it, 32 at a
+// time, one per lane: from the leaf's list, or from a walk of the tree that
+// expands up to 32 nodes a step. Those that pass the lane's test give their
+// points in one stream, one per lane; the points near the query box are
+// staged, and a full stage is tested against the tile's points.
 //
-// Two exact shortcuts cut the pair tests in dense regions:
-//  * containment: when the farthest corner of a leaf's box is within eps of a
-//    query, every point of the leaf is a neighbour (no per-point tests);
+// Exact shortcuts cut the pair tests in dense regions:
+//  * containment: when the farthest corners of a leaf's box and the query box
+//    are within eps, every pair between them is (no per-point tests);
 //  * solid leaves: a leaf whose points are all core and already one set
-//    (every dense cell, and every tile that becomes so after its own pairs
-//    are united) behaves like a dense cell of Sec. 4.2: one adjacent pair
-//    decides, and nothing is tested when the two sides already share a root.
+//    (every dense cell, and every tile that becomes so) behaves like a dense
+//    cell of Sec. 4.2: one adjacent pair decides;
+//  * sets: a pair whose points shared a set at any time needs no test (sets
+//    never split). Consecutive leaves are united first (link_next), so that
+//    dense regions start the main phase as a few sets.
 //
 // Preprocessing (minPts > 2 only): each point outside dense cells counts its
 // neighbours (itself included) and stops at minPts; points of dense cells are
 // core by construction.
-// Intra: each tile unites its own pairs and records whether it is solid.
+// Intra: each tile unites its own pairs, records whether it is solid, and is
+// united with the next leaf.
 // Main: each leaf visits only the leaves with index > its own (the pair mask
 // of Sec. 4.1, Figure "pair traversal"), so every pair is seen once, and
 // applies the rule of Algorithm 3 as it finds each pair, with no neighbour
 // list: core-core pairs are united, a core point claims a non-core neighbour
 // with one compare-and-swap (Sec. 3.2).
+#include <climits>
+
 #include "build.cuh"
 
 namespace gbd {
 
 namespace {
 
-constexpr int STACK = 128;  // > the largest possible tree depth (97 for 64-bit keys + index tie-break)
+constexpr int TREE_DEPTH = 97;    // the largest possible tree depth (64-bit keys and an index tie-break)
+constexpr int STACK = 384;        // a walk's stack: wide steps, which add up to 32 entries, up to STACK_WIDE,
+constexpr int STACK_WIDE = 224;   // then one node a step, whose depth-first growth stays below the tree depth
+static_assert(STACK_WIDE + 32 + TREE_DEPTH < STACK, "a walk's stack");
 
 // Node access and the box tests of both children at once (packed pairs: the
 // left child in the low half, the right child in the high half). The general
@@ -223,6 +230,13 @@ template <int D> struct __align__(16) SoA {
 #pragma unroll
         for (int k = 0; k < D; ++k) c[k][l] = p.c[k];
     }
+    __device__ __forceinline__ typename Traits<D>::Point get(int l) const
+    {
+        typename Traits<D>::Point p{};
+#pragma unroll
+        for (int k = 0; k < D; ++k) p.c[k] = c[k][l];
+        return p;
+    }
     __device__ __forceinline__ void d2pair(const typename NB<D>::PP& p, int u, float& d0, float& d1) const
     {
         GBD_COUNT(CNT_DIST, 2);
@@ -243,6 +257,7 @@ template <int D> struct __align__(16) SoA {
 template <> struct __align__(16) SoA<3> {
     float x[32], y[32], z[32];
     __device__ __forceinline__ void put(int l, const float4& p) { x[l] = p.x; y[l] = p.y; z[l] = p.z; }
+    __device__ __forceinline__ float4 get(int l) const { return make_float4(x[l], y[l], z[l], 0.f); }
     // dist2(p, point u) and dist2(p, point u + 1) for even u (p packed)
     __device__ __forceinline__ void d2pair(const NB<3>::PP& p, int u, float& d0, float& d1) const
     {
@@ -260,6 +275,7 @@ template <> struct __align__(16) SoA<3> {
 template <> struct __align__(16) SoA<2> {
     float x[32], y[32];
     __device__ __forceinline__ void put(int l, const float2& p) { x[l] = p.x; y[l] = p.y; }
+    __device__ __forceinline__ float2 get(int l) const { return make_float2(x[l], y[l]); }
     __device__ __forceinline__ void d2pair(const NB<2>::PP& p, int u, float& d0, float& d1) const
     {
         GBD_COUNT(CNT_DIST, 2);
@@ -272,71 +288,6 @@ template <> struct __align__(16) SoA<2> {
     __device__ __forceinline__ float d2(const float2& p, int u) const { return dist2(p, make_float2(x[u], y[u])); }
 };
 
-template <int D>
-struct WarpMem {
-    SoA<D> soa;
-    typename Traits<D>::Point buf[32];
-    int stack[STACK];
-    uint8_t cbuf[32];
-};
-
-// Warp-cooperative stack traversal from internal node `node` with sp
-// entries already on the stack. Children whose last leaf is below
-// v.mask_lo are never entered (the pair mask). v.leaf(L, mask, box) gets the
-// lanes that reached leaf L and its box; it returns true to stop early.
-template <int D, class V>
-__device__ __forceinline__ void traverse_loop(const typename Traits<D>::Node* __restrict__ nodes, int64_t m, V& v,
-                                              int* stack, uint32_t* ctrl, int node, int sp)
-{
-    const int lane = threadIdx.x & 31;
-    const int leaf0 = (int)(m - 1);
-    // a traversal enters each internal node at most once; more steps than
-    // that can only come from a corrupt tree: flag it and stop
-    int64_t steps = 0;
-    for (;;) {
-        if (++steps > m) {
-            if (lane == 0) atomicOr(&ctrl[CTRL_ERR], ERR_STACK);
-            return;
-        }
-        const auto nd = NB<D>::load(nodes, node);
-        GBD_COUNT(CNT_NODE, lane == 0);
-        bool hl, hr;
-        v.hits(nd, hl, hr);
-        const unsigned ml = nd.m.z >= v.mask_lo ? __ballot_sync(FULL, hl) : 0u;
-        const unsigned mr = nd.m.w >= v.mask_lo ? __ballot_sync(FULL, hr) : 0u;
-        int next = -1;
-        // left child, then right child; one call site of v.leaf keeps the
-        // kernel's code small
-#pragma unroll 1
-        for (int c = 0; c < 2; ++c) {
-            const unsigned mk = c ? mr : ml;
-            if (!mk) continue;
-            const int child = c ? nd.m.y : nd.m.x;
-            if (child >= leaf0) {
-                GBD_COUNT(CNT_LEAF, lane == 0);
-                if (v.leaf(child - leaf0, mk, c ? NB<D>::box_r(nd) : NB<D>::box_l(nd))) return;
-            } else if (next < 0) {
-                next = child;
-            } else {
-                if (sp >= STACK) {
-                    if (lane == 0) atomicOr(&ctrl[CTRL_ERR], ERR_STACK);
-                    return;
-                }
-                if (lane == 0) stack[sp] = child;
-                ++sp;
-            }
-        }
-        if (next < 0) {
-            if (sp == 0) return;
-            __syncwarp();
-            next = stack[--sp];
-        }
-        node = next;
-    }
-}
-
-// The traversal of one leaf's points from node `start` (an internal node,
-// or the leaf itself when it is a whole tree).
 // a node or leaf box: one 256-bit load where it is a 32-byte record (2D, 3D)
 template <int D>
 __device__ __forceinline__ typename Traits<D>::Box load_box(const typename Traits<D>::Box* __restrict__ nodebox,
@@ -348,66 +299,82 @@ __device__ __forceinline__ typename Traits<D>::Box load_box(const typename Trait
     return b;
 }
 
-template <int D, class V>
-__device__ __forceinline__ void traverse(const typename Traits<D>::Node* __restrict__ nodes,
-                                         const typename Traits<D>::Box* __restrict__ nodebox, int64_t m, V& v,
-                                         int* stack, uint32_t* ctrl, int start)
-{
-    const int leaf0 = (int)(m - 1);
-    if (start >= leaf0) {
-        typename Traits<D>::Box b;
-        b.lo = nodebox[start].lo;
-        b.hi = nodebox[start].hi;
-        v.leaf(start - leaf0, v.root_mask(), b);
-        return;
-    }
-    traverse_loop<D>(nodes, m, v, stack, ctrl, start, 0);
-}
+// The points of up to 32 leaves (one per lane with `on`: [us, ue)) in one
+// stream, in lane order and ascending within a leaf: each lane gets one point
+// a step, whatever the sizes of the leaves, and the next step's points are
+// loaded while the current ones are looked at. Visiting the leaves one by one
+// cost a chain of dependent loads for each, with a third of the lanes idle.
+// (PointStream needs a leaf with `on` in some lane.)
+struct StreamMem {
+    int us[32];
+    int off[32];
+};
 
-// The traversal of one leaf's points from the subtrees roots[0 .. n) (node,
-// last leaf): the siblings along the leaf's path to its start node whose
-// boxes come within eps of the leaf box. Every neighbour of the leaf's points
-// outside the leaf lies in one of them (k_tile_start), so the path nodes
-// themselves are not visited. Roots whose leaves all precede v.mask_lo are
-// skipped; leaf roots are tested lane by lane against their box.
-template <int D, class V>
-__device__ __forceinline__ void traverse_roots(const typename Traits<D>::Node* __restrict__ nodes,
-                                               const typename Traits<D>::Box* __restrict__ nodebox, int64_t m,
-                                               V& v, int* stack, uint32_t* ctrl, const int2* __restrict__ roots,
-                                               int n)
-{
-    const int lane = threadIdx.x & 31;
-    const int leaf0 = (int)(m - 1);
-    int sp = 0;
-    for (int j = n - 1; j >= 0; --j) {  // pushed in reverse: the nearest sibling is taken first
-        const int2 r = roots[j];
-        if (r.y < v.mask_lo) continue;
-        if (r.x >= leaf0) {
-            typename Traits<D>::Box b;
-            b.lo = nodebox[r.x].lo;
-            b.hi = nodebox[r.x].hi;
-            const unsigned mk = __ballot_sync(FULL, v.hit_box(b));
-            GBD_COUNT(CNT_LEAF, lane == 0 && mk);
-            if (mk && v.leaf(r.x - leaf0, mk, b)) return;
-        } else {
-            if (lane == 0) stack[sp] = r.x;
-            ++sp;
+template <int D>
+struct PointStream {
+    using P = typename Traits<D>::Point;
+    const P* __restrict__ sp;
+    StreamMem& st;
+    int off;       // first position of this lane's leaf in the stream (no leaf: past its end)
+    int total;
+    int before;    // leaves that start before the current 32 positions, less one
+    int b;         // the step's first position
+    int lane;
+    // this lane's point of the step (in: it has one), and the next step's
+    bool in;
+    int j, jn;
+    P p, pn;
+
+    __device__ __forceinline__ PointStream(const P* sp_, StreamMem& st_, bool on, int us, int ue, int lane_)
+        : sp(sp_), st(st_), lane(lane_)
+    {
+        const int size = on ? ue - us : 0;
+        off = size;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, off, o);
+            if (lane >= o) off += y;
         }
+        total = __shfl_sync(FULL, off, 31);
+        off -= size;
+        const unsigned om = __ballot_sync(FULL, on);
+        __syncwarp();
+        if (on) {
+            const int r = __popc(om & ((1u << lane) - 1u));
+            st.us[r] = us;
+            st.off[r] = off;
+        } else {
+            off = total;
+        }
+        __syncwarp();
+        before = -1;
+        b = -32;
+        load(0);
     }
-    if (sp == 0) return;
-    __syncwarp();
-    const int node = stack[--sp];
-    traverse_loop<D>(nodes, m, v, stack, ctrl, node, sp);
-}
+    __device__ __forceinline__ void load(int at)
+    {
+        const unsigned sm = __reduce_or_sync(FULL, (unsigned)(off - at) < 32u && off < total ? 1u << (off - at) : 0u);
+        const int r = before + __popc(sm & (0xffffffffu >> (31 - lane)));
+        before += __popc(sm);
+        jn = at + lane < total ? st.us[r] + (at + lane - st.off[r]) : st.us[0];
+        pn = sp[jn];
+    }
+    __device__ __forceinline__ bool next()
+    {
+        b += 32;
+        in = b + lane < total;
+        j = jn;
+        p = pn;
+        if (b + 32 < total) load(b + 32);
+        return b < total;
+    }
+};
 
 // per leaf: at most SIBCAP sibling subtrees are recorded (more: the start
 // node is used instead), and at most LEAFCAP leaves within eps
 constexpr int SIBCAP = TRAVERSAL_SIBCAP;
 constexpr int LEAFCAP = TRAVERSAL_LEAFCAP;
 
-// ---------------------------------------------------------------------------
-// Preprocessing visitor: count neighbours up to minPts (Sec. 3.2, 4.1, 4.2).
-// ---------------------------------------------------------------------------
 // The bounding box of the points of the lanes with `on` (empty if none): a
 // query box for all of them at once. For p inside it every per-axis gap to a
 // box is at least the box-to-box gap (monotone rounding, same order of the
@@ -425,518 +392,14 @@ __device__ __forceinline__ typename Traits<D>::Box warp_box(const typename Trait
 // the lanes of a tile of k <= 32 points
 __device__ __forceinline__ unsigned tile_lanes(int k) { return k >= 32 ? FULL : ((1u << k) - 1u); }
 
+// Per-warp shared memory of both phases.
 template <int D>
-struct PreV {
-    using T = Traits<D>;
-    using P = typename T::Point;
-    const P* __restrict__ sp;
-    const int2* __restrict__ leafr;
-    SoA<D>* soa;
-    float e2;
-    int min_pts;
-    int mask_lo;
-    int own;  // the query tile's own leaf, already counted
-    int lane;
-    P p;
-    bool act;
-    int cnt;
-    // neighbour lists (null: none): lane l's query (point qs + l) records
-    // its out-of-tile neighbours while its count is below minPts, so a query
-    // that ends non-core has all of them (nl <= minPts - 1 = lcap)
-    int32_t* nlist;
-    int lcap;
-    int qs;
-    int nl;
-
-    __device__ __forceinline__ void note(int idx)
-    {
-        if (nl < lcap) nlist[(int64_t)(qs + lane) * lcap + nl] = idx;
-        ++nl;
-    }
-
-    typename NB<D>::PP pp;  // p, packed
-
-    __device__ __forceinline__ void hits(const typename T::Node& n, bool& hl, bool& hr) const
-    {
-        float dl, dr;
-        NB<D>::pd2(n, pp, dl, dr);
-        hl = act && dl <= e2;
-        hr = act && dr <= e2;
-    }
-    __device__ __forceinline__ bool hit_box(const typename T::Box& b) const { return act && NB<D>::pbox(p, b) <= e2; }
-    __device__ __forceinline__ unsigned root_mask() const { return __ballot_sync(FULL, act); }
-    // list entries are worth a first test against the box of the active queries
-    static constexpr bool PREFILTER = true;
-    static constexpr bool NEEDS_SOLID = false;
-    // the box of the queries active when the walk starts (set before it;
-    // queries only drop out, so it stays a bound for those still counting)
-    typename T::Box qbox;
-    __device__ __forceinline__ typename T::Box query_box() const { return qbox; }
-
-    __device__ __forceinline__ bool leaf(int L, unsigned mask, const typename T::Box& box)
-    {
-        return leaf_rec(L, mask, box, __ldg(&leafr[L]), 0);
-    }
-    // the same with the leaf's record (start, end) already loaded
-    __device__ bool leaf_rec(int L, unsigned mask, const typename T::Box& box, int2 r, int)
-    {
-        if (L == own) return false;
-        const int s = r.x, e = r.y & 0x7fffffff;
-        mask &= __ballot_sync(FULL, act);
-        // the whole leaf within eps: count it at once
-        const bool cont = ((mask >> lane) & 1u) && T::far_dist2(p, box) <= e2;
-        if (cont) {
-            cnt += e - s;
-            if (cnt >= min_pts) act = false;
-            else if (nlist)
-                for (int u = s; u < e; ++u) note(u);
-        }
-        mask &= ~__ballot_sync(FULL, cont);
-        for (int c = s; c < e && mask; c += 32) {
-            const int k = min(32, e - c);
-            if (__popc(mask) < k) {
-                // lane per leaf point, looping over the queries in `mask`
-                const bool in = lane < k;
-                const P rp = in ? sp[c + lane] : sp[c];
-                unsigned mm = mask;
-                while (mm) {
-                    const int q = __ffs(mm) - 1;
-                    mm &= mm - 1;
-                    const P pq = NB<D>::shfl(p, q);
-                    const unsigned h = __ballot_sync(FULL, in && dist2(pq, rp) <= e2);
-                    if (!h) continue;  // the common case in sparse regions: nothing to record
-                    if (nlist) {
-                        // each hit leaf point writes itself into q's list
-                        const int at = __shfl_sync(FULL, nl, q) + __popc(h & ((1u << lane) - 1u));
-                        if (((h >> lane) & 1u) && at < lcap) nlist[(int64_t)(qs + q) * lcap + at] = c + lane;
-                    }
-                    if (lane == q) {
-                        cnt += __popc(h);
-                        nl += __popc(h);
-                        if (cnt >= min_pts) act = false;
-                    }
-                }
-            } else {
-                // lane per query, looping over the staged leaf points two
-                // at a time (packed); a count that reaches minPts stops
-                if (lane < k) soa->put(lane, sp[c + lane]);
-                __syncwarp();
-                if ((mask >> lane) & 1u) {
-                    int u = 0;
-                    for (; u + 1 < k && act; u += 2) {
-                        float d0, d1;
-                        soa->d2pair(pp, u, d0, d1);
-                        if (d0 <= e2) {
-                            if (nlist) note(c + u);
-                            if (++cnt >= min_pts) act = false;
-                        }
-                        if (d1 <= e2 && act) {
-                            if (nlist) note(c + u + 1);
-                            if (++cnt >= min_pts) act = false;
-                        }
-                    }
-                    if (u < k && act && soa->d2(p, u) <= e2) {
-                        if (nlist) note(c + u);
-                        if (++cnt >= min_pts) act = false;
-                    }
-                }
-                __syncwarp();
-            }
-            mask &= __ballot_sync(FULL, act);
-        }
-        return !__any_sync(FULL, act);
-    }
-};
-
-// ---------------------------------------------------------------------------
-// The pair rule of Algorithm 3 (Sec. 3.2), for a pair (a, b) within eps.
-// ---------------------------------------------------------------------------
-struct Rule {
-    int* labels;
-    uint8_t* core;
-    int min_pts;
-    // core-to-non-core claims: DBSCAN mode, and no preprocessing lists (with
-    // lists every border point has already claimed a core neighbour)
-    bool claims;
-
-    __device__ __forceinline__ void unite(int a, int b) const
-    {
-        if (__ldcg(labels + a) == __ldcg(labels + b)) return;  // same parent: same set
-        uf_union(labels, a, b);
-    }
-    // pair() with a per-lane memo of the last core partner's parent: a
-    // partner with the same parent is in a set already united with a (sets
-    // never split), so the union is skipped. Partners come in sorted order and
-    // mostly share an intra-tile root, so most unions are skipped this way.
-    __device__ __forceinline__ void pair_memo(int a, bool acore, int b, bool bcore, int& last) const
-    {
-        if (min_pts <= 2 || (acore && bcore)) {
-            if (min_pts == 2) { core[a] = 1; core[b] = 1; }
-            const int lb = __ldcg(labels + b);
-            if (lb == last) return;
-            unite(a, b);
-            last = lb;
-        } else if (claims) {
-            if (acore) uf_claim(labels, b, a);
-            else if (bcore) uf_claim(labels, a, b);
-        }
-    }
-    // would point x (core flag xcore) change anything by joining the solid
-    // leaf whose first point is s?
-    __device__ __forceinline__ bool need_solid(int x, bool xcore, int s) const
-    {
-        if (min_pts <= 2 || xcore) {
-            int a = x, b = s;
-            uf_find2(labels, a, b);
-            return a != b;
-        }
-        return claims && __ldcg(labels + x) == x;
-    }
-    __device__ __forceinline__ void join_solid(int x, bool xcore, int s) const
-    {
-        if (min_pts <= 2 || xcore) {
-            if (min_pts == 2) core[x] = 1;
-            uf_union(labels, x, s);
-        } else {
-            uf_claim(labels, x, s);
-        }
-    }
-};
-
-// Main visitor for a tile that is not solid (one point per lane).
-template <int D>
-struct MainPtV {
-    using T = Traits<D>;
-    using P = typename T::Point;
-    const P* __restrict__ sp;
-    const int2* __restrict__ leafr;
-    const uint8_t* __restrict__ lsolid;
-    const uint8_t* core;
-    SoA<D>* soa;
-    uint8_t* cbuf;
-    Rule rule;
-    float e2;
-    int mask_lo;  // = own leaf index + 1: only leaves after this one
-    int lane;
-    int sQ;       // first point of own leaf
-    P p;
-    int q;
-    bool valid;
-    bool qcore;
-    int last = -1;  // pair_memo state of this lane's query
-
-    typename NB<D>::PP pp;  // p, packed
-
-    __device__ __forceinline__ void hits(const typename T::Node& n, bool& hl, bool& hr) const
-    {
-        float dl, dr;
-        NB<D>::pd2(n, pp, dl, dr);
-        hl = valid && dl <= e2;
-        hr = valid && dr <= e2;
-    }
-    __device__ __forceinline__ bool hit_box(const typename T::Box& b) const { return valid && NB<D>::pbox(p, b) <= e2; }
-    static constexpr bool PREFILTER = true;
-    static constexpr bool NEEDS_SOLID = true;
-    typename T::Box qbox;  // the box of the valid queries (set before the walk)
-    __device__ __forceinline__ typename T::Box query_box() const { return qbox; }
-    __device__ __forceinline__ unsigned root_mask() const { return __ballot_sync(FULL, valid); }
-
-    __device__ __forceinline__ bool leaf(int L, unsigned mask, const typename T::Box& box)
-    {
-        return leaf_rec(L, mask, box, __ldg(&leafr[L]), lsolid[L]);
-    }
-    // the same with the leaf's record and solid flag already loaded
-    __device__ bool leaf_rec(int L, unsigned mask, const typename T::Box& box, int2 r, int solid)
-    {
-        if (L < mask_lo) return false;
-        const int s = r.x, e = r.y & 0x7fffffff;
-        const bool cont = ((mask >> lane) & 1u) && T::far_dist2(p, box) <= e2;
-        if (!solid) {
-            const int k = e - s;
-            if (__popc(mask) < k) {
-                const bool in = lane < k;
-                const int ri = s + lane;
-                const P rp = in ? sp[ri] : sp[s];
-                const bool rc = in && core[ri];
-                int rlast = -1;  // pair_memo state of this lane's leaf point
-                unsigned mm = mask;
-                while (mm) {
-                    const int qq = __ffs(mm) - 1;
-                    mm &= mm - 1;
-                    const P pq = NB<D>::shfl(p, qq);
-                    const bool qc = __shfl_sync(FULL, qcore, qq);
-                    const bool qcont = __shfl_sync(FULL, cont, qq);
-                    if (in && (qcont || dist2(pq, rp) <= e2)) rule.pair_memo(ri, rc, sQ + qq, qc, rlast);
-                    __syncwarp();
-                }
-            } else {
-                if (lane < k) { soa->put(lane, sp[s + lane]); cbuf[lane] = core[s + lane]; }
-                __syncwarp();
-                if ((mask >> lane) & 1u) {
-                    if (cont) {
-                        for (int u = 0; u < k; ++u) rule.pair_memo(q, qcore, s + u, cbuf[u] != 0, last);
-                    } else {
-                        // two staged points at a time (packed)
-                        int u = 0;
-                        for (; u + 1 < k; u += 2) {
-                            float d0, d1;
-                            soa->d2pair(pp, u, d0, d1);
-                            if (d0 <= e2) rule.pair_memo(q, qcore, s + u, cbuf[u] != 0, last);
-                            if (d1 <= e2) rule.pair_memo(q, qcore, s + u + 1, cbuf[u + 1] != 0, last);
-                        }
-                        if (u < k && soa->d2(p, u) <= e2) rule.pair_memo(q, qcore, s + u, cbuf[u] != 0, last);
-                    }
-                }
-                __syncwarp();
-            }
-            return false;
-        }
-        // solid leaf: one adjacent point decides (its points are all core and
-        // already one set rooted at that of its first point s)
-        const bool need = ((mask >> lane) & 1u) && rule.need_solid(q, qcore, s);
-        if (need && cont) rule.join_solid(q, qcore, s);
-        unsigned nm = __ballot_sync(FULL, need && !cont);
-        if (nm) {
-            // the leaf's points in chunks, each pruned to those within eps of
-            // the box of the queries (exact, reading 3); each query still
-            // looking is tested against the survivors until it finds one
-            for (int c = s; c < e && nm; c += 32) {
-                const int j = c + lane;
-                const P rp = j < e ? sp[j] : sp[c];
-                const bool keep = j < e && NB<D>::pbox(rp, qbox) <= e2;
-                if (!__any_sync(FULL, keep)) continue;
-                unsigned mm = nm;
-                while (mm) {
-                    const int qq = __ffs(mm) - 1;
-                    mm &= mm - 1;
-                    const P pq = NB<D>::shfl(p, qq);
-                    if (__any_sync(FULL, keep && dist2(pq, rp) <= e2)) {
-                        if (lane == qq) rule.join_solid(q, qcore, s);
-                        nm &= ~(1u << qq);
-                    }
-                }
-                __syncwarp();
-            }
-        }
-        return false;
-    }
-};
-
-// Main visitor for a solid tile (one point per lane, all core, one set): the
-// traversal keeps per-lane point tests; at a leaf one adjacent pair decides.
-template <int D>
-struct MainSolidV {
-    using T = Traits<D>;
-    using P = typename T::Point;
-    const P* __restrict__ sp;
-    const int2* __restrict__ leafr;
-    const uint8_t* __restrict__ lsolid;
-    const uint8_t* core;
-    P* buf;
-    Rule rule;
-    float e2;
-    int mask_lo;  // = own leaf index + 1
-    int lane;
-    int sQ;
-    P p;
-    bool valid;
-    typename T::Box qb;
-
-    typename NB<D>::PP pp;  // p, packed
-
-    __device__ __forceinline__ void hits(const typename T::Node& n, bool& hl, bool& hr) const
-    {
-        float dl, dr;
-        NB<D>::pd2(n, pp, dl, dr);
-        hl = valid && dl <= e2;
-        hr = valid && dr <= e2;
-    }
-    __device__ __forceinline__ bool hit_box(const typename T::Box& b) const { return valid && NB<D>::pbox(p, b) <= e2; }
-    // the query box is the leaf box, which every listed leaf passes
-    static constexpr bool PREFILTER = false;
-    __device__ __forceinline__ typename T::Box query_box() const { return qb; }
-    __device__ __forceinline__ unsigned root_mask() const { return __ballot_sync(FULL, valid); }
-
-    __device__ bool leaf(int L, unsigned mask, const typename T::Box& box)
-    {
-        if (L < mask_lo) return false;
-        const int2 r = __ldg(&leafr[L]);
-        const int s = r.x, e = r.y & 0x7fffffff;
-        if (lsolid[L]) {
-            int same = 0;
-            if (lane == 0) {
-                int a = sQ, b = s;
-                uf_find2(rule.labels, a, b);
-                same = a == b;
-            }
-            if (__shfl_sync(FULL, same, 0)) return false;
-            const bool act = (mask >> lane) & 1u;
-            bool found = __any_sync(FULL, act && T::far_dist2(p, box) <= e2);
-            // only the leaf's points within eps of this tile's box can be
-            // partners (exact pruning, reading 3)
-            const unsigned lt = (1u << lane) - 1u;
-            for (int c = s; c < e && !found; c += 32) {
-                const int k = min(32, e - c);
-                const P rp = lane < k ? sp[c + lane] : sp[c];
-                const bool keep = lane < k && NB<D>::pbox(rp, qb) <= e2;
-                const unsigned km = __ballot_sync(FULL, keep);
-                if (!km) continue;
-                const int kk = __popc(km);
-                if (__popc(mask) < kk) {
-                    unsigned mm = mask;
-                    while (mm && !found) {
-                        const int qq = __ffs(mm) - 1;
-                        mm &= mm - 1;
-                        const P pq = NB<D>::shfl(p, qq);
-                        found = __any_sync(FULL, keep && dist2(pq, rp) <= e2);
-                    }
-                } else {
-                    if (keep) buf[__popc(km & lt)] = rp;
-                    __syncwarp();
-                    bool h = false;
-                    if (act)
-                        for (int u = 0; u < kk; ++u)
-                            if (dist2(p, buf[u]) <= e2) { h = true; break; }
-                    __syncwarp();
-                    found = __any_sync(FULL, h);
-                }
-            }
-            if (found && lane == 0) uf_union(rule.labels, sQ, s);
-            __syncwarp();
-            return false;
-        }
-        // a tile that is not solid: one lane per tile point
-        const int k = e - s;
-        const bool in = lane < k;
-        const int ri = s + lane;
-        const P rp = in ? sp[ri] : sp[s];
-        const bool rc = in && core[ri];
-        const bool need = in && rule.need_solid(ri, rc, sQ);
-        bool found = need && T::far_dist2(rp, qb) <= e2;
-        unsigned mm = mask;
-        while (mm && __any_sync(FULL, need && !found)) {
-            const int qq = __ffs(mm) - 1;
-            mm &= mm - 1;
-            const P pq = NB<D>::shfl(p, qq);
-            if (need && !found && dist2(rp, pq) <= e2) found = true;
-        }
-        if (need && found) rule.join_solid(ri, rc, sQ);
-        __syncwarp();
-        return false;
-    }
-};
-
-// Main visitor for a dense cell larger than a tile as the query:
-// its box is tested against the nodes; its points are all core and one set.
-template <int D>
-struct MainBoxV {
-    using T = Traits<D>;
-    using P = typename T::Point;
-    const P* __restrict__ sp;
-    const int2* __restrict__ leafr;
-    const uint8_t* __restrict__ lsolid;
-    const uint8_t* core;
-    P* buf;
-    Rule rule;
-    float e2;
-    int mask_lo;  // = own leaf index + 1
-    int lane;
-    int sQ, eQ;
-    typename T::Box qb;
-    // the cell's work can be split over `parts` warps: this one takes the
-    // neighbour leaves with L % parts == part
-    int part = 0, parts = 1;
-
-    __device__ __forceinline__ void hits(const typename T::Node& n, bool& hl, bool& hr) const
-    {
-        float dl, dr;
-        NB<D>::bd2(n, qb, dl, dr);
-        hl = dl <= e2;
-        hr = dr <= e2;
-    }
-    __device__ __forceinline__ bool hit_box(const typename T::Box& b) const { return NB<D>::bbox(qb, b) <= e2; }
-    // the query box is the leaf box, which every listed leaf passes
-    static constexpr bool PREFILTER = false;
-    __device__ __forceinline__ typename T::Box query_box() const { return qb; }
-    __device__ __forceinline__ unsigned root_mask() const { return FULL; }
-
-    __device__ bool leaf(int L, unsigned, const typename T::Box& box)
-    {
-        if (L < mask_lo || L % parts != part) return false;
-        const int2 r = __ldg(&leafr[L]);
-        const int s = r.x, e = r.y & 0x7fffffff;
-        const unsigned lt = (1u << lane) - 1u;
-        if (lsolid[L]) {
-            // solid against solid: any adjacent cross pair unites the two sets
-            int same = 0;
-            if (lane == 0) {
-                int a = sQ, b = s;
-                uf_find2(rule.labels, a, b);
-                same = a == b;
-            }
-            if (__shfl_sync(FULL, same, 0)) return false;
-            bool found = T::box_far2(qb, box) <= e2;
-            // only the cell's points within eps of the other leaf's box can
-            // have a partner there, and of the other leaf only the points
-            // within eps of the cell's box (exact pruning, reading 3); the
-            // survivors are compacted into the staging buffer
-            for (int cq = sQ; cq < eQ && !found; cq += 32) {
-                const int iq = cq + lane;
-                const bool inq = iq < eQ;
-                const P pq = inq ? sp[iq] : sp[sQ];
-                const bool near = inq && NB<D>::pbox(pq, box) <= e2;
-                if (!__any_sync(FULL, near)) continue;
-                for (int c = s; c < e; c += 32) {
-                    const int k = min(32, e - c);
-                    const P rp = lane < k ? sp[c + lane] : sp[c];
-                    const bool keep = lane < k && NB<D>::pbox(rp, qb) <= e2;
-                    const unsigned km = __ballot_sync(FULL, keep);
-                    if (!km) continue;
-                    if (keep) buf[__popc(km & lt)] = rp;
-                    __syncwarp();
-                    const int kk = __popc(km);
-                    bool h = false;
-                    if (near)
-                        for (int u = 0; u < kk; ++u)
-                            if (dist2(pq, buf[u]) <= e2) { h = true; break; }
-                    __syncwarp();
-                    if (__any_sync(FULL, h)) { found = true; break; }
-                }
-            }
-            if (found && lane == 0) uf_union(rule.labels, sQ, s);
-            __syncwarp();
-            return false;
-        }
-        // a tile that is not solid: one lane per tile point, against the
-        // cell's points within eps of the tile's box
-        const int k = e - s;
-        const bool in = lane < k;
-        const int ri = s + lane;
-        const P rp = in ? sp[ri] : sp[s];
-        const bool rc = in && core[ri];
-        const bool need = in && rule.need_solid(ri, rc, sQ);
-        bool found = need && T::far_dist2(rp, qb) <= e2;
-        if (__any_sync(FULL, need && !found)) {
-            for (int cq = sQ; cq < eQ; cq += 32) {
-                if (!__any_sync(FULL, need && !found)) break;
-                const int kq = min(32, eQ - cq);
-                const P ap = lane < kq ? sp[cq + lane] : sp[sQ];
-                const bool keep = lane < kq && NB<D>::pbox(ap, box) <= e2;
-                const unsigned km = __ballot_sync(FULL, keep);
-                if (!km) continue;
-                if (keep) buf[__popc(km & lt)] = ap;
-                __syncwarp();
-                const int kk = __popc(km);
-                if (need && !found)
-                    for (int u = 0; u < kk; ++u)
-                        if (dist2(rp, buf[u]) <= e2) { found = true; break; }
-                __syncwarp();
-            }
-        }
-        if (need && found) rule.join_solid(ri, rc, sQ);
-        __syncwarp();
-        return false;
-    }
+struct WarpMem {
+    SoA<D> soa;      // staged points
+    int idx[32];     // and their indices (main phase: top bit: not core)
+    StreamMem st;
+    int stack[STACK];
+    int cand[64];
 };
 
 template <int D>
@@ -963,13 +426,13 @@ struct DevArgs {
     const int32_t* mps;
     const int32_t* iroot;
     // per leaf: the node its traversals start at, and the sibling subtrees
-    // along the way that come within eps (k_tile_start)
+    // along the way that come within eps (tile_start)
     int32_t* tstart;
     int2* tsib;
     int8_t* tnsib;
     // multi-minPts runs: neighbour counts capped at min_pts (null otherwise)
     int32_t* ncount;
-    // per leaf: the leaves within eps of its box (k_leaf_lists; null: none)
+    // per leaf: the leaves within eps of its box (k_leaf_lists)
     int32_t* llist;
     int16_t* lcount;
 };
@@ -1012,66 +475,60 @@ __device__ __forceinline__ TileParams tile_params(const DevArgs<D>& a, int L)
 // box) then start at A instead of the root and skip the levels above it,
 // where only one path could lead to a neighbour.
 template <int D>
-__global__ void k_tile_start(DevArgs<D> a, const int32_t* __restrict__ parent, const int4* __restrict__ nmeta)
+__device__ __forceinline__ int tile_start(const DevArgs<D>& a, const int32_t* __restrict__ parent,
+                                          const int4* __restrict__ nmeta, int64_t L, int leaf0, const TileParams& tp,
+                                          const typename Traits<D>::Box& tb)
 {
-    using T = Traits<D>;
-    const int64_t m = a.ctrl[CTRL_M];
-    const int leaf0 = (int)(m - 1);
-    for (int64_t L = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; L < m; L += (int64_t)gridDim.x * blockDim.x) {
-        const TileParams tp = tile_params(a, (int)L);
-        int cur = leaf0 + (int)L;
-        int start = cur;
-        int ns = 0;  // siblings recorded (-1: more than SIBCAP)
-        int2* sib_out = a.tsib + L * SIBCAP;
-        const typename T::Box tb = load_box<D>(a.nodebox, cur);
-        // the depth of a tree over 64-bit keys with index tie-breaks is
-        // below STACK; a longer walk means a corrupt tree: start at the root
-        int steps = 0;
-        while (cur != tp.start) {
-            const int p = parent[cur];
-            if (p < 0 || ++steps > STACK) {
-                start = tp.start;
-                ns = -1;
-                break;
-            }
-            const int4 nm = nmeta[p];
-            const int sib = nm.x == cur ? nm.y : nm.x;
-            const typename T::Box sb = load_box<D>(a.nodebox, sib);
-            if (box_box<D>(tb, sb) <= tp.e2) {
-                start = p;
-                if (ns >= 0 && ns < SIBCAP) {
-                    // the sibling and the last leaf under it
-                    sib_out[ns++] = make_int2(sib, sib >= leaf0 ? sib - leaf0 : nmeta[sib].w);
-                } else {
-                    ns = -1;
-                }
-            }
-            cur = p;
+    int cur = leaf0 + (int)L;
+    int start = cur;
+    int ns = 0;  // siblings recorded (-1: more than SIBCAP)
+    int2* sib_out = a.tsib + L * SIBCAP;
+    // a longer climb than the tree is deep means a corrupt tree: start at the
+    // root
+    int steps = 0;
+    while (cur != tp.start) {
+        const int p = parent[cur];
+        if (p < 0 || ++steps > TREE_DEPTH) {
+            start = tp.start;
+            ns = -1;
+            break;
         }
-        a.tstart[L] = start;
-        a.tnsib[L] = (int8_t)ns;
+        const int4 nm = nmeta[p];
+        const int sib = nm.x == cur ? nm.y : nm.x;
+        const typename Traits<D>::Box sb = load_box<D>(a.nodebox, sib);
+        if (box_box<D>(tb, sb) <= tp.e2) {
+            start = p;
+            if (ns >= 0 && ns < SIBCAP) {
+                // the sibling and the last leaf under it
+                sib_out[ns++] = make_int2(sib, sib >= leaf0 ? sib - leaf0 : nmeta[sib].w);
+            } else {
+                ns = -1;
+            }
+        }
+        cur = p;
     }
+    a.tstart[L] = start;
+    a.tnsib[L] = (int8_t)ns;
+    return ns;
 }
 
-// the traversal of leaf L's points: from its recorded sibling subtrees, or
-// from its start node when it has more than SIBCAP of them
 // The leaves whose boxes come within eps of each leaf's box (itself
 // excluded), found once per leaf by one thread walking the subtrees recorded
-// by k_tile_start with the leaf box as the query (box-to-box test, exact by
+// by tile_start with the leaf box as the query (box-to-box test, exact by
 // the same monotone-rounding argument). Every neighbour of a point of the
 // leaf lies in one of them, so the traversals of both phases can go through
 // the list instead of the tree. More than LEAFCAP leaves: count -1, and the
-// phases walk the tree for that leaf.
+// phases walk the tree for that leaf (walk_next).
 // (each thread's walk stack lives in shared memory as column threadIdx.x of
 // [depth][LL_THREADS]: lanes at different depths still fall in distinct
 // banks, where a local-memory stack costs a transaction per distinct depth;
-// a walk deeper than LL_STACK gives up its list, and the phases walk the
-// tree for that leaf)
+// a walk deeper than LL_STACK gives up its list as well)
 constexpr int LL_THREADS = 256;
 constexpr int LL_STACK = 48;
 
 template <int D>
-__global__ void __launch_bounds__(LL_THREADS) k_leaf_lists(DevArgs<D> a)
+__global__ void __launch_bounds__(LL_THREADS)
+    k_leaf_lists(const __grid_constant__ DevArgs<D> a, const int32_t* __restrict__ parent, const int4* __restrict__ nmeta)
 {
     using T = Traits<D>;
     const int64_t m = a.ctrl[CTRL_M];
@@ -1084,7 +541,7 @@ __global__ void __launch_bounds__(LL_THREADS) k_leaf_lists(DevArgs<D> a)
         q = load_box<D>(a.nodebox, leaf0 + L);
         int32_t* out = a.llist + L * LEAFCAP;
         int cnt = 0, sp = 0;
-        const int ns = a.tnsib[L];
+        const int ns = tile_start<D>(a, parent, nmeta, L, leaf0, tp, q);
         if (ns >= 0) {
             for (int j = 0; j < ns; ++j) {
                 const int r = a.tsib[L * SIBCAP + j].x;
@@ -1098,7 +555,7 @@ __global__ void __launch_bounds__(LL_THREADS) k_leaf_lists(DevArgs<D> a)
                 }
             }
         } else {
-            cnt = LEAFCAP + 1;  // no recorded roots: the phases walk the tree
+            cnt = LEAFCAP + 1;
         }
         int64_t steps = 0;
         while (sp > 0 && cnt <= LEAFCAP) {
@@ -1131,70 +588,110 @@ __global__ void __launch_bounds__(LL_THREADS) k_leaf_lists(DevArgs<D> a)
     }
 }
 
-template <int D, class V>
-__device__ __forceinline__ void walk(const DevArgs<D>& a, int64_t m, V& v, int* stack, int L)
+// The roots of leaf L's walk onto an empty stack (the top is taken first):
+// its sibling leaves from the farthest ancestor down, then the sibling
+// subtrees from the nearest up, or the start node where there are more than
+// SIBCAP of them. Subtrees whose leaves all precede mask_lo are left out.
+template <int D>
+__device__ __forceinline__ int walk_roots(const DevArgs<D>& a, int L, int leaf0, int mask_lo, int* stack, int lane)
 {
-    const int lc = a.lcount ? a.lcount[L] : -1;
-    if (lc >= 0) {
-        // the leaf list, no tree walk. Per-point queries: each lane tests
-        // one listed leaf against the box of the warp's queries, then the
-        // leaves that pass are taken in list order with the lane-wise test
-        // of each query
-        const int leaf0 = (int)(m - 1);
-        const int lane = threadIdx.x & 31;
-        const int32_t* lst = a.llist + (int64_t)L * LEAFCAP;
-        if constexpr (!V::PREFILTER) {
-            for (int j = 0; j < lc; ++j) {
-                const int U = __ldg(&lst[j]);
-                if (U < v.mask_lo) continue;
-                typename Traits<D>::Box b;
-                b.lo = a.nodebox[leaf0 + U].lo;
-                b.hi = a.nodebox[leaf0 + U].hi;
-                const unsigned mk = __ballot_sync(FULL, v.hit_box(b));
-                GBD_COUNT(CNT_LEAF, lane == 0 && mk);
-                if (mk && v.leaf(U, mk, b)) return;
-            }
-        } else {
-            const typename Traits<D>::Box qb = v.query_box();
-            for (int j0 = 0; j0 < lc; j0 += 32) {
-                int U = -1, sol = 0;
-                int2 r = make_int2(0, 0);
-                bool cand = false;
-                if (j0 + lane < lc) {
-                    U = __ldg(&lst[j0 + lane]);
-                    if (U >= v.mask_lo) {
-                        typename Traits<D>::Box b;
-                        b.lo = a.nodebox[leaf0 + U].lo;
-                        b.hi = a.nodebox[leaf0 + U].hi;
-                        cand = NB<D>::bbox(qb, b) <= v.e2;
-                        // the records of all candidates in one lane-parallel load
-                        if (cand) {
-                            r = __ldg(&a.leafr[U]);
-                            if constexpr (V::NEEDS_SOLID) sol = a.lsolid[U];
-                        }
-                    }
-                }
-                unsigned cm = __ballot_sync(FULL, cand);
-                while (cm) {
-                    const int src = __ffs(cm) - 1;
-                    cm &= cm - 1;
-                    const int Us = __shfl_sync(FULL, U, src);
-                    const int2 rs = make_int2(__shfl_sync(FULL, r.x, src), __shfl_sync(FULL, r.y, src));
-                    const int ss = V::NEEDS_SOLID ? __shfl_sync(FULL, sol, src) : 0;
-                    typename Traits<D>::Box b;
-                    b.lo = a.nodebox[leaf0 + Us].lo;
-                    b.hi = a.nodebox[leaf0 + Us].hi;
-                    const unsigned mk = __ballot_sync(FULL, v.hit_box(b));
-                    GBD_COUNT(CNT_LEAF, lane == 0 && mk);
-                    if (mk && v.leaf_rec(Us, mk, b, rs, ss)) return;
-                }
-            }
-        }
-        return;
-    }
     const int ns = a.tnsib[L];
-    if (ns >= 0) traverse_roots<D>(a.nodes, a.nodebox, m, v, stack, a.ctrl, a.tsib + (int64_t)L * SIBCAP, ns);
-    else traverse<D>(a.nodes, a.nodebox, m, v, stack, a.ctrl, a.tstart[L]);
+    int item = -1;
+    if (ns >= 0) {
+        if (lane < ns) {
+            const int2 t = a.tsib[(int64_t)L * SIBCAP + lane];
+            if (t.y >= mask_lo) item = t.x;
+        }
+    } else if (lane == 0) {
+        item = a.tstart[L];
+    }
+    const unsigned lm = __ballot_sync(FULL, item >= leaf0), im = __ballot_sync(FULL, item >= 0 && item < leaf0);
+    const int sp = __popc(lm) + __popc(im);
+    const int pos = item >= leaf0 ? __popc(lm >> lane) - 1 : __popc(lm) + __popc(im & ((1u << lane) - 1u));
+    if (item >= 0) stack[sp - 1 - pos] = item;
+    __syncwarp();
+    return sp;
+}
+
+// A node's children within eps of the box q, in the order they are taken:
+// leaves before subtrees, left before right (-1: none)
+template <int D>
+__device__ __forceinline__ int2 near_children(const DevArgs<D>& a, int node, const typename Traits<D>::Box& q, float e2,
+                                              int leaf0, int mask_lo)
+{
+    const auto nd = NB<D>::load(a.nodes, node);
+    float dl, dr;
+    NB<D>::bd2(nd, q, dl, dr);
+    int l = dl <= e2 && nd.m.z >= mask_lo ? nd.m.x : -1;
+    int r = dr <= e2 && nd.m.w >= mask_lo ? nd.m.y : -1;
+    if (l < 0 || (l < leaf0 && r >= leaf0)) { const int t = l; l = r; r = t; }
+    return make_int2(l, r);
+}
+
+// Where a leaf has no list (more than LEAFCAP leaves within eps): the next
+// leaves of its walk through the tree, up to 32 of them into wm.cand (mask_lo:
+// only leaves from there on). Up to 32 nodes from the top of the stack are
+// expanded a step, each in place, so that the leaves come out in the order of
+// a walk that takes one node at a time -- whose chain of dependent loads, one
+// per node, was a third of the main phase on dense data. Returns how many
+// (fewer than 32: the walk is over).
+template <int D>
+__device__ __forceinline__ int walk_next(const DevArgs<D>& a, WarpMem<D>& wm, int& sp, int& nc, int64_t& steps,
+                                         int64_t m, const typename Traits<D>::Box& q, float e2, int mask_lo, int lane)
+{
+    const int leaf0 = (int)(m - 1);
+    const unsigned lt = (1u << lane) - 1u;
+#pragma unroll 1
+    while (sp > 0 && nc < 32) {
+        // each step enters a node or emits a leaf, each at most once; more
+        // steps can only come from a corrupt tree: flag it and stop
+        if (++steps > 2 * m) {
+            if (lane == 0) atomicOr(&a.ctrl[CTRL_ERR], ERR_STACK);
+            sp = 0;
+            break;
+        }
+        const int np = sp > STACK_WIDE ? 1 : min(sp, 32);
+        const int item = lane < np ? wm.stack[sp - 1 - lane] : -1;
+        __syncwarp();
+        // the leaves before the first subtree are next in order
+        const unsigned sub = __ballot_sync(FULL, item >= 0 && item < leaf0);
+        const int lead = sub ? __ffs(sub) - 1 : np;
+        const bool emit = lane < lead && item - leaf0 >= mask_lo;
+        const unsigned em = __ballot_sync(FULL, emit);
+        if (emit) wm.cand[nc + __popc(em & lt)] = item - leaf0;
+        nc += __popc(em);
+        // the others stay, subtrees replaced by their children
+        int2 c = make_int2(-1, -1);
+        if (lane >= lead && lane < np) {
+            GBD_COUNT(CNT_NODE, item < leaf0);
+            c = item >= leaf0 ? make_int2(item, -1) : near_children<D>(a, item, q, e2, leaf0, mask_lo);
+        }
+        const unsigned c1 = __ballot_sync(FULL, c.x >= 0), c2 = __ballot_sync(FULL, c.y >= 0);
+        sp += __popc(c1) + __popc(c2) - np;
+        if (sp > STACK) {
+            if (lane == 0) atomicOr(&a.ctrl[CTRL_ERR], ERR_STACK);
+            sp = 0;
+            break;
+        }
+        const int pos = sp - 1 - __popc(c1 & lt) - __popc(c2 & lt);
+        if (c.x >= 0) wm.stack[pos] = c.x;
+        if (c.y >= 0) wm.stack[pos - 1] = c.y;
+        __syncwarp();
+    }
+    return min(nc, 32);
+}
+
+// the leaves handed out by walk_next are done with: the rest moves up
+template <int D>
+__device__ __forceinline__ int walk_take(WarpMem<D>& wm, int& nc, int lane)
+{
+    const int U = lane < nc ? wm.cand[lane] : -1;
+    const int V = lane + 32 < nc ? wm.cand[lane + 32] : -1;
+    __syncwarp();
+    if (V >= 0) wm.cand[lane] = V;
+    nc = max(nc - 32, 0);
+    __syncwarp();
+    return U;
 }
 
 __device__ __forceinline__ int next_leaf(uint32_t* ctr)
@@ -1213,8 +710,212 @@ constexpr int traversal_regs()
     return D <= 3 ? 56 : (D <= 5 ? 96 : 128);
 }
 
+// (the main phase holds more state per lane and waits on union-find chains)
 template <int D>
-__global__ void __maxnreg__(traversal_regs<D>()) k_pre(DevArgs<D> a)
+constexpr int main_regs()
+{
+    return D <= 3 ? 64 : (D <= 5 ? 96 : 128);
+}
+
+// Preprocessing: each point outside dense cells counts its neighbours (itself
+// included) and stops at minPts (Sec. 3.2, 4.1, 4.2). A warp takes a tile,
+// one point per lane: its own points first, then the points of the leaves
+// within eps, 32 leaves at a time. Their points pass by in one stream, one per
+// lane; those within eps of the box of the queries still counting are staged,
+// and every 32 of them (or the last) are tested against the queries, looping
+// over the smaller side. The order of the list and of the points in a leaf is
+// kept, so a query's neighbours are found in the order of the lists.
+// Issue-bound (75% of the slots; 1700 instructions per tile on 16.8M halos,
+// a quarter of them the tile's own pairs): visiting leaf by leaf, with a test
+// of each query against each leaf's box, took 1580 us there and 338 us on 400K
+// 5D points, this takes 1460 and 263 us.
+constexpr int FEW_QUERIES = 8;
+
+template <int D>
+struct PreWarp {
+    using T = Traits<D>;
+    using P = typename T::Point;
+    const DevArgs<D>& a;
+    WarpMem<D>& wm;
+    int lane;
+    float e2;
+    int min_pts;
+    int qs;       // the tile's first point
+    P p;
+    bool act;     // this lane's query still counts
+    int cnt;
+    // lane l's query (point qs + l) records its out-of-tile neighbours while
+    // its count is below minPts, so a query that ends non-core has all of
+    // them (nl <= minPts - 1 = lcap; lcap 0: no lists)
+    int nl;
+    typename T::Box qbox;  // box of the queries that count when the walk starts
+
+    // n staged points against the queries still counting
+    __device__ __forceinline__ void flush(int n)
+    {
+        __syncwarp();
+        unsigned am = __ballot_sync(FULL, act);
+        const unsigned am0 = am;
+        const bool list = a.lcap > 0;
+        int32_t* row = a.nlist + (int64_t)(qs + lane) * a.lcap;
+        if (__popc(am) < n) {
+            // lane per staged point, looping over the queries
+            const bool in = lane < n;
+            const P rp = wm.soa.get(lane);
+            const int ri = wm.idx[lane];
+#pragma unroll 1
+            while (am) {
+                const int q = __ffs(am) - 1;
+                am &= am - 1;
+                const P pq = NB<D>::shfl(p, q);
+                const unsigned h = __ballot_sync(FULL, in && dist2(pq, rp) <= e2);
+                if (!h) continue;  // the common case in sparse regions: nothing to record
+                if (list) {
+                    // each hit point writes itself into q's list
+                    const int at = __shfl_sync(FULL, nl, q) + __popc(h & ((1u << lane) - 1u));
+                    if (((h >> lane) & 1u) && at < a.lcap) a.nlist[(int64_t)(qs + q) * a.lcap + at] = ri;
+                }
+                if (lane == q) {
+                    cnt += __popc(h);
+                    nl += __popc(h);
+                    act = cnt < min_pts;
+                }
+            }
+        } else {
+            // lane per query, looping over the staged points two at a time
+            // (packed; of an odd count the last distance is of a slot not in
+            // use); a count that reaches minPts stops
+            const typename NB<D>::PP pp = NB<D>::pack(p);
+#pragma unroll 1
+            for (int u = 0; u < n && act; u += 2) {
+                float d0, d1;
+                wm.soa.d2pair(pp, u, d0, d1);
+                const bool h0 = d0 <= e2, h1 = d1 <= e2 && u + 1 < n;
+                if (h0 || h1) {
+                    if (list) {
+                        int at = nl;
+                        if (h0 && at < a.lcap) row[at] = wm.idx[u];
+                        at += h0;
+                        if (h1 && at < a.lcap) row[at] = wm.idx[u + 1];
+                    }
+                    cnt += h0 + h1;
+                    nl += h0 + h1;
+                    act = cnt < min_pts;
+                }
+            }
+        }
+        __syncwarp();
+        // fewer queries, a smaller box
+        am = __ballot_sync(FULL, act);
+        if (am && am != am0) qbox = warp_box<D>(p, act);
+    }
+
+    // up to 32 candidate leaves, one per lane (U < 0: none); whether any
+    // query still counts
+    __device__ __forceinline__ bool batch(int U, int64_t m)
+    {
+        int us = 0, ue = 0;
+        bool cand = false, whole = false;
+        typename T::Box bx = qbox;
+        if (U >= 0) {
+            const int2 r = __ldg(&a.leafr[U]);
+            us = r.x;
+            ue = r.y & 0x7fffffff;
+            bx = load_box<D>(a.nodebox, (m - 1) + U);
+            cand = NB<D>::bbox(qbox, bx) <= e2;
+            whole = cand && ue - us >= min_pts && T::box_far2(qbox, bx) <= e2;
+        }
+        if (!__any_sync(FULL, cand)) return true;
+        if (__any_sync(FULL, whole)) {
+            // a leaf of at least minPts points lies within eps of all queries
+            if (act) cnt = min_pts;
+            act = false;
+            return false;
+        }
+        // a dense cell larger than a tile: the queries that it lies within
+        // eps of as a whole are done, and it is not streamed unless another
+        // query is within eps of its box
+        unsigned bm = __ballot_sync(FULL, cand && ue - us > TILE);
+        if (bm) {
+            const bool was = act;
+#pragma unroll 1
+            while (bm) {
+                const int src = __ffs(bm) - 1;
+                bm &= bm - 1;
+                const typename T::Box big = load_box<D>(a.nodebox, (m - 1) + __shfl_sync(FULL, U, src));
+                const int size = __shfl_sync(FULL, ue - us, src);
+                if (act && size >= min_pts && T::far_dist2(p, big) <= e2) {
+                    cnt = min_pts;
+                    act = false;
+                }
+                const bool near = __any_sync(FULL, act && NB<D>::pbox(p, big) <= e2);
+                if (lane == src) cand = near;
+            }
+            if (!__any_sync(FULL, act)) return false;
+            if (__any_sync(FULL, act != was)) qbox = warp_box<D>(p, act);
+        }
+        // few queries: their box says little, so each of them is tested against
+        // the lanes' leaves
+        unsigned am = __ballot_sync(FULL, act);
+        if (__popc(am) <= FEW_QUERIES) {
+            bool near = false;
+#pragma unroll 1
+            while (am) {
+                const P pq = NB<D>::shfl(p, __ffs(am) - 1);
+                am &= am - 1;
+                near = near || NB<D>::pbox(pq, bx) <= e2;
+            }
+            cand = cand && near;
+            if (!__any_sync(FULL, cand)) return true;
+        }
+        GBD_COUNT(CNT_LEAF, cand);
+        PointStream<D> ps(a.sp, wm.st, cand, us, ue, lane);
+        int n = 0;
+#pragma unroll 1
+        for (;;) {
+            const bool more = ps.next();
+            const bool keep = more && ps.in && NB<D>::pbox(ps.p, qbox) <= e2;
+            const unsigned km = __ballot_sync(FULL, keep);
+            if (more ? n + __popc(km) > 32 : n > 0) {
+                flush(n);
+                if (!__any_sync(FULL, act)) return false;
+                n = 0;
+            }
+            if (!more) return true;
+            if (keep) {
+                const int at = n + __popc(km & ((1u << lane) - 1u));
+                wm.soa.put(at, ps.p);
+                wm.idx[at] = ps.j;
+            }
+            n += __popc(km);
+        }
+    }
+
+    __device__ __forceinline__ void walk(int L, int64_t m)
+    {
+        const int lc = a.lcount[L];
+        int sp = 0, nc = 0, j0 = 0;
+        int64_t steps = 0;
+        if (lc < 0) sp = walk_roots<D>(a, L, (int)(m - 1), 0, wm.stack, lane);
+#pragma unroll 1
+        for (;;) {
+            int U = -1;
+            if (lc >= 0) {
+                if (j0 >= lc) return;
+                if (j0 + lane < lc) U = __ldg(a.llist + (int64_t)L * LEAFCAP + j0 + lane);
+                j0 += 32;
+            } else {
+                if (walk_next<D>(a, wm, sp, nc, steps, m, qbox, e2, 0, lane) == 0) return;
+                U = walk_take<D>(wm, nc, lane);
+                if (U == L) U = -1;
+            }
+            if (!batch(U, m)) return;
+        }
+    }
+};
+
+template <int D>
+__global__ void __maxnreg__(traversal_regs<D>()) k_pre(const __grid_constant__ DevArgs<D> a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     WarpMem<D>* wm = reinterpret_cast<WarpMem<D>*>(smem) + (threadIdx.x >> 5);
@@ -1234,49 +935,46 @@ __global__ void __maxnreg__(traversal_regs<D>()) k_pre(DevArgs<D> a)
         // points of dense cells inside the tile are core already
         const bool counts = q < e && !a.core[q];
         if (!__any_sync(FULL, counts)) continue;
-        const typename Traits<D>::Point p = a.sp[q < e ? q : s];
+        PreWarp<D> w{a, *wm};
+        w.lane = lane;
+        w.e2 = tp.e2;
+        w.min_pts = tp.min_pts;
+        w.qs = s;
+        w.p = a.sp[q < e ? q : s];
         // the tile's own points first: in dense regions most queries reach
         // minPts here and need no traversal at all (two points at a time)
-        wm->soa.put(lane, p);
+        wm->soa.put(lane, w.p);
         __syncwarp();
-        const typename NB<D>::PP pp = NB<D>::pack(p);
         int cnt = 0;
         if (counts) {
+            const typename NB<D>::PP pp = NB<D>::pack(w.p);
             int u = 0;
             for (; u + 1 < k && cnt < tp.min_pts; u += 2) {
                 float d0, d1;
                 wm->soa.d2pair(pp, u, d0, d1);
                 cnt += (d0 <= tp.e2) + (d1 <= tp.e2);
             }
-            if (u < k && cnt < tp.min_pts && wm->soa.d2(p, u) <= tp.e2) ++cnt;
+            if (u < k && cnt < tp.min_pts && wm->soa.d2(w.p, u) <= tp.e2) ++cnt;
         }
         __syncwarp();
-        PreV<D> v;
-        v.sp = a.sp; v.leafr = a.leafr; v.soa = &wm->soa; v.e2 = tp.e2; v.min_pts = tp.min_pts;
-        v.mask_lo = 0; v.own = L; v.lane = lane;
-        v.act = counts && cnt < tp.min_pts;
-        v.p = p;
-        v.pp = pp;
-        v.cnt = cnt;
-        v.nlist = a.lcap > 0 ? a.nlist : nullptr;
-        v.lcap = a.lcap;
-        v.qs = s;
-        v.nl = 0;
-        const unsigned am = __ballot_sync(FULL, v.act);
+        w.act = counts && cnt < tp.min_pts;
+        w.cnt = cnt;
+        w.nl = 0;
+        const unsigned am = __ballot_sync(FULL, w.act);
         if (am) {
             // every point of the tile still counting: their box is the
             // leaf's own (exact min/max of the same points), no reduction
-            v.qbox = am == tile_lanes(k) ? load_box<D>(a.nodebox, (m - 1) + L) : warp_box<D>(p, v.act);
-            walk(a, m, v, wm->stack, L);
+            w.qbox = am == tile_lanes(k) ? load_box<D>(a.nodebox, (m - 1) + L) : warp_box<D>(w.p, w.act);
+            w.walk(L, m);
         }
         if (counts) {
-            const bool c = v.cnt >= tp.min_pts;
+            const bool c = w.cnt >= tp.min_pts;
             a.core[q] = c ? 1 : 0;
             // lists: how many out-of-tile neighbours the list of a non-core
             // point holds; else whether another point is within eps (the
             // count includes q)
-            a.nbr[q] = a.lcap > 0 ? (c ? 0 : (uint8_t)v.nl) : (v.cnt >= 2 ? 1 : 0);
-            if (a.ncount) a.ncount[q] = v.cnt;
+            a.nbr[q] = a.lcap > 0 ? (c ? 0 : (uint8_t)w.nl) : (w.cnt >= 2 ? 1 : 0);
+            if (a.ncount) a.ncount[q] = w.cnt;
         }
     }
 }
@@ -1304,14 +1002,63 @@ __global__ void k_list_claims(const int32_t* __restrict__ nlist, int lcap, const
 
 // Each tile resolves its own pairs (q, q') with q' > q. Every lane builds the
 // bit mask of the tile points within eps of its point; the components of the
-// core points follow from doubling reach sets (the union of the reach sets
-// of the points already reached) over warp shuffles, at most five rounds for
-// 32 points; each core point then joins its component's first point
+// core points follow by growing each from its first point with one warp
+// reduction per step; each core point then joins its component's first point
 // globally (at most one union per point), and a non-core point with a core
 // neighbour in the tile claims it. Finally the tile records whether it is
 // solid: all points core and in one set. Dense cells larger than a tile are
 // solid by construction.
 constexpr int INTRA_THREADS = 256;
+
+// a leaf's flag: no core point and none to claim (the main phase skips it),
+// solid (all points core and in one set), or neither
+constexpr uint8_t LEAF_IDLE = 0, LEAF_SOLID = 1, LEAF_MIXED = 2;
+
+// Leaf L (nA staged points in soa, of which those in `am` are core; staged
+// point j is point sA + j * step) united with the next leaf in sorted order
+// where a pair of their points (up to 32 of a dense cell) is within eps. In
+// dense regions nearly every leaf is adjacent to the next one, so the main
+// phase starts from sets that span stretches of the curve and drops most of
+// its candidate leaves by their sets.
+template <int D>
+__device__ __forceinline__ void link_next(const DevArgs<D>& a, const SoA<D>& soa, int64_t L, int64_t m,
+                                          const TileParams& tp, int nA, unsigned am, int sA, int step, int lane)
+{
+    using P = typename Traits<D>::Point;
+    if (L + 1 >= m || (a.linst && a.linst[L + 1] != a.linst[L])) return;
+    const int2 r = a.leafr[L + 1];
+    const int n = (r.y & 0x7fffffff) - r.x;
+    const int idx = r.x + (n <= 32 ? min(lane, n - 1) : (int)((int64_t)n * lane / 32));
+    const P p = a.sp[idx];
+    const typename Traits<D>::Box box = load_box<D>(a.nodebox, (m - 1) + L);
+    const bool c = lane < n && (tp.min_pts <= 2 || r.y < 0 || a.core[idx]) && NB<D>::pbox(p, box) <= tp.e2;
+    if (!__any_sync(FULL, c)) return;
+    unsigned hit = 0;
+    if (c) {
+        const typename NB<D>::PP pp = NB<D>::pack(p);
+        for (int j = 0; j < nA; j += 2) {  // (an odd count: the last distance is of a slot that `am` drops)
+            float d0, d1;
+            soa.d2pair(pp, j, d0, d1);
+            hit |= (d0 <= tp.e2 ? 1u : 0u) << j;
+            hit |= (d1 <= tp.e2 ? 2u : 0u) << j;
+        }
+        hit &= am;
+    }
+    const unsigned hm = __ballot_sync(FULL, hit != 0);
+    if (!hm) return;
+    const int q = hit ? sA + (__ffs(hit) - 1) * step : sA;
+    if (hit && tp.min_pts == 2) {
+        a.core[idx] = 1;
+        a.core[q] = 1;
+    }
+    // one lane first: the others mostly find their pair united then
+    const bool lead = lane == __ffs(hm) - 1;
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+        if (hit && lead == (h == 0) && __ldcg(a.labels + idx) != __ldcg(a.labels + q)) uf_union(a.labels, idx, q);
+        __syncwarp();
+    }
+}
 
 template <int D>
 __global__ void __launch_bounds__(INTRA_THREADS) k_intra(DevArgs<D> a)
@@ -1326,7 +1073,12 @@ __global__ void __launch_bounds__(INTRA_THREADS) k_intra(DevArgs<D> a)
     for (int64_t L = wid; L < m; L += nw) {
         const int2 r = a.leafr[L];
         if (r.y < 0) {
-            if (lane == 0) a.lsolid[L] = 1;
+            if (lane == 0) a.lsolid[L] = LEAF_SOLID;
+            const int n = (r.y & 0x7fffffff) - r.x;
+            soa.put(lane, a.sp[r.x + (int)((int64_t)n * lane / 32)]);
+            __syncwarp();
+            link_next<D>(a, soa, L, m, tile_params(a, (int)L), 32, FULL, r.x, 0, lane);
+            __syncwarp();
             continue;
         }
         const int s = r.x, k = r.y - r.x;
@@ -1335,8 +1087,9 @@ __global__ void __launch_bounds__(INTRA_THREADS) k_intra(DevArgs<D> a)
         bool c = valid && a.core[s + lane];
         if (tp.min_pts > 2 && !__any_sync(FULL, c)) {
             // core flags known and none in the tile: no pair inside it
-            // unites or claims anything, and it is not solid
-            if (lane == 0) a.lsolid[L] = 0;
+            // unites or claims anything; the main phase needs the tile only
+            // where it claims border points
+            if (lane == 0) a.lsolid[L] = a.lcap > 0 || a.mode != DBSCAN_MODE_DBSCAN ? LEAF_IDLE : LEAF_MIXED;
             continue;
         }
         const P p = a.sp[valid ? s + lane : s];
@@ -1366,16 +1119,20 @@ __global__ void __launch_bounds__(INTRA_THREADS) k_intra(DevArgs<D> a)
         const unsigned cm = __ballot_sync(FULL, c);
         if (tp.min_pts > 2 && a.mode == DBSCAN_MODE_DBSCAN && valid && !c && (adj & cm))
             uf_claim(a.labels, s + lane, s + __ffs(adj & cm) - 1);
-        unsigned reach = c ? ((adj & cm) | (1u << lane)) : 0u;
-        for (int it = 0; it < 5; ++it) {
-            unsigned acc = reach;
-            for (int j = 0; j < k; ++j) {
-                const unsigned rj = __shfl_sync(FULL, reach, j);
-                if ((reach >> j) & 1u) acc |= rj;
-            }
-            const bool changed = acc != reach;
-            reach = acc;
-            if (!__any_sync(FULL, changed)) break;
+        // the components, each grown from its first point by one reduction
+        // over the lanes already in it per step
+        const unsigned near = c ? adj & cm : 0u;
+        unsigned reach = 1u << lane;
+        unsigned left = __ballot_sync(FULL, near != 0);
+        const bool pairs = left != 0;
+        while (left) {
+            unsigned grown = left & (0u - left), set;
+            do {
+                set = grown;
+                grown |= __reduce_or_sync(FULL, ((set >> lane) & 1u) ? near : 0u);
+            } while (grown != set);
+            if ((set >> lane) & 1u) reach = set;
+            left &= ~set;
         }
         if (c) {
             const int lr = __ffs(reach) - 1;
@@ -1385,20 +1142,27 @@ __global__ void __launch_bounds__(INTRA_THREADS) k_intra(DevArgs<D> a)
         const int root = c ? uf_find(a.labels, s + lane) : -1;
         const int root0 = __shfl_sync(FULL, root, 0);
         const bool solid = __all_sync(FULL, !valid || (c && root == root0));
-        if (lane == 0) a.lsolid[L] = solid ? 1 : 0;
+        if (lane == 0) a.lsolid[L] = solid ? LEAF_SOLID : LEAF_MIXED;
+        if (pairs) link_next<D>(a, soa, L, m, tp, k, tp.min_pts <= 2 ? tile_lanes(k) : cm, s, 1, lane);
         __syncwarp();
     }
 }
 
 // Leaf kinds for the main phase: 0 a tile that is not solid, 1 a solid tile,
-// 2 a dense cell larger than a tile. Lists are grouped by kind; within a warp
-// (32 consecutive leaves) the order is kept.
+// 2 a dense cell larger than a tile, -1 a tile with nothing to do. Lists are
+// grouped by kind; within a warp (32 consecutive leaves) the order is kept.
 __device__ __forceinline__ int leaf_kind(const int2* leafr, const uint8_t* lsolid, int64_t L)
 {
-    return leafr[L].y < 0 ? 2 : (lsolid[L] ? 1 : 0);
+    if (leafr[L].y < 0) return 2;
+    const uint8_t f = lsolid[L];
+    return f == LEAF_IDLE ? -1 : (f == LEAF_SOLID ? 1 : 0);
 }
 
-__global__ void k_kinds_count(const int2* __restrict__ leafr, const uint8_t* __restrict__ lsolid, uint32_t* ctrl)
+// (the links between consecutive leaves leave chains of sets as long as a
+// stretch of the curve; every leaf's thread shortens its own here, all of
+// them at once, so that the chains shrink by doubling)
+__global__ void k_kinds_count(const int2* __restrict__ leafr, const uint8_t* __restrict__ lsolid, uint32_t* ctrl,
+                              int32_t* labels)
 {
     const int lane = threadIdx.x & 31;
     const int64_t m = ctrl[CTRL_M];
@@ -1411,6 +1175,7 @@ __global__ void k_kinds_count(const int2* __restrict__ leafr, const uint8_t* __r
             const unsigned b = __ballot_sync(FULL, kind == t);
             if (lane == 0 && b) atomicAdd(&ctrl[CTRL_KIND_COUNT + t], (uint32_t)__popc(b));
         }
+        if (kind > 0) uf_find(labels, leafr[L].x);
     }
 }
 
@@ -1437,95 +1202,571 @@ __global__ void k_kinds_write(const int2* __restrict__ leafr, const uint8_t* __r
     }
 }
 
-// The main phase (KIND 0: tiles that are not solid, MainPtV; 1: solid
-// tiles, MainSolidV; 2: dense cells larger than a tile, MainBoxV; 3: all of
-// them in one launch), taken from the kinds' lists through a work counter.
-// In one launch the dense cells come first -- few, each much work -- and the
-// warps that finish them go on to the tiles instead of leaving the GPU idle
-// until the slowest cell is done.
-template <int D, int KIND>
-__global__ void __maxnreg__(traversal_regs<D>()) k_main(DevArgs<D> a)
+// ---------------------------------------------------------------------------
+// The main phase.
+//
+// A warp takes one leaf L (a tile of up to 32 points, one per lane, or a
+// dense cell larger than a tile) and unites it with the leaves after it (the
+// pair mask of Sec. 4.1). What bounds it is the latency of dependent loads
+// (leaf record, points, union-find chains), not arithmetic, so the candidate
+// leaves are taken 32 at a time, one per lane: each lane loads its leaf's
+// record, box and flag and follows the chain of its first point, and only
+// the leaves that can still change something are visited one after another
+// by the whole warp. Three things decide that nothing can change: the boxes
+// are farther apart than eps; the leaf holds no core point (and no border
+// point can be claimed); or it is solid and already in the set that all of
+// L's points are in. A visited tile is cut to its points near L's box whose
+// set differs from L's before any distance is taken: sets never split, so a
+// pair that shared a root at any time needs no test. Testing the pairs first
+// and looking at the sets of those within eps, one leaf after another, took
+// 1241 us on 16.8M halos, 1524 us on 8M halos at minPts 2 and 1243 us on 400K
+// 5D points; this takes 514, 943 and 515 us (kernel times).
+// ---------------------------------------------------------------------------
+
+// What a point can still do, by its code: the root of its set (core points;
+// for minPts <= 2 all points), CODE_FREE for a non-core point that no core
+// point has claimed, CODE_DONE for all others.
+constexpr int CODE_FREE = -1, CODE_DONE = -2;
+
+// can a pair within eps change something: a core point with a point of
+// another set, or with an unclaimed non-core one
+__device__ __forceinline__ bool pairable(int x, int y) { return x != y && min(x, y) >= CODE_FREE; }
+
+// The union-find steps of the main phase are calls, not inlined: with its
+// visitors and their union-find loops inlined at every use the kernel was
+// 279 KB of code, and a fifth to a third of its warps' stalls were waits for
+// instructions.
+__device__ __noinline__ int uf_find_call(int* L, int x) { return uf_find(L, x); }
+
+// unites the sets of x and y; returns the root of the union
+__device__ __noinline__ int uf_join(int* L, int x, int y)
+{
+#pragma unroll 1
+    for (;;) {
+        uf_find2(L, x, y);
+        if (x == y) return x;
+        if (x > y) { const int t = x; x = y; y = t; }
+        if (atomicCAS(L + y, y, x) == y) return x;
+    }
+}
+
+template <int D>
+struct MainWarp {
+    using T = Traits<D>;
+    using P = typename T::Point;
+    using B = typename T::Box;
+    const DevArgs<D>& a;
+    WarpMem<D>& wm;
+    int64_t m;
+    int lane;
+    float e2;
+    int min_pts;
+    bool claims;  // core-to-non-core claims: DBSCAN mode without preprocessing lists
+    bool cell;    // a dense cell larger than a tile (else a tile)
+    int L;
+    int s, e;     // its points
+    P p;          // tile: this lane's point and its code
+    int rq;
+    bool uni;     // all of L's points that take part are in set R
+    int R;
+    B qbox;       // box of the points that take part
+
+    __device__ __forceinline__ int find(int x) const { return uf_find_call(a.labels, x); }
+    // the set of x where L is in one set: a parent that is R settles it, so
+    // that the many points of a large set do not all read its root's word
+    __device__ __forceinline__ int find_near(int x) const
+    {
+        return uni && __ldcg(a.labels + x) == R ? R : find(x);
+    }
+    // the root of x, the same in all lanes (they decide together on it)
+    __device__ __forceinline__ int warp_root(int x) const { return __shfl_sync(FULL, find(x), 0); }
+
+    // the code of point i (core flag c)
+    __device__ __forceinline__ int code_of(int i, bool c) const
+    {
+        if (min_pts <= 2 || c) return find_near(i);
+        return claims && __ldcg(a.labels + i) == i ? CODE_FREE : CODE_DONE;
+    }
+    // are all points that take part in one set (tiles)
+    __device__ __forceinline__ void uniform()
+    {
+        const unsigned part = __ballot_sync(FULL, rq >= CODE_FREE);
+        R = part ? __shfl_sync(FULL, rq, __ffs(part) - 1) : CODE_DONE;
+        uni = __all_sync(FULL, rq == CODE_DONE || rq == R) && R >= 0;
+    }
+    // codes after unions and claims
+    __device__ __forceinline__ void refresh()
+    {
+        if (rq >= 0) rq = find(rq);
+        else if (rq == CODE_FREE && __ldcg(a.labels + s + lane) != s + lane) rq = CODE_DONE;
+        uniform();
+    }
+    // the sets x and y united (codes are mostly roots still: then one
+    // compare-and-swap does it); returns a node of the union near its root
+    __device__ __forceinline__ int join(int x, int y) const
+    {
+        const int hi = max(x, y), lo = min(x, y);
+        return atomicCAS(a.labels + hi, hi, lo) == hi ? lo : uf_join(a.labels, hi, lo);
+    }
+    // the rule of Algorithm 3 for a pair (i, j) within eps with codes ci, cj
+    // (pairable); the union's node, or INT_MAX after a claim
+    __device__ __forceinline__ int act(int i, int ci, int j, int cj) const
+    {
+        if (min(ci, cj) >= 0) return join(ci, cj);
+        // a non-core point joins the core point's set, unless another claimed it first
+        const int y = ci >= 0 ? j : i;
+        atomicCAS(a.labels + y, y, max(ci, cj));
+        return INT_MAX;
+    }
+
+    // L's set (uni) united with the sets ru of the lanes with `on`: all of
+    // them are hooked under the smallest root at once, so no lane waits for
+    // another's union. R becomes the set's root.
+    __device__ __forceinline__ void unite_lanes(bool on, int ru)
+    {
+        const int lo = min(R, __reduce_min_sync(FULL, on ? ru : R));
+        int r = lo;
+        const unsigned peers = __match_any_sync(FULL, on ? ru : -1);
+        if (on && ru != lo && lane == __ffs(peers) - 1) r = join(ru, lo);
+        if (lane == 0 && R != lo) r = min(r, join(R, lo));
+        R = __reduce_min_sync(FULL, r);
+        if (rq >= 0) {
+            rq = R;
+            // (several points in one set are core already, a tile's only point is by this pair)
+            if (min_pts == 2) a.core[s + lane] = 1;
+        }
+    }
+
+    // One round of a tile against n staged points (within eps of the query
+    // box, allowed to take part): their sets, the pairs that can still change
+    // something, their distances, the unions. The smaller side is looped over
+    // (the pivot), the other sits in the lanes; after a union the codes on
+    // both sides are brought up to date by value, without reading them again.
+    __device__ __forceinline__ void flush(int n)
+    {
+        __syncwarp();
+        // lane u: staged point u
+        int cu = CODE_DONE, ui = 0;
+        P up = p;
+        if (lane < n) {
+            const int enc = wm.idx[lane];
+            ui = enc & 0x7fffffff;
+            cu = code_of(ui, enc >= 0);
+            up = wm.soa.get(lane);
+        }
+        __syncwarp();
+        if (uni && cu == R) cu = CODE_DONE;
+        const unsigned km = __ballot_sync(FULL, cu >= CODE_FREE);
+        if (!km) return;
+        const unsigned mq = __ballot_sync(FULL, rq >= CODE_FREE);
+        const bool byq = __popc(mq) <= __popc(km);  // the queries are the pivots
+        const P x = byq ? up : p, y = byq ? p : up;
+        const int ix = byq ? ui : s + lane, iy = byq ? s + lane : ui;
+        int cx = byq ? cu : rq, cy = byq ? rq : cu;
+        unsigned mask = byq ? mq : km;
+#pragma unroll 1
+        while (mask) {
+            const int v = __ffs(mask) - 1;
+            mask &= mask - 1;
+            const P py = NB<D>::shfl(y, v);
+            const int pc = __shfl_sync(FULL, cy, v);
+            const bool hit = pairable(pc, cx) && dist2(py, x) <= e2;
+            if (!__any_sync(FULL, hit)) continue;
+            const int pi = __shfl_sync(FULL, iy, v);
+            // one union per set that was hit
+            bool lead = hit && min(pc, cx) < 0;
+            for (unsigned mm = __ballot_sync(FULL, hit && !lead); mm;) {
+                const int src = __ffs(mm) - 1;
+                lead = lead || lane == src;
+                mm &= ~__ballot_sync(FULL, cx == __shfl_sync(FULL, cx, src));
+            }
+            if (hit && min_pts == 2) { a.core[pi] = 1; a.core[ix] = 1; }
+            int r = INT_MAX;
+            if (lead) r = act(pi, pc, ix, cx);
+            __syncwarp();
+            if (pc == CODE_FREE) {  // claimed
+                if (lane == v) cy = CODE_DONE;
+                continue;
+            }
+            r = __reduce_min_sync(FULL, r);
+            const int old = cx;
+            if (hit && cx == CODE_FREE) cx = CODE_DONE;
+            unsigned mm = __ballot_sync(FULL, hit && old >= 0);
+            if (!mm) continue;
+            if (cy == pc) cy = r;
+            while (mm) {
+                const int c = __shfl_sync(FULL, old, __ffs(mm) - 1);
+                if (cx == c) cx = r;
+                mm &= ~__ballot_sync(FULL, old == c);
+            }
+            // all that is left in one set
+            if (!__any_sync(FULL, (cx >= CODE_FREE && cx != r) || (((mask >> lane) & 1u) && cy != r))) break;
+        }
+        rq = byq ? cy : cx;
+        uniform();
+    }
+
+    // A tile that is not in one set against a dense cell larger than a tile:
+    // each query of another set looks for one adjacent point.
+    __device__ __forceinline__ void tile_big(int us, int ue, const B& box)
+    {
+        const int ru = warp_root(us);
+        if (rq >= 0 && rq != ru) rq = find(rq);
+        const bool need = pairable(rq, ru) && NB<D>::pbox(p, box) <= e2;
+        if (!__any_sync(FULL, need)) return;
+        unsigned hm = __ballot_sync(FULL, need && T::far_dist2(p, box) <= e2);
+        unsigned open = __ballot_sync(FULL, need) & ~hm;
+#pragma unroll 1
+        for (int c = us; c < ue && open; c += 32) {
+            // the cell's points within eps of the queries' box (exact pruning)
+            const P rp = a.sp[min(c + lane, ue - 1)];
+            const bool keep = c + lane < ue && NB<D>::pbox(rp, qbox) <= e2;
+            if (!__any_sync(FULL, keep)) continue;
+            unsigned mm = open;
+#pragma unroll 1
+            while (mm) {
+                const int qq = __ffs(mm) - 1;
+                mm &= mm - 1;
+                const P pq = NB<D>::shfl(p, qq);
+                if (__any_sync(FULL, keep && dist2(pq, rp) <= e2)) hm |= 1u << qq;
+            }
+            open &= ~hm;
+        }
+        if (!hm) return;
+        if ((hm >> lane) & 1u) {
+            if (min_pts == 2) { a.core[s + lane] = 1; a.core[us] = 1; }
+            act(s + lane, rq, us, ru);
+        }
+        __syncwarp();
+        refresh();
+    }
+
+    // L in one set (a tile or a dense cell) against a solid leaf: is there an
+    // adjacent pair? Of L only the points within eps of the leaf's box can
+    // have a partner, of the leaf only those within eps of L's box (exact
+    // pruning). Up to 32 of L's are staged at a time; the leaf's points pass
+    // by them, one per lane, four loads in flight.
+    // [ls, le): the part of L looked at.
+    __device__ __forceinline__ bool adjacent(int ls, int le, int us, int ue, const B& box)
+    {
+        const unsigned lt = (1u << lane) - 1u;
+        int cq = ls;
+#pragma unroll 1
+        while (cq < le) {
+            int n = 0;
+            if (cell) {
+#pragma unroll 1
+                for (; cq < le; cq += 32) {
+                    const P pq = a.sp[min(cq + lane, le - 1)];
+                    const bool near = cq + lane < le && NB<D>::pbox(pq, box) <= e2;
+                    const unsigned nm = __ballot_sync(FULL, near);
+                    if (n + __popc(nm) > 32) break;
+                    if (near) wm.soa.put(n + __popc(nm & lt), pq);
+                    n += __popc(nm);
+                }
+            } else {
+                const bool near = rq >= 0 && NB<D>::pbox(p, box) <= e2;
+                const unsigned nm = __ballot_sync(FULL, near);
+                if (near) wm.soa.put(__popc(nm & lt), p);
+                n = __popc(nm);
+                cq = le;
+            }
+            if (!n) continue;
+            __syncwarp();
+            // (the next points are loaded while the current ones are tested)
+            P r = a.sp[min(us + lane, ue - 1)];
+#pragma unroll 1
+            for (int c = us; c < ue; c += 32) {
+                const P rn = a.sp[min(c + 32 + lane, ue - 1)];
+                bool hit = false;
+                if (NB<D>::pbox(r, qbox) <= e2) {
+                    const typename NB<D>::PP pr = NB<D>::pack(r);
+#pragma unroll 1
+                    for (int u = 0; u < n && !hit; u += 2) {
+                        float d0, d1;
+                        wm.soa.d2pair(pr, u, d0, d1);
+                        hit = d0 <= e2 || (d1 <= e2 && u + 1 < n);
+                    }
+                }
+                if (__any_sync(FULL, hit)) return true;
+                r = rn;
+            }
+            __syncwarp();
+        }
+        return false;
+    }
+
+    // ---- dense cell against a tile that is not solid: lane per tile point
+    __device__ __forceinline__ void cell_mixed(int us, int ue, const B& box)
+    {
+        const int k = ue - us;
+        const bool in = lane < k;
+        const int ri = us + (in ? lane : 0);
+        const P rp = a.sp[ri];
+        const bool rc = a.core[ri];
+        int cu = CODE_DONE;
+        if (in && NB<D>::pbox(rp, qbox) <= e2) cu = code_of(ri, rc);
+        bool need = pairable(R, cu);
+        if (!__any_sync(FULL, need)) return;
+        bool found = need && T::far_dist2(rp, qbox) <= e2;
+        const unsigned lt = (1u << lane) - 1u;
+#pragma unroll 1
+        for (int cq = s; cq < e; cq += 32) {
+            if (!__any_sync(FULL, need && !found)) break;
+            const P ap = a.sp[min(cq + lane, e - 1)];
+            const bool keep = cq + lane < e && NB<D>::pbox(ap, box) <= e2;
+            const unsigned km = __ballot_sync(FULL, keep);
+            if (!km) continue;
+            if (keep) wm.soa.put(__popc(km & lt), ap);
+            __syncwarp();
+            const int kk = __popc(km);
+            if (need)
+#pragma unroll 1
+                for (int u = 0; u < kk && !found; ++u) found = wm.soa.d2(rp, u) <= e2;
+            __syncwarp();
+        }
+        if (need && found) {
+            if (min_pts == 2) a.core[ri] = 1;
+            act(s, R, ri, cu);
+        }
+        __syncwarp();
+        R = warp_root(R);
+    }
+
+    // what the head of a batch needs to know of a lane's candidate leaf
+    struct Head {
+        int U, us, ue, fl;  // leaf (-1: none), its points, its flag
+        B box;
+    };
+    __device__ __forceinline__ Head head(int U) const
+    {
+        Head h;
+        h.U = U;
+        h.us = h.ue = 0;
+        h.fl = LEAF_IDLE;
+        h.box = qbox;
+        if (U >= 0) {
+            h.fl = *(volatile const uint8_t*)&a.lsolid[U];
+            const int2 r = __ldg(&a.leafr[U]);
+            h.box = load_box<D>(a.nodebox, (m - 1) + U);
+            h.us = r.x;
+            h.ue = r.y & 0x7fffffff;
+        }
+        return h;
+    }
+
+    // up to 32 candidate leaves, one per lane
+    __device__ __forceinline__ void batch(const Head& h)
+    {
+        const int us = h.us, ue = h.ue;
+        const bool solid = h.fl == LEAF_SOLID;
+        const float near = NB<D>::bbox(qbox, h.box);
+        bool cand = h.U >= 0 && h.fl != LEAF_IDLE && near <= e2;
+        int ru = 0;
+        if (uni) {
+            if (cand && solid) cand = (ru = find_near(us)) != R;
+            bool far = false;
+            if (__any_sync(FULL, cand && solid)) {
+                R = warp_root(R);
+                if (rq >= 0) rq = R;
+                if (cand && solid) cand = ru != R;
+                far = cand && solid && T::box_far2(qbox, h.box) <= e2;
+            }
+            if (__any_sync(FULL, far)) {
+                // leaves that lie within eps of all of L
+                unite_lanes(far, ru);
+                if (cand && solid) cand = !far && (ru = find_near(ru)) != R;
+            }
+        }
+        if (!cell) {
+            // tiles: their points in one stream, in any order. Of several
+            // solid ones the nearest goes first: the others are often in L's
+            // set once it is
+            const bool small = cand && ue - us <= 32;
+            const unsigned sm = __ballot_sync(FULL, small && solid);
+            bool first = small;
+            if (uni && __popc(sm) > 2) {
+                const unsigned d = small && solid ? __float_as_uint(near) : 0xffffffffu;
+                const unsigned best = __ballot_sync(FULL, d == __reduce_min_sync(FULL, d));
+                first = lane == __ffs(best) - 1;
+            }
+            bool todo = small;
+#pragma unroll 1
+            while (__any_sync(FULL, todo)) {
+                const bool firsts = __any_sync(FULL, todo && first);
+                const bool on = todo && (first || !firsts);
+                PointStream<D> ps(a.sp, wm.st, on, us, ue, lane);
+                int n = 0;
+#pragma unroll 1
+                for (;;) {
+                    const bool more = ps.next();
+                    bool keep = more && ps.in && NB<D>::pbox(ps.p, qbox) <= e2;
+                    const bool c = min_pts > 2 && keep && a.core[ps.j];
+                    keep = keep && (c || min_pts <= 2 || claims);
+                    const unsigned km = __ballot_sync(FULL, keep);
+                    if (more ? n + __popc(km) > 32 : n > 0) {
+                        flush(n);
+                        n = 0;
+                    }
+                    if (!more) break;
+                    if (keep) {
+                        const int at = n + __popc(km & ((1u << lane) - 1u));
+                        wm.soa.put(at, ps.p);
+                        wm.idx[at] = c || min_pts <= 2 ? ps.j : (int)(ps.j | 0x80000000u);
+                    }
+                    n += __popc(km);
+                }
+                todo = todo && !on;
+                if (todo && solid && uni) todo = (ru = find_near(ru)) != R;
+            }
+            cand = cand && !small;
+            if (uni && cand) cand = find_near(us) != R;
+        }
+        // one leaf at a time, the nearer ones first (they are likely adjacent,
+        // and then often join L with the farther ones)
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) {
+            unsigned cm = __ballot_sync(FULL, cand && (near <= 0.25f * e2) == (pass == 0));
+#pragma unroll 1
+            while (cm) {
+                const int src = __ffs(cm) - 1;
+                cm &= cm - 1;
+                const int Us = __shfl_sync(FULL, h.U, src);
+                const int vs = __shfl_sync(FULL, us, src), ve = __shfl_sync(FULL, ue, src);
+                const bool sol = __shfl_sync(FULL, (int)solid, src);
+                const B box = load_box<D>(a.nodebox, (m - 1) + Us);
+                GBD_COUNT(CNT_LEAF, lane == 0);
+                if (!sol) {
+                    cell_mixed(vs, ve, box);
+                } else if (!uni) {
+                    tile_big(vs, ve, box);
+                } else {
+                    // (the points of a dense cell are in input order, so its
+                    // first ones are a sample of it: they settle most pairs)
+                    bool adj = false;
+#pragma unroll 1
+                    for (int part = 0; part < 2 && !adj; ++part) {
+                        const int le = part ? e : min(s + 64, e), v1 = part ? ve : min(vs + 64, ve);
+                        if (part && le == min(s + 64, e) && v1 == min(vs + 64, ve)) break;
+                        adj = adjacent(s, le, vs, v1, box);
+                    }
+                    if (adj) {
+                        const int rv = warp_root(vs);
+                        unite_lanes(lane == src, rv);
+                        // the others may be in L's set now
+                        if (cand && solid) cand = find_near(us) != R;
+                        cm &= __ballot_sync(FULL, cand);
+                    }
+                }
+                __syncwarp();
+            }
+        }
+    }
+
+    // the leaves after L within eps of the query box, from L's list or by
+    // walking the tree
+    __device__ __forceinline__ void walk(int lc, const Head& h0)
+    {
+        int j0 = 0, sp = 0, nc = 0;
+        int64_t steps = 0;
+        Head h = h0;
+        bool have = lc >= 0;  // the first batch of a list comes loaded
+        if (lc < 0) sp = walk_roots<D>(a, L, (int)(m - 1), L + 1, wm.stack, lane);
+#pragma unroll 1
+        for (;;) {
+            int U = -1;
+            if (lc >= 0) {
+                if (j0 >= lc) return;
+                if (!have && j0 + lane < lc) U = __ldg(a.llist + (int64_t)L * LEAFCAP + j0 + lane);
+                j0 += 32;
+            } else {
+                if (walk_next<D>(a, wm, sp, nc, steps, m, qbox, e2, L + 1, lane) == 0) return;
+                U = walk_take<D>(wm, nc, lane);
+            }
+            if (!have) h = head(U > L ? U : -1);
+            have = false;
+            if (__any_sync(FULL, h.U >= 0)) batch(h);
+        }
+    }
+};
+
+template <int D>
+__global__ void __maxnreg__(main_regs<D>()) k_main(const __grid_constant__ DevArgs<D> a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     WarpMem<D>* wm = reinterpret_cast<WarpMem<D>*>(smem) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     const int64_t m = a.ctrl[CTRL_M];
     const int64_t c0 = a.ctrl[CTRL_KIND_COUNT], c1 = a.ctrl[CTRL_KIND_COUNT + 1], c2 = a.ctrl[CTRL_KIND_COUNT + 2];
-    // dense cells larger than a tile are few and each is much work: when
-    // there are more warps than cells, up to 8 warps share a cell (split by
-    // neighbour leaf), so that no warp is left with a whole large cell
-    int parts = 1;
-    if ((KIND == 2 || KIND == 3) && c2 > 0) {
-        const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-        parts = (int)max((int64_t)1, min((int64_t)8, warps / c2));
-    }
-    const int64_t n2 = (KIND == 2 || KIND == 3) ? c2 * parts : 0;
-    const int64_t total = KIND == 3 ? n2 + c1 + c0 : (KIND == 2 ? n2 : (KIND == 1 ? c1 : c0));
-    for (;;) {
-        const int idx = next_leaf(&a.ctrl[CTRL_KIND_WORK + (KIND == 3 ? 0 : KIND)]);
-        if (idx >= total) break;
-        // the list holds kind 0, then 1, then 2
-        int kind, L, part = 0;
-        if (KIND == 3) {
-            if (idx < n2) {
-                kind = 2;
-                L = a.klist[c0 + c1 + idx / parts];
-                part = idx % parts;
-            } else if (idx < n2 + c1) {
-                kind = 1;
-                L = a.klist[c0 + (idx - n2)];
-            } else {
-                kind = 0;
-                L = a.klist[idx - n2 - c1];
-            }
-        } else {
-            kind = KIND;
-            L = a.klist[(KIND == 0 ? 0 : (KIND == 1 ? c0 : c0 + c1)) + (KIND == 2 ? idx / parts : idx)];
-            part = KIND == 2 ? idx % parts : 0;
-        }
+    // One warp per leaf, also when there are more warps than leaves: warps
+    // sharing a leaf contend for the same sets (with up to eight per leaf the
+    // phase took 97 us on 16K dense points, with one 59). The dense cells
+    // larger than a tile come first -- few, each much work.
+    const int64_t total = c0 + c1 + c2;
+    // The chain of dependent loads at the start of a leaf is what a warp
+    // would wait for most: the next leaf's index is taken while the current
+    // one is worked on, and the first batch's lists and leaves are loaded
+    // together with the leaf's own points.
+    int L;
+    auto resolve = [&](int64_t idx) {
+        // the list holds kind 0, then 1, then 2; taken as 2, 1, 0
+        if (idx >= total) L = -1;
+        else if (idx < c2) L = __ldg(&a.klist[c0 + c1 + idx]);
+        else L = __ldg(&a.klist[idx < c2 + c1 ? c0 + (idx - c2) : idx - c2 - c1]);
+    };
+    int pend = 0;
+    if (lane == 0) pend = (int)atomicAdd(&a.ctrl[CTRL_KIND_WORK], 1u);
+    resolve(__shfl_sync(FULL, pend, 0));
+    while (L >= 0) {
+        if (lane == 0) pend = (int)atomicAdd(&a.ctrl[CTRL_KIND_WORK], 1u);
         const TileParams tp = tile_params(a, L);
         const bool listed = a.lcap > 0 && tp.min_pts > 2;
-        const Rule rule{a.labels, a.core, tp.min_pts, a.mode == DBSCAN_MODE_DBSCAN && !listed};
         const int2 r = a.leafr[L];
-        const int s = r.x, e = r.y & 0x7fffffff;
-        if (kind == 0) {
-            MainPtV<D> v;
-            v.sp = a.sp; v.leafr = a.leafr; v.lsolid = a.lsolid; v.core = a.core; v.soa = &wm->soa;
-            v.cbuf = wm->cbuf; v.rule = rule; v.e2 = tp.e2; v.mask_lo = L + 1; v.lane = lane; v.sQ = s;
-            v.q = s + lane;
-            const bool in = v.q < e;
-            v.qcore = in && a.core[v.q];
-            // after preprocessing a non-core point with no other point within
-            // eps takes part in no pair, and in DBSCAN* no non-core point does
-            // (with lists, non-core points took their pairs with core points
-            // from their lists and need no traversal)
-            v.valid = in && (tp.min_pts <= 2 || v.qcore || (rule.claims && a.nbr[v.q]));
-            v.p = a.sp[in ? v.q : s];
-            v.pp = NB<D>::pack(v.p);
-            const unsigned vm = __ballot_sync(FULL, v.valid);
-            if (vm) {
-                v.qbox = vm == tile_lanes(e - s) ? load_box<D>(a.nodebox, (m - 1) + L) : warp_box<D>(v.p, v.valid);
-                walk(a, m, v, wm->stack, L);
-            }
-        } else if (kind == 1) {
-            MainSolidV<D> v;
-            v.sp = a.sp; v.leafr = a.leafr; v.lsolid = a.lsolid; v.core = a.core; v.buf = wm->buf;
-            v.rule = rule; v.e2 = tp.e2; v.mask_lo = L + 1; v.lane = lane; v.sQ = s;
-            v.valid = s + lane < e;
-            v.p = a.sp[v.valid ? s + lane : s];
-            v.pp = NB<D>::pack(v.p);
-            v.qb.lo = a.nodebox[(m - 1) + L].lo;
-            v.qb.hi = a.nodebox[(m - 1) + L].hi;
-            walk(a, m, v, wm->stack, L);
+        const int lc = a.lcount[L];
+        MainWarp<D> w{a, *wm};
+        w.m = m;
+        w.lane = lane;
+        w.e2 = tp.e2;
+        w.min_pts = tp.min_pts;
+        w.claims = a.mode == DBSCAN_MODE_DBSCAN && !listed && tp.min_pts > 2;
+        w.L = L;
+        w.s = r.x;
+        w.e = r.y & 0x7fffffff;
+        w.cell = r.y < 0;
+        int U = -1;
+        if (lane < lc) U = __ldg(a.llist + (int64_t)L * LEAFCAP + lane);
+        if (U <= L) U = -1;
+        // a tile's points that take part: after preprocessing a non-core
+        // point with no other point within eps takes part in no pair, and in
+        // DBSCAN* no non-core point does (with lists, non-core points took
+        // their pairs with core points from their lists)
+        const int q = w.s + lane;
+        const bool in = !w.cell && q < w.e;
+        const bool c = in && a.core[q];
+        w.p = a.sp[in ? q : w.s];
+        w.qbox = load_box<D>(a.nodebox, (m - 1) + L);
+        const typename MainWarp<D>::Head h = w.head(U);
+        w.rq = CODE_DONE;
+        w.uni = false;
+        if (in && (tp.min_pts <= 2 || c || (w.claims && a.nbr[q]))) w.rq = w.code_of(q, c);
+        bool work = true;
+        if (w.cell) {
+            w.uni = true;
+            w.R = w.warp_root(w.s);
         } else {
-            MainBoxV<D> v;
-            v.sp = a.sp; v.leafr = a.leafr; v.lsolid = a.lsolid; v.core = a.core; v.buf = wm->buf;
-            v.rule = rule; v.e2 = tp.e2; v.mask_lo = L + 1; v.lane = lane; v.sQ = s; v.eQ = e;
-            v.part = part; v.parts = parts;
-            v.qb.lo = a.nodebox[(m - 1) + L].lo;
-            v.qb.hi = a.nodebox[(m - 1) + L].hi;
-            walk(a, m, v, wm->stack, L);
+            w.uniform();
+            const unsigned vm = __ballot_sync(FULL, w.rq >= CODE_FREE);
+            work = vm != 0;
+            if (vm == tile_lanes(w.e - w.s)) {
+                // every point core and in one set by now: solid from here on
+                // (others may read the old flag, which only costs them tests)
+                if (w.uni && w.e - w.s > 1 && lane == 0) *(volatile uint8_t*)&a.lsolid[L] = LEAF_SOLID;
+            } else {
+                w.qbox = warp_box<D>(w.p, w.rq >= CODE_FREE);
+            }
         }
+        resolve(__shfl_sync(FULL, pend, 0));
+        if (work) w.walk(lc, h);
     }
 }
 
@@ -1634,6 +1875,8 @@ void count_phase(int phase, cudaStream_t s)
 int persistent_blocks(const void* kernel, int block, size_t smem)
 {
     int dev = 0, sms = 0, per = 0;
+    // (large blocks: more shared memory than a launch gets by default)
+    if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, block, smem);
@@ -1682,14 +1925,14 @@ void run_pre(const ClusterArgs& a, cudaStream_t s)
     k_pre<D><<<g, a.block, smem, s>>>(dev_args<D>(a));
 }
 
-template <int D, int KIND>
-void run_main_kind(const ClusterArgs& a, cudaStream_t s)
+template <int D>
+void run_main_walk(const ClusterArgs& a, cudaStream_t s)
 {
     static int blocks[33] = {};
     const size_t smem = sizeof(WarpMem<D>) * (size_t)(a.block / 32);
     int& g = blocks[a.block / 32];
-    if (!g) g = persistent_blocks((const void*)k_main<D, KIND>, a.block, smem);
-    k_main<D, KIND><<<g, a.block, smem, s>>>(dev_args<D>(a));
+    if (!g) g = persistent_blocks((const void*)k_main<D>, a.block, smem);
+    k_main<D><<<g, a.block, smem, s>>>(dev_args<D>(a));
 }
 
 template <int D>
@@ -1700,9 +1943,9 @@ void run_main(const ClusterArgs& a, cudaStream_t s)
     k_intra<D><<<(unsigned)gw, INTRA_THREADS, 0, s>>>(dev_args<D>(a));
     int64_t gk = (a.m_cap + 255) / 256;
     if (gk > 152 * 8) gk = 152 * 8;
-    k_kinds_count<<<(unsigned)gk, 256, 0, s>>>(a.leafr, a.lsolid, a.ctrl);
+    k_kinds_count<<<(unsigned)gk, 256, 0, s>>>(a.leafr, a.lsolid, a.ctrl, a.labels);
     k_kinds_write<<<(unsigned)gk, 256, 0, s>>>(a.leafr, a.lsolid, a.ctrl, a.klist);
-    run_main_kind<D, 3>(a, s);
+    run_main_walk<D>(a, s);
 }
 
 }  // namespace
@@ -1744,15 +1987,9 @@ cudaError_t launch_cluster_starts(const ClusterArgs& a, cudaStream_t s)
     count_phase(0, s);
     int64_t gm = (a.m_cap + 255) / 256;
     if (gm > 152 * 8) gm = 152 * 8;
-#define TS_LAUNCH(D) k_tile_start<D><<<(unsigned)gm, 256, 0, s>>>(dev_args<D>(a), a.parent, a.nmeta)
-    GBD_DIM_SWITCH(a.dim, TS_LAUNCH)
-#undef TS_LAUNCH
-    if (a.llist) {
-#define LL_LAUNCH(D) k_leaf_lists<D><<<(unsigned)gm, LL_THREADS, 0, s>>>(dev_args<D>(a))
-        GBD_DIM_SWITCH(a.dim, LL_LAUNCH)
+#define LL_LAUNCH(D) k_leaf_lists<D><<<(unsigned)gm, LL_THREADS, 0, s>>>(dev_args<D>(a), a.parent, a.nmeta)
+    GBD_DIM_SWITCH(a.dim, LL_LAUNCH)
 #undef LL_LAUNCH
-        note_launches(1);
-    }
     note_launches(1);
     return cudaGetLastError();
 }
