@@ -126,55 +126,6 @@ __global__ void k_bgather(const int64_t* __restrict__ offs,
     }
 }
 
-// dense cells of every instance (see k_dense_classify): runs of equal keys,
-// with the instance's minPts and eps^2
-__global__ void k_bdense_classify(const uint64_t* __restrict__ keys, const float4* __restrict__ sp, int64_t n,
-                                  int lb, const InstDev* __restrict__ inst, uint8_t* __restrict__ pdense,
-                                  int32_t* __restrict__ dstart, uint32_t* __restrict__ ctrl)
-{
-    using T = Traits<3>;
-    if (!stage_on(ctrl, -1)) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) - lane; base < n; base += stride) {
-        const int64_t i = base + lane;
-        bool cand = false;
-        if (i < n) {
-            const uint64_t k = keys[i];
-            const int mp = inst[k >> lb].min_pts;
-            const int64_t j = i + mp - 1;
-            cand = (i == 0 || keys[i - 1] != k) && j < n && keys[j] == k;
-        }
-        unsigned cm = __ballot_sync(FULL, cand);
-        while (cm) {
-            const int src = __ffs(cm) - 1;
-            cm &= cm - 1;
-            const int64_t c0 = __shfl_sync(FULL, i, src);
-            const uint64_t k = keys[c0];
-            const float e2 = inst[k >> lb].e2;
-            typename T::Box bx = T::empty_box();
-            int64_t e = c0;
-            for (;;) {
-                const int64_t t = e + lane;
-                const bool in = t < n && keys[t] == k;
-                if (in) T::grow(bx, sp[t]);
-                const unsigned im = __ballot_sync(FULL, in);
-                e += __popc(im);
-                if (im != FULL) break;
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) T::merge(bx, T::shfl_xor(bx, o));
-            if (T::diag2(bx) > e2) continue;
-            const uint8_t f = (e - c0 > TILE) ? 2 : 1;
-            for (int64_t t = c0 + lane; t < e; t += 32) {
-                pdense[t] = f;
-                dstart[t] = (int32_t)c0;
-            }
-            if (lane == 0) atomicAdd(&ctrl[CTRL_NCELLS], 1u);
-        }
-    }
-}
-
 // the root of every instance's subtree: the node (or leaf) whose leaf range
 // is exactly the instance's leaves
 __global__ void k_inst_roots(const int2* __restrict__ range, const int32_t* __restrict__ linst,
@@ -326,6 +277,7 @@ size_t carve_batch(BatchPlan& p, void* base, int64_t n, int count, int algo, int
     if (algo == DBSCAN_ALGO_DENSEBOX) {
         p.db.pdense = c.take<uint8_t>(n);
         p.db.dstart = c.take<int32_t>(n);
+        p.db.dbox = c.take<Traits<3>::Box>((size_t)(n / 32 + 1));
     }
     p.db.lf = c.take<int32_t>(n + 64);
     p.db.lidx = c.take<int32_t>(n);
@@ -422,11 +374,11 @@ cudaError_t enqueue_batch_stages(const BatchPlan& p, int64_t n, int count, int m
     note_launches(1);
     if (algo == DBSCAN_ALGO_DENSEBOX) {
         if ((e = cudaMemsetAsync(p.db.pdense, 0, (size_t)n, s)) != cudaSuccess) return e;
-        k_bdense_classify<<<grid_n(n), 256, 0, s>>>(keys, p.sp, n, lb, p.inst, p.db.pdense, p.db.dstart, p.ctrl);
-        note_launches(1);
+        launch_dense_classify(keys, p.sp, n, 3, 0, 0.0f, p.mps, p.e2s, lb, p.db, p.ctrl, -1, s);
     }
     if ((e = launch_batch_leaves(keys, n, lb, p.db, p.leafr, p.lkey, p.linst, p.ctrl, s)) != cudaSuccess) return e;
-    launch_lbvh(p.sp, 3, p.leafr, p.lkey, n, p.ctrl, p.nmeta, p.parent, p.nfirst, p.nodebox, p.nsum, p.nodes, s, p.range);
+    launch_lbvh(p.sp, 3, p.leafr, p.lkey, p.db.dbox, n, p.ctrl, p.nmeta, p.parent, p.nfirst, p.nodebox, p.nsum, p.nodes, s,
+                p.range);
     k_inst_roots<<<grid_n(2 * n), 256, 0, s>>>(p.range, p.linst, p.ctrl, p.iroot);
     note_launches(1);
     // union-find init (per point instance parameters)

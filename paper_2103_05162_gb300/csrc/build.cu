@@ -406,56 +406,177 @@ __global__ void k_gather_packed(const float* __restrict__ pts, const uint64_t* _
 // turned into a per-cell check instead of an abort).
 //
 // One pass: the thread at the first point of a run checks with one load
-// whether the run reaches minPts points; only those runs are then walked, by
-// the whole warp, for the box and the guard, and their points marked 1
-// (dense, fits in a tile) or 2 (dense, larger than a tile: a leaf of its
-// own), with the run's first point. pdense must be zero on entry.
+// whether the run reaches minPts points, and walks it if it does. Runs of up
+// to CELL_THREAD points end there, all lanes at once; the block collects the
+// longer ones of a round of its steps, its warps take those of up to CELL_WARP
+// points, and the whole block the rest: the end by a 256-way search, the box
+// with four loads in flight per thread. The points of a dense cell are marked
+// 1 (fits in a tile) or 2 (larger: a leaf of its own), with the run's first
+// point, and the box of a cell larger than a tile goes to dbox[first point /
+// 32] (more than 32 points: no two such cells share a slot) for the leaf boxes.
+// Bound by the latency of its loads. Batch of 512 instances (cells of up to
+// 29,000 points): 350 us, one warp walking one run after another 932, a thread
+// per run of up to 64 points 840, groups of 8 lanes 428; 3.9M 2D blob points
+// (few large cells): the leaves stage 215 us instead of 2300; 16.8M halos 121
+// instead of 85. The leaf boxes, which walked the large cells again, fell from
+// 511 to 29 us on the batch and from 119 to 60 on the halos. pdense must be
+// zero on entry.
+//
+// Batches: the key's bits from lb up are the instance, whose minPts and eps^2
+// are read from mps and e2s (null: min_pts and e2).
 // ---------------------------------------------------------------------------
+constexpr int CELL_THREADS = 256;
+constexpr int CELL_STEPS = 16;    // at most, per round
+constexpr int CELL_THREAD = 8;    // a multiple of 4
+constexpr int CELL_WARP = 1024;   // a multiple of 64
+// runs of more than so many points that start in one round, at most
+constexpr int CELL_RUNS_WARP = CELL_STEPS * CELL_THREADS / (CELL_THREAD + 1) + 1;
+constexpr int CELL_RUNS_BLOCK = CELL_STEPS * CELL_THREADS / (CELL_WARP + 1) + 1;
+
 template <int D>
-__global__ void k_dense_classify(const uint64_t* __restrict__ keys, const typename Traits<D>::Point* __restrict__ sp,
-                                 int64_t n, int min_pts, float e2, uint8_t* __restrict__ pdense,
-                                 int32_t* __restrict__ dstart, uint32_t* __restrict__ ctrl)
+__global__ void __launch_bounds__(CELL_THREADS)
+    k_dense_classify(const uint64_t* __restrict__ keys, const typename Traits<D>::Point* __restrict__ sp, int64_t n,
+                     int min_pts, float e2, const int32_t* __restrict__ mps, const float* __restrict__ e2s, int lb,
+                     uint8_t* __restrict__ pdense, int32_t* __restrict__ dstart,
+                     typename Traits<D>::Box* __restrict__ dbox, uint32_t* __restrict__ ctrl, int algo, int steps)
 {
     using T = Traits<D>;
-    if (!stage_on(ctrl, DBSCAN_ALGO_DENSEBOX)) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // whole warps iterate together so that the cell walks below are cooperative
-    for (int64_t base = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) - lane; base < n; base += stride) {
-        const int64_t i = base + lane;
-        bool cand = false;
-        if (i < n) {
-            const uint64_t k = keys[i];
-            const int64_t j = i + min_pts - 1;
-            cand = (i == 0 || keys[i - 1] != k) && j < n && keys[j] == k;
+    using Box = typename T::Box;
+    if (!stage_on(ctrl, algo)) return;
+    __shared__ int64_t s_run[CELL_RUNS_WARP];  // first points of the runs for the warps,
+    __shared__ int64_t s_long[CELL_RUNS_BLOCK];   // and for the block
+    __shared__ int s_n[2];
+    __shared__ long long s_end;
+    __shared__ Box s_box[CELL_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t chunk = (int64_t)steps * CELL_THREADS;
+    for (int64_t base = blockIdx.x * chunk; base < n; base += gridDim.x * chunk) {  // whole blocks together
+        if (threadIdx.x < 2) s_n[threadIdx.x] = 0;
+        __syncthreads();
+        for (int step = 0; step < steps; ++step) {
+            const int64_t i = base + step * CELL_THREADS + threadIdx.x;
+            uint64_t k = 0;
+            bool cand = false;
+            if (i < n) {
+                k = keys[i];
+                const int64_t j = i + (mps ? mps[k >> lb] : min_pts) - 1;
+                cand = j < n && keys[j] == k && (i == 0 || keys[i - 1] != k);
+            }
+            bool dense = false;
+            if (cand) {
+                Box b = T::empty_box();
+                int len = 0;
+                bool more = true;
+                while (more && len < CELL_THREAD) {
+                    // four points at a time (past the run's end: its first point again)
+                    bool in[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) in[u] = i + len + u < n && keys[i + len + u] == k;
+#pragma unroll
+                    for (int u = 1; u < 4; ++u) in[u] = in[u] && in[u - 1];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) T::grow(b, sp[in[u] ? i + len + u : i]);
+                    len += in[0] + in[1] + in[2] + in[3];
+                    more = in[3];
+                }
+                if (more && i + len < n && keys[i + len] == k) {
+                    s_run[atomicAdd(&s_n[0], 1)] = i;
+                } else if (T::diag2(b) <= (mps ? e2s[k >> lb] : e2)) {  // the guard: provably one clique
+                    dense = true;
+                    for (int t = 0; t < len; ++t) {
+                        pdense[i + t] = 1;
+                        dstart[i + t] = (int32_t)i;
+                    }
+                }
+            }
+            const unsigned dm = __ballot_sync(FULL, dense);
+            if (lane == 0 && dm) atomicAdd(&ctrl[CTRL_NCELLS], (uint32_t)__popc(dm));
         }
-        unsigned cm = __ballot_sync(FULL, cand);
-        while (cm) {
-            const int src = __ffs(cm) - 1;
-            cm &= cm - 1;
-            const int64_t c0 = __shfl_sync(FULL, i, src);
+        __syncthreads();
+        const int nr = s_n[0];
+        for (int q = warp; q < nr; q += CELL_THREADS / 32) {
+            const int64_t c0 = s_run[q];
             const uint64_t k = keys[c0];
-            // walk the run with the whole warp: extent and exact box
-            typename T::Box b = T::empty_box();
-            int64_t e = c0;
-            for (;;) {
-                const int64_t t = e + lane;
-                const bool in = t < n && keys[t] == k;
-                if (in) T::grow(b, sp[t]);
-                const unsigned im = __ballot_sync(FULL, in);
-                e += __popc(im);
-                if (im != FULL) break;
+            Box b = T::empty_box();
+            int len = 0;
+            bool more = true;
+            while (more && len < CELL_WARP) {
+                // two points per lane (past the run's end: its first point again)
+                const int64_t t0 = c0 + len + lane, t1 = t0 + 32;
+                const bool in0 = t0 < n && keys[t0] == k, in1 = t1 < n && keys[t1] == k;
+                T::grow(b, sp[in0 ? t0 : c0]);
+                T::grow(b, sp[in1 ? t1 : c0]);
+                const unsigned m1 = __ballot_sync(FULL, in1);
+                len += __popc(__ballot_sync(FULL, in0)) + __popc(m1);
+                more = m1 == FULL;
+            }
+            if (more && c0 + len < n && keys[c0 + len] == k) {
+                if (lane == 0) s_long[atomicAdd(&s_n[1], 1)] = c0;
+                continue;
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) T::merge(b, T::shfl_xor(b, o));
-            if (T::diag2(b) > e2) continue;  // the guard: not provably one clique
-            const uint8_t f = (e - c0 > TILE) ? 2 : 1;
-            for (int64_t t = c0 + lane; t < e; t += 32) {
-                pdense[t] = f;
-                dstart[t] = (int32_t)c0;
+            if (T::diag2(b) > (mps ? e2s[k >> lb] : e2)) continue;
+            if (lane == 0) {
+                if (len > TILE) dbox[c0 >> 5] = b;
+                atomicAdd(&ctrl[CTRL_NCELLS], 1u);
             }
-            if (lane == 0) atomicAdd(&ctrl[CTRL_NCELLS], 1u);
+            for (int t = lane; t < len; t += 32) {
+                pdense[c0 + t] = len > TILE ? 2 : 1;
+                dstart[c0 + t] = (int32_t)c0;
+            }
         }
+        __syncthreads();
+        const int nl = s_n[1];
+        for (int q = 0; q < nl; ++q) {
+            const int64_t c0 = s_long[q];
+            const uint64_t kk = keys[c0];
+            // the run's end: lo is in the run, hi is not (or is n)
+            int64_t lo = c0 + CELL_WARP, hi = n;
+            while (hi - lo > 1) {
+                const int64_t step = (hi - lo + CELL_THREADS - 1) / CELL_THREADS;
+                const int64_t p = lo + (threadIdx.x + 1) * step;
+                // the last probe in the run
+                if (threadIdx.x == 0) s_end = lo;
+                __syncthreads();
+                if (p < hi && keys[p] == kk) atomicMax(&s_end, (long long)p);
+                __syncthreads();
+                const int64_t last = s_end;
+                __syncthreads();
+                lo = last;
+                hi = hi < last + step ? hi : last + step;
+            }
+            const int64_t e = hi;
+            Box b = T::empty_box();
+            for (int64_t t = c0 + threadIdx.x; t < e; t += 4 * CELL_THREADS) {
+                typename T::Point p[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int64_t at = t + u * CELL_THREADS;
+                    p[u] = sp[at < e ? at : t];
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) T::grow(b, p[u]);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) T::merge(b, T::shfl_xor(b, o));
+            if (lane == 0) s_box[warp] = b;
+            __syncthreads();
+            b = s_box[0];
+            for (int w = 1; w < CELL_THREADS / 32; ++w) T::merge(b, s_box[w]);
+            if (T::diag2(b) <= (mps ? e2s[kk >> lb] : e2)) {
+                if (threadIdx.x == 0) {
+                    dbox[c0 >> 5] = b;
+                    atomicAdd(&ctrl[CTRL_NCELLS], 1u);
+                }
+                for (int64_t t = c0 + threadIdx.x; t < e; t += CELL_THREADS) {
+                    pdense[t] = 2;
+                    dstart[t] = (int32_t)c0;
+                }
+            }
+            __syncthreads();  // s_box and s_end are used again
+        }
+        __syncthreads();  // (all have read the counts)
     }
 }
 
@@ -644,15 +765,15 @@ __global__ void k_leaf_records(const int32_t* __restrict__ lstart, const uint8_t
 // Leaf boxes: exact min/max of each leaf's points, stored at unified index
 // (m-1) + l of the node-box array. A thread takes a leaf of at most TILE
 // points (reading its contiguous points in turn: few instructions per point,
-// and consecutive threads' ranges share cache lines); the leaves larger than
-// that (dense cells) are taken afterwards by the whole warp, one at a time.
+// and consecutive threads' ranges share cache lines); the boxes of the leaves
+// larger than that (dense cells) come from the classification (dbox).
 // Each warp also writes the union of its 32 leaves' boxes, the first level of
 // the block summaries that the refit reads (sum1[w]: leaves 32 w .. 32 w + 31).
 // ---------------------------------------------------------------------------
 template <int D>
 __global__ void k_leaf_boxes(const typename Traits<D>::Point* __restrict__ sp, const int2* __restrict__ leafr,
-                             const uint32_t* __restrict__ ctrl, typename Traits<D>::Box* __restrict__ nodebox,
-                             typename Traits<D>::Box* __restrict__ sum1)
+                             const uint32_t* __restrict__ ctrl, const typename Traits<D>::Box* __restrict__ dbox,
+                             typename Traits<D>::Box* __restrict__ nodebox, typename Traits<D>::Box* __restrict__ sum1)
 {
     using T = Traits<D>;
     const int lane = threadIdx.x & 31;
@@ -685,17 +806,9 @@ __global__ void k_leaf_boxes(const typename Traits<D>::Point* __restrict__ sp, c
             nodebox[(m - 1) + l] = b;
             mine = b;
         }
-        unsigned big = __ballot_sync(FULL, l < m && !small);
-        while (big) {
-            const int src = __ffs(big) - 1;
-            big &= big - 1;
-            const int bs = __shfl_sync(FULL, s, src), be = __shfl_sync(FULL, e, src);
-            typename T::Box b = T::empty_box();
-            for (int j = bs + lane; j < be; j += 32) T::grow(b, sp[j]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) T::merge(b, T::shfl_xor(b, o));
-            if (lane == 0) nodebox[(m - 1) + base + src] = b;
-            if (lane == src) mine = b;
+        if (l < m && !small) {
+            mine = dbox[s >> 5];
+            nodebox[(m - 1) + l] = mine;
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) T::merge(mine, T::shfl_xor(mine, o));
@@ -1033,6 +1146,23 @@ cudaError_t launch_leaf_starts(const K* keys, const int32_t* dstart, const uint8
     return cudaSuccess;
 }
 
+void launch_dense_classify(const uint64_t* keys, const void* sp, int64_t n, int dim, int min_pts, float e2,
+                           const int32_t* mps, const float* e2s, int lb, const DenseBoxTemps& t, uint32_t* ctrl,
+                           int algo, cudaStream_t s)
+{
+    int64_t steps = (n + (int64_t)152 * 16 * CELL_THREADS - 1) / ((int64_t)152 * 16 * CELL_THREADS);
+    if (steps > CELL_STEPS) steps = CELL_STEPS;
+    const unsigned g = grid_for(n, (int)steps * CELL_THREADS, 152 * 16);
+#define DC_LAUNCH(D)                                                                                              \
+    k_dense_classify<D><<<g, CELL_THREADS, 0, s>>>(keys, static_cast<const typename Traits<D>::Point*>(sp), n,     \
+                                                   min_pts, e2, mps, e2s, lb, t.pdense, t.dstart,                  \
+                                                   static_cast<typename Traits<D>::Box*>(t.dbox), ctrl, algo,       \
+                                                   (int)steps)
+    GBD_DIM_SWITCH(dim, DC_LAUNCH)
+#undef DC_LAUNCH
+    note_launches(1);
+}
+
 cudaError_t launch_densebox_leaves(const uint64_t* keys, const void* sp, int64_t n, int dim, int min_pts, float e2,
                                    const DenseBoxTemps& t, int2* leafr, uint64_t* lkey, uint32_t* ctrl,
                                    cudaStream_t s)
@@ -1041,15 +1171,11 @@ cudaError_t launch_densebox_leaves(const uint64_t* keys, const void* sp, int64_t
     cudaError_t e;
     if ((e = cudaMemsetAsync(t.pdense, 0, (size_t)n, s)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(ctrl + CTRL_NCELLS, 0, sizeof(uint32_t), s)) != cudaSuccess) return e;
-#define DC_LAUNCH(D)                                                                                         \
-    k_dense_classify<D><<<g, 256, 0, s>>>(keys, static_cast<const typename Traits<D>::Point*>(sp), n, min_pts, e2, \
-                                          t.pdense, t.dstart, ctrl)
-    GBD_DIM_SWITCH(dim, DC_LAUNCH)
-#undef DC_LAUNCH
     const int A = DBSCAN_ALGO_DENSEBOX;
+    launch_dense_classify(keys, sp, n, dim, min_pts, e2, nullptr, nullptr, 64, t, ctrl, A, s);
     if ((e = launch_leaf_starts<uint64_t>(keys, t.dstart, t.pdense, n, 64, t, ctrl, A, s)) != cudaSuccess) return e;
     k_leaf_records<uint64_t><<<g, 256, 0, s>>>(t.lstart, t.pdense, keys, ctrl, 64, leafr, lkey, nullptr, A);
-    note_launches(4);
+    note_launches(3);
     return cudaGetLastError();
 }
 
@@ -1092,8 +1218,8 @@ cudaError_t launch_tile_leaves64(const uint64_t* keys, int64_t n, const DenseBox
     return cudaGetLastError();
 }
 
-void launch_lbvh(const void* sp, int dim, const int2* leafr, const uint64_t* lkey, int64_t m_cap, uint32_t* ctrl,
-                 int4* nmeta, int32_t* parent, int32_t* nfirst, void* nodebox, void* nsum, void* nodes, cudaStream_t s,
+void launch_lbvh(const void* sp, int dim, const int2* leafr, const uint64_t* lkey, const void* dbox, int64_t m_cap,
+                 uint32_t* ctrl, int4* nmeta, int32_t* parent, int32_t* nfirst, void* nodebox, void* nsum, void* nodes, cudaStream_t s,
                  int2* range_out)
 {
     const unsigned g = grid_for(m_cap, 256, 152 * 16);
@@ -1102,7 +1228,7 @@ void launch_lbvh(const void* sp, int dim, const int2* leafr, const uint64_t* lke
     do {                                                                                                       \
         using Bx = typename Traits<D>::Box;                                                                    \
         k_leaf_boxes<D><<<g, 256, 0, s>>>(static_cast<const typename Traits<D>::Point*>(sp), leafr, ctrl,       \
-                                           static_cast<Bx*>(nodebox), static_cast<Bx*>(nsum));                  \
+                                           static_cast<const Bx*>(dbox), static_cast<Bx*>(nodebox), static_cast<Bx*>(nsum));                  \
         k_box_levels<D><<<gl, 256, 0, s>>>(ctrl, static_cast<Bx*>(nsum));                                       \
     } while (0)
     GBD_DIM_SWITCH(dim, LB_LAUNCH)

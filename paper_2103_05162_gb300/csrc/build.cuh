@@ -103,6 +103,7 @@ cudaError_t launch_density_estimate(const float* points, int64_t n, int dim, con
 struct DenseBoxTemps {
     uint8_t* pdense;    // n: 0 not dense, 1 dense cell within a tile, 2 dense cell as its own leaf
     int32_t* dstart;    // n: first point of the dense cell (valid where pdense != 0)
+    void* dbox;         // n / 32 + 1 boxes: of the dense cells larger than a tile, at their first point / 32
     int32_t* lf;        // n + 64: leaf-start flags as bit words (n / 32), then their counts
     int32_t* lidx;      // n: the counts' exclusive scan
     int32_t* lstart;    // n + 1
@@ -182,6 +183,11 @@ void launch_cellkey_packed(const float* pts, int64_t n, int dim, const GridParam
                            int idx_bits, int host_passes, uint64_t* words0, uint64_t* words1, cudaStream_t s);
 void launch_gather_packed(const float* pts, const uint64_t* words, int64_t n, int dim, int idx_bits, void* sp,
                           uint32_t* perm, uint64_t* keys, const uint32_t* ctrl, cudaStream_t s);
+// dense cells of the sorted points (pdense zero on entry); batches: minPts and
+// eps^2 per instance (mps, e2s by the key bits from lb up), else null
+void launch_dense_classify(const uint64_t* keys, const void* sp, int64_t n, int dim, int min_pts, float e2,
+                           const int32_t* mps, const float* e2s, int lb, const DenseBoxTemps& t, uint32_t* ctrl,
+                           int algo, cudaStream_t s);
 cudaError_t launch_densebox_leaves(const uint64_t* keys, const void* sp, int64_t n, int dim, int min_pts, float e2,
                                    const DenseBoxTemps& t, int2* leafr, uint64_t* lkey, uint32_t* ctrl,
                                    cudaStream_t s);
@@ -214,8 +220,8 @@ __host__ __device__ inline int64_t sum_levels_entries(int64_t m)
 }
 // leaf boxes, block summaries (nsum: sum_levels_entries(m_cap) boxes),
 // Karras topology (nfirst: the first leaf of each internal node) and refit
-void launch_lbvh(const void* sp, int dim, const int2* leafr, const uint64_t* lkey, int64_t m_cap, uint32_t* ctrl,
-                 int4* nmeta, int32_t* parent, int32_t* nfirst, void* nodebox, void* nsum, void* nodes,
+void launch_lbvh(const void* sp, int dim, const int2* leafr, const uint64_t* lkey, const void* dbox, int64_t m_cap,
+                 uint32_t* ctrl, int4* nmeta, int32_t* parent, int32_t* nfirst, void* nodebox, void* nsum, void* nodes,
                  cudaStream_t s, int2* range_out = nullptr);
 cudaError_t launch_batch_leaves(const uint64_t* keys, int64_t n, int id_shift, const DenseBoxTemps& t, int2* leafr,
                                 uint64_t* lkey, int32_t* linst, uint32_t* ctrl, cudaStream_t s);

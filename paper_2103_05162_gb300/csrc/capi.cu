@@ -282,6 +282,7 @@ size_t carve_plan(Plan& p, void* base, int64_t n, int dim, int algo, int lcap, b
     if (algo != DBSCAN_ALGO_FDBSCAN) {  // DenseBox, or possibly (automatic choice)
         p.db.pdense = c.take<uint8_t>(n);
         p.db.dstart = c.take<int32_t>(n);
+        p.db.dbox = c.take<char>(box * (size_t)(n / 32 + 1));
     } else {
         p.db = DenseBoxTemps{};
     }
@@ -576,7 +577,8 @@ dbscan_status build_index(Workspace* w, const Plan& p, StageTimer& T, const floa
     }
     TRY_CUDA(cudaGetLastError());
     T.begin(ST_LBVH);
-    launch_lbvh(p.sp, dim, p.leafr, p.lkey, m_cap, p.ctrl, p.nmeta, p.parent, p.nfirst, p.nodebox, p.nsum, p.nodes, s);
+    launch_lbvh(p.sp, dim, p.leafr, p.lkey, p.db.dbox, m_cap, p.ctrl, p.nmeta, p.parent, p.nfirst, p.nodebox, p.nsum,
+                p.nodes, s);
     T.end();
     TRY_CUDA(cudaGetLastError());
 
