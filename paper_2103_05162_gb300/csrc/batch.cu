@@ -279,10 +279,8 @@ size_t carve_batch(BatchPlan& p, void* base, int64_t n, int count, int algo, int
         p.db.dstart = c.take<int32_t>(n);
         p.db.dbox = c.take<Traits<3>::Box>((size_t)(n / 32 + 1));
     }
-    p.db.lf = c.take<int32_t>(n + 64);
-    p.db.lidx = c.take<int32_t>(n);
-    p.db.lstart = c.take<int32_t>(n + 1);
-    p.db.scan_temp = c.take<int32_t>(scan_temp_words(n));
+    p.db.lf = c.take<uint32_t>(n / 32 + 1);
+    p.db.lfc = c.take<uint32_t>(LEAF_BLOCKS * 8);
     p.leafr = c.take<int2>(n);
     p.lkey = c.take<uint64_t>(n);
     p.linst = c.take<int32_t>(n);

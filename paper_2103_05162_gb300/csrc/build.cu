@@ -580,18 +580,6 @@ __global__ void __launch_bounds__(CELL_THREADS)
     }
 }
 
-// Common-prefix length of the sorted keys a (at position pa) and b (at
-// position pb, -1 outside [0, n)), equal keys told apart by position: the
-// delta of Karras (2012).
-template <typename K>
-__device__ __forceinline__ int key_delta(K a, int64_t pa, K b, int64_t pb, int64_t n)
-{
-    constexpr int KB = 8 * (int)sizeof(K);
-    if (pb < 0 || pb >= n) return -1;
-    if (a != b) return sizeof(K) == 8 ? __clzll((long long)(a ^ b)) : __clz((int)(a ^ b));
-    return KB + __clz((int)((uint32_t)pa ^ (uint32_t)pb));
-}
-
 template <typename K>
 __device__ __forceinline__ K shfl_key(K v, int src)
 {
@@ -603,161 +591,192 @@ __device__ __forceinline__ K shfl_key(K v, int src)
     }
 }
 
-// Leaf starts. A new leaf starts at point i where the node of the points'
-// radix tree (Karras: keys with position tie-break) that splits i - 1 from i
-// covers more than TILE points -- tiles are then the maximal subtrees of at
-// most TILE points, spatially compact unlike fixed runs in Morton order; and
-// at the first point of every dense cell larger than a tile, after such a
-// cell, and (batches) where the instance changes.
-// The node splitting g and g + 1 has prefix length d = delta(g, g + 1) and
-// covers the run around them of keys sharing d bits with key g; delta(g, j)
-// only falls as j moves away from g. A warp holds the keys of the 96
-// positions around its 32 points in registers (three coalesced loads per
-// lane), so four probes per point, taken by shuffles, decide most splits:
-// delta(g, g - 31) >= d or delta(g, g + 32) >= d means more than 32 points;
-// delta(g, g - 15) < d and delta(g, g + 16) < d means at most 30. For the
-// points left undecided the warp ballots, per point, which adjacent prefix
-// lengths of the window reach its d (the common prefix of sorted keys a < b
-// is the smallest adjacent one between them), and the run lengths to the
-// left and right follow from bit scans.
+// Leaves. A new leaf starts at point i where the node of the points' radix
+// tree (Karras: keys with position tie-break) that splits i - 1 from i covers
+// more than TILE points -- tiles are then the maximal subtrees of at most TILE
+// points, spatially compact unlike fixed runs in Morton order; and at the
+// first point of every dense cell larger than a tile, after such a cell, and
+// (batches) where the instance changes.
+// With e[i] the prefix length delta(i - 1, i), that node covers the run of
+// splits around i of prefix length at least e[i] (the common prefix of two
+// sorted keys is the smallest adjacent one between them): it covers more than
+// TILE points iff some TILE consecutive splits that include i have no smaller
+// prefix than e[i], i.e. iff the largest over those windows of their smallest
+// prefix reaches e[i] -- a sliding minimum and a sliding maximum of width 32,
+// five doubling steps of warp shuffles each. (Probes of the keys 15 and 31
+// positions away with ballots for the undecided took 233 us on 16.8M halos.)
+//
+// Two kernels over the same split of the positions into contiguous parts, one
+// per warp (at most LF_BLOCKS blocks, so that every block can add up the counts
+// of those before it): k_leaf_flags writes the starts as bit words and counts
+// them, k_leaf_records numbers them and writes the leaf records, a leaf's end
+// by the thread that finds the next start. Flags by key probes and ballots, a
+// three-kernel scan, starts and records took 284 us on 16.8M halos in seven
+// launches; these take 111 and 50. (One kernel with a decoupled look-back took 186:
+// the blocks stood at its barrier while their offsets came.)
 constexpr int LEAF_T = TILE;
-static_assert(LEAF_T == 32, "the window holds 32 points on each side");
+static_assert(LEAF_T == 32, "windows of one warp");
+constexpr int LF_THREADS = 256;
+constexpr int LF_WARPS = LF_THREADS / 32;
+constexpr int LF_BLOCKS = LEAF_BLOCKS;
+constexpr int LF_MIN_WINDOWS = 4;  // windows of 32 positions per warp, an even number
+
+// Sliding minima and maxima of two windows at once, one in each 16-bit half
+// (prefix lengths are at most 96, -1 outside the points).
+__device__ __forceinline__ unsigned pack2(int lo, int hi) { return __byte_perm((unsigned)lo, (unsigned)hi, 0x5410); }
+__device__ __forceinline__ int half_lo(unsigned v) { return (int)(short)v; }
+__device__ __forceinline__ int half_hi(unsigned v) { return (int)v >> 16; }
+// the smallest of e[s .. s + 31], for s in the window a (this lane: s), which
+// the window b follows
+__device__ __forceinline__ unsigned window_min(unsigned a, unsigned b, int lane)
+{
+#pragma unroll
+    for (int k = 1; k < 32; k <<= 1) {
+        // (within b, positions past its end repeat its last one: a's minima
+        // never reach them)
+        const unsigned x = __shfl_sync(FULL, a, (lane + k) & 31), y = __shfl_sync(FULL, b, (lane + k) & 31);
+        b = __vmins2(b, __shfl_down_sync(FULL, b, k));
+        a = __vmins2(a, lane + k < 32 ? x : y);
+    }
+    return a;
+}
+// the largest of v[s - 31 .. s], for s in the window b, which follows a
+__device__ __forceinline__ unsigned window_max(unsigned a, unsigned b, int lane)
+{
+#pragma unroll
+    for (int k = 1; k < 32; k <<= 1) {
+        const unsigned x = __shfl_sync(FULL, a, (lane - k) & 31), y = __shfl_sync(FULL, b, (lane - k) & 31);
+        a = __vmaxs2(a, __shfl_up_sync(FULL, a, k));
+        b = __vmaxs2(b, lane >= k ? y : x);
+    }
+    return b;
+}
 
 template <typename K>
-__global__ void k_leaf_flags(const K* __restrict__ keys, const int32_t* __restrict__ dstart,
-                             const uint8_t* __restrict__ pdense, int64_t n, int id_shift, uint32_t* __restrict__ lfw,
-                             int32_t* __restrict__ lfc, const uint32_t* __restrict__ ctrl, int algo)
+__global__ void __launch_bounds__(LF_THREADS)
+    k_leaf_flags(const K* __restrict__ keys, const int32_t* __restrict__ dstart, const uint8_t* __restrict__ pdense,
+                 int64_t n, int windows, int id_shift, uint32_t* __restrict__ words, uint32_t* __restrict__ counts,
+                 const uint32_t* __restrict__ ctrl, int algo)
 {
     if (!stage_on(ctrl, algo)) return;
     const int lane = threadIdx.x & 31;
-    const int64_t warp0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int prev = (lane + 31) & 31;
-    for (int64_t base = warp0 * 32; base < n; base += nwarps * 32) {  // whole warps iterate together
-        // window: positions base - 32 + lane, base + lane, base + 32 + lane
-        const int64_t p0 = base - 32 + lane, p1 = base + lane, p2 = base + 32 + lane;
-        const K k0 = p0 >= 0 ? keys[p0] : K(0);  // (p0 < base < n)
-        const K k1 = p1 < n ? keys[p1] : K(0);
-        const K k2 = p2 < n ? keys[p2] : K(0);
-        // this lane's point i = p1 and split g = i - 1 (all lanes take part in
-        // every shuffle; lane-dependent sources pick the window segment)
-        const int64_t i = p1, g = i - 1;
-        K kg = shfl_key(k1, prev);
-        const K kg_first = shfl_key(k0, 31);
-        if (lane == 0) kg = kg_first;
-        const K kr_a = shfl_key(k2, prev), kr_b = shfl_key(k1, 31);      // g + 32
-        const K kl_a = shfl_key(k0, (lane + 16) & 31), kl_b = shfl_key(k1, (lane + 16) & 31);  // g - 15
-        const K km_a = shfl_key(k1, (lane + 15) & 31), km_b = shfl_key(k2, (lane + 15) & 31);  // g + 16
-        const K k_right32 = lane == 0 ? kr_b : kr_a;
-        const K k_left15 = lane < 16 ? kl_a : kl_b;
-        const K k_right16 = lane <= 16 ? km_a : km_b;
-        const bool generic = i < n && i > 0;
-        int d = -1;
-        int state = 0;  // 1 exceeds, 2 does not, 0 undecided
-        if (generic) {
-            d = key_delta(kg, g, k1, i, n);
-            if (key_delta(kg, g, k0, g - 31, n) >= d || key_delta(kg, g, k_right32, g + 32, n) >= d)
-                state = 1;
-            else if (key_delta(kg, g, k_left15, g - 15, n) < d && key_delta(kg, g, k_right16, g + 16, n) < d)
-                state = 2;
-        } else {
-            state = 2;
-        }
-        unsigned und = __ballot_sync(FULL, state == 0);
-        if (und) {
-            // adjacent prefix lengths of the window; -1 outside [0, n)
-            K n0 = shfl_key(k0, (lane + 1) & 31), n1 = shfl_key(k1, (lane + 1) & 31),
-              n2 = shfl_key(k2, (lane + 1) & 31);
-            const K f1 = shfl_key(k1, 0), f2 = shfl_key(k2, 0);
-            if (lane == 31) {
-                n0 = f1;
-                n1 = f2;
-                n2 = base + 64 < n ? keys[base + 64] : K(0);
-            }
-            const int w0 = p0 >= 0 ? key_delta(k0, p0, n0, p0 + 1, n) : -1;
-            const int w1 = p1 < n ? key_delta(k1, p1, n1, p1 + 1, n) : -1;
-            const int w2 = p2 < n ? key_delta(k2, p2, n2, p2 + 1, n) : -1;
-            uint32_t m0 = 0, m1 = 0, m2 = 0;
-            while (und) {
-                const int src = __ffs(und) - 1;
-                und &= und - 1;
-                const int ds = __shfl_sync(FULL, d, src);
-                const uint32_t b0 = __ballot_sync(FULL, w0 >= ds);
-                const uint32_t b1 = __ballot_sync(FULL, w1 >= ds);
-                const uint32_t b2 = __ballot_sync(FULL, w2 >= ds);
-                if (lane == src) {
-                    m0 = b0;
-                    m1 = b1;
-                    m2 = b2;
+    const int warp = blockIdx.x * LF_WARPS + (threadIdx.x >> 5);
+    const int64_t base64 = (int64_t)warp * (32 * windows);
+    const int base = base64 < n ? (int)base64 : (int)n;  // (positions fit 31 bits)
+    const int np = (int)n;
+
+    // the splits' prefix lengths of the window at p (e[p + lane]; -1 outside
+    // the points), given its keys and the last key before it
+    auto key_at = [&](int i) { return (unsigned)i < (unsigned)np ? keys[i] : K(0); };
+    auto splits = [&](int p, K k, K before) {
+        K kp = shfl_key(k, (lane + 31) & 31);
+        if (lane == 0) kp = before;
+        const int i = p + lane;
+        constexpr int KB = 8 * (int)sizeof(K);
+        const int d = k != kp ? (sizeof(K) == 8 ? __clzll((long long)(k ^ kp)) : __clz((int)(k ^ kp)))
+                              : KB + __clz(i ^ (i - 1));
+        return i >= 1 && i < np ? d : -1;
+    };
+    uint32_t count = 0;
+    if (base < np) {
+        K kc = key_at(base + lane), k1 = key_at(base + 32 + lane), k2 = key_at(base + 64 + lane);
+        const K kp = key_at(base - 32 + lane);
+        int ec = splits(base, kc, shfl_key(kp, 31));
+        int wp = half_lo(window_min(pack2(splits(base - 32, kp, key_at(base - 33)), 0), pack2(ec, 0), lane));
+        K kprev = shfl_key(kp, 31);  // the key before the current window
+        unsigned carry = pdense && base > 0 && pdense[base - 1] == 2;
+#pragma unroll 1
+        for (int w = 0; w < windows && base + 32 * (int64_t)w < n; w += 2) {
+            const int p = base + 32 * w;
+            const int e1 = splits(p + 32, k1, shfl_key(kc, 31)), e2 = splits(p + 64, k2, shfl_key(k1, 31));
+            const K k3 = key_at(p + 96 + lane), k4 = key_at(p + 128 + lane);  // (in flight during this step)
+            const unsigned wc = window_min(pack2(ec, e1), pack2(e1, e2), lane);
+            const unsigned mx = window_max(pack2(wp, half_lo(wc)), wc, lane);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int i = p + 32 * h + lane;
+                const bool in = i < np;
+                unsigned word = __ballot_sync(FULL, in && (h ? half_hi(mx) >= e1 : half_lo(mx) >= ec));
+                if (id_shift < 64) {
+                    const K k = h ? k1 : kc, before = h ? shfl_key(kc, 31) : kprev;
+                    K kl = shfl_key(k, (lane + 31) & 31);
+                    if (lane == 0) kl = before;
+                    word |= __ballot_sync(FULL, in && ((uint64_t)k >> id_shift) != ((uint64_t)kl >> id_shift));
                 }
+                if (pdense) {
+                    // dense cells larger than a tile: only their first point
+                    // starts a leaf, and the point after them does
+                    const unsigned d2 = __ballot_sync(FULL, in && pdense[in ? i : 0] == 2);
+                    if (d2 | carry) {
+                        const unsigned st = __ballot_sync(FULL, ((d2 >> lane) & 1u) && dstart[in ? i : 0] == i);
+                        const unsigned valid = __ballot_sync(FULL, in);
+                        word = ((word | ((d2 << 1) | carry)) & ~d2 & valid) | st;
+                    }
+                    carry = d2 >> 31;
+                }
+                if (p + 32 * h == 0) word |= 1u;
+                if (lane == 0 && p + 32 * h < np) words[(p >> 5) + h] = word;
+                count += __popc(word);
             }
-            if (state == 0) {
-                // window index of g is lane + 31
-                const uint64_t lo = (uint64_t)m0 | ((uint64_t)m1 << 32), hi = m2;
-                const int pg = lane + 31;
-                const uint64_t below = ~lo & ((1ull << pg) - 1ull);
-                const int r_left = below ? pg - 1 - (63 - __clzll((long long)below)) : pg;
-                const uint64_t y = (lo >> (pg + 1)) | (hi << (63 - pg));
-                const int r_right = ~y ? __ffsll((long long)~y) - 1 : 64;
-                state = (r_left + r_right + 2) > LEAF_T ? 1 : 2;
-            }
-        }
-        bool f = false;
-        if (i >= n) f = false;
-        else if (i == 0) f = true;
-        else if (id_shift < 64 && ((uint64_t)k1 >> id_shift) != ((uint64_t)kg >> id_shift)) f = true;
-        else if (pdense && pdense[i] == 2) f = dstart[i] == (int32_t)i;
-        else if (pdense && pdense[i - 1] == 2) f = true;
-        else f = state == 1;
-        // the window's 32 flags as one word, and how many are set
-        const unsigned word = __ballot_sync(FULL, f);
-        if (lane == 0) {
-            lfw[base >> 5] = word;
-            lfc[base >> 5] = __popc(word);
+            kprev = shfl_key(k1, 31);
+            kc = k2;
+            k1 = k3;
+            k2 = k4;
+            ec = e2;
+            wp = half_hi(wc);
         }
     }
+
+    if (lane == 0) counts[warp] = count;
 }
 
-// Leaf starts from the flag words (bit b of word w: position 32 w + b
-// starts a leaf) and woff, the exclusive scan of their counts: one thread
-// per word writes its starts in order; the last word's thread writes m and
-// the closing entry lstart[m] = n.
-__global__ void k_leaf_write(const uint32_t* __restrict__ lfw, const int32_t* __restrict__ woff, int64_t nw,
-                             int64_t n, int32_t* __restrict__ lstart, uint32_t* __restrict__ ctrl, int algo)
-{
-    // skipped (aborted run, or the other algorithm's chain): m stays 0 and
-    // every later stage finds no leaves
-    if (!stage_on(ctrl, algo)) return;
-    for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < nw; w += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t word = lfw[w];
-        int32_t o = woff[w];
-        while (word) {
-            const int b = __ffs((int)word) - 1;
-            word &= word - 1;
-            lstart[o++] = (int32_t)(w * 32 + b);
-        }
-        if (w == nw - 1) {
-            lstart[o] = (int32_t)n;
-            ctrl[CTRL_M] = (uint32_t)o;
-        }
-    }
-}
-
-// leaf records (start, end | dense << 31) and the leaf keys
 template <typename K>
-__global__ void k_leaf_records(const int32_t* __restrict__ lstart, const uint8_t* __restrict__ pdense,
-                               const K* __restrict__ keys, const uint32_t* __restrict__ ctrl, int id_shift,
-                               int2* __restrict__ leafr, uint64_t* __restrict__ lkey, int32_t* __restrict__ linst,
-                               int algo)
+__global__ void __launch_bounds__(LF_THREADS)
+    k_leaf_records(const K* __restrict__ keys, const uint8_t* __restrict__ pdense, int64_t n, int windows, int id_shift,
+                   const uint32_t* __restrict__ words, const uint32_t* __restrict__ counts, int2* __restrict__ leafr,
+                   uint64_t* __restrict__ lkey, int32_t* __restrict__ linst, uint32_t* __restrict__ ctrl, int algo)
 {
+    // (skipped -- aborted run, or the other algorithm's chain --: m stays 0
+    // and every later stage finds no leaves)
     if (!stage_on(ctrl, algo)) return;
-    const int64_t m = ctrl[CTRL_M];
-    for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < m; l += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t s = lstart[l], e = lstart[l + 1];
-        const uint32_t dense = (pdense && pdense[s] == 2) ? 1u : 0u;
-        leafr[l] = make_int2(s, (int32_t)((uint32_t)e | (dense << 31)));
-        lkey[l] = (uint64_t)keys[s];
-        if (linst) linst[l] = (int32_t)((uint64_t)keys[s] >> id_shift);
+    __shared__ uint32_t s_sum[LF_WARPS];
+    const int lane = threadIdx.x & 31, wb = threadIdx.x >> 5;
+    const int warp = blockIdx.x * LF_WARPS + wb;
+    // the starts before this block: all counts before it, by all threads
+    uint32_t sum = 0;
+    for (int j = threadIdx.x; j < blockIdx.x * LF_WARPS; j += LF_THREADS) sum += counts[j];
+    sum = __reduce_add_sync(FULL, sum);
+    if (lane == 0) s_sum[wb] = sum;
+    __syncthreads();
+    uint32_t o = 0;
+#pragma unroll
+    for (int w = 0; w < LF_WARPS; ++w) o += s_sum[w];
+    for (int w = 0; w < wb; ++w) o += counts[blockIdx.x * LF_WARPS + w];
+    const int64_t base = (int64_t)warp * (32 * windows);
+    const unsigned lt = (1u << lane) - 1u;
+    unsigned mine = 0;
+    for (int w = 0; w < windows && base + 32 * (int64_t)w < n; ++w) {
+        if ((w & 31) == 0) {  // the next 32 words, one per lane
+            const int64_t at = (base >> 5) + w + lane;
+            mine = w + lane < windows && 32 * at < n ? words[at] : 0u;
+        }
+        const unsigned word = __shfl_sync(FULL, mine, w & 31);
+        if (!word) continue;
+        const int64_t i = base + 32 * w + lane;
+        if ((word >> lane) & 1u) {
+            const uint32_t l = o + __popc(word & lt);
+            const uint64_t k = (uint64_t)keys[i];
+            leafr[l].x = (int32_t)i;
+            lkey[l] = k;
+            if (linst) linst[l] = (int32_t)(k >> id_shift);
+            if (l > 0) leafr[l - 1].y = (int32_t)((uint32_t)i | (pdense && pdense[i - 1] == 2 ? 0x80000000u : 0u));
+        }
+        o += __popc(word);
+    }
+    // the warp of the last position: the last leaf's end and the number of leaves
+    if (lane == 0 && base < n && base + 32 * (int64_t)windows >= n) {
+        leafr[o - 1].y = (int32_t)((uint32_t)n | (pdense && pdense[n - 1] == 2 ? 0x80000000u : 0u));
+        ctrl[CTRL_M] = o;
     }
 }
 
@@ -1129,21 +1148,22 @@ void launch_gather(const float* pts, const uint32_t* perm, int64_t n, int dim, v
     note_launches(1);
 }
 
-// Leaf starts of n sorted keys into t.lstart and m into ctrl (flags as bit
-// words in t.lf, their counts after them, the counts' scan in t.lidx).
+// Leaves of n sorted keys: records and keys, and m into ctrl
 template <typename K>
-cudaError_t launch_leaf_starts(const K* keys, const int32_t* dstart, const uint8_t* pdense, int64_t n, int id_shift,
-                               const DenseBoxTemps& t, uint32_t* ctrl, int algo, cudaStream_t s)
+cudaError_t launch_leaves(const K* keys, const int32_t* dstart, const uint8_t* pdense, int64_t n, int id_shift,
+                          const DenseBoxTemps& t, int2* leafr, uint64_t* lkey, int32_t* linst, uint32_t* ctrl, int algo,
+                          cudaStream_t s)
 {
-    const int64_t nw = (n + 31) / 32;
-    uint32_t* words = reinterpret_cast<uint32_t*>(t.lf);
-    int32_t* counts = t.lf + nw;
-    k_leaf_flags<K><<<grid_for(n, 256, 152 * 16), 256, 0, s>>>(keys, dstart, pdense, n, id_shift, words, counts,
-                                                                ctrl, algo);
-    cudaError_t e;
-    if ((e = scan_i32(counts, t.lidx, nw, SCAN_ADD, false, t.scan_temp, s)) != cudaSuccess) return e;
-    k_leaf_write<<<grid_for(nw, 256, 152 * 16), 256, 0, s>>>(words, t.lidx, nw, n, t.lstart, ctrl, algo);
-    return cudaSuccess;
+    const int64_t per = (int64_t)LF_BLOCKS * LF_THREADS * 2;
+    int64_t w2 = (n + per - 1) / per;
+    if (w2 < LF_MIN_WINDOWS / 2) w2 = LF_MIN_WINDOWS / 2;
+    const int windows = (int)(2 * w2);
+    const unsigned g = (unsigned)((n + (int64_t)LF_THREADS * windows - 1) / ((int64_t)LF_THREADS * windows));
+    k_leaf_flags<K><<<g, LF_THREADS, 0, s>>>(keys, dstart, pdense, n, windows, id_shift, t.lf, t.lfc, ctrl, algo);
+    k_leaf_records<K><<<g, LF_THREADS, 0, s>>>(keys, pdense, n, windows, id_shift, t.lf, t.lfc, leafr, lkey, linst, ctrl,
+                                               algo);
+    note_launches(2);
+    return cudaGetLastError();
 }
 
 void launch_dense_classify(const uint64_t* keys, const void* sp, int64_t n, int dim, int min_pts, float e2,
@@ -1167,16 +1187,12 @@ cudaError_t launch_densebox_leaves(const uint64_t* keys, const void* sp, int64_t
                                    const DenseBoxTemps& t, int2* leafr, uint64_t* lkey, uint32_t* ctrl,
                                    cudaStream_t s)
 {
-    const unsigned g = grid_for(n, 256, 152 * 16);
     cudaError_t e;
     if ((e = cudaMemsetAsync(t.pdense, 0, (size_t)n, s)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(ctrl + CTRL_NCELLS, 0, sizeof(uint32_t), s)) != cudaSuccess) return e;
     const int A = DBSCAN_ALGO_DENSEBOX;
     launch_dense_classify(keys, sp, n, dim, min_pts, e2, nullptr, nullptr, 64, t, ctrl, A, s);
-    if ((e = launch_leaf_starts<uint64_t>(keys, t.dstart, t.pdense, n, 64, t, ctrl, A, s)) != cudaSuccess) return e;
-    k_leaf_records<uint64_t><<<g, 256, 0, s>>>(t.lstart, t.pdense, keys, ctrl, 64, leafr, lkey, nullptr, A);
-    note_launches(3);
-    return cudaGetLastError();
+    return launch_leaves<uint64_t>(keys, t.dstart, t.pdense, n, 64, t, leafr, lkey, nullptr, ctrl, A, s);
 }
 
 // Leaves of a batch: keys carry the instance in their bits from id_shift up;
@@ -1185,37 +1201,21 @@ cudaError_t launch_densebox_leaves(const uint64_t* keys, const void* sp, int64_t
 cudaError_t launch_batch_leaves(const uint64_t* keys, int64_t n, int id_shift, const DenseBoxTemps& t, int2* leafr,
                                 uint64_t* lkey, int32_t* linst, uint32_t* ctrl, cudaStream_t s)
 {
-    const unsigned g = grid_for(n, 256, 152 * 16);
-    cudaError_t e;
-    if ((e = launch_leaf_starts<uint64_t>(keys, t.dstart, t.pdense, n, id_shift, t, ctrl, -1, s)) != cudaSuccess)
-        return e;
-    k_leaf_records<uint64_t><<<g, 256, 0, s>>>(t.lstart, t.pdense, keys, ctrl, id_shift, leafr, lkey, linst, -1);
-    note_launches(3);
-    return cudaGetLastError();
+    return launch_leaves<uint64_t>(keys, t.dstart, t.pdense, n, id_shift, t, leafr, lkey, linst, ctrl, -1, s);
 }
 
 cudaError_t launch_tile_leaves(const uint32_t* keys32, int64_t n, const DenseBoxTemps& t, int2* leafr,
                                uint64_t* lkey, uint32_t* ctrl, cudaStream_t s)
 {
-    const unsigned g = grid_for(n, 256, 152 * 16);
-    cudaError_t e;
-    const int A = DBSCAN_ALGO_FDBSCAN;
-    if ((e = launch_leaf_starts<uint32_t>(keys32, nullptr, nullptr, n, 64, t, ctrl, A, s)) != cudaSuccess) return e;
-    k_leaf_records<uint32_t><<<g, 256, 0, s>>>(t.lstart, nullptr, keys32, ctrl, 64, leafr, lkey, nullptr, A);
-    note_launches(3);
-    return cudaGetLastError();
+    return launch_leaves<uint32_t>(keys32, nullptr, nullptr, n, 64, t, leafr, lkey, nullptr, ctrl,
+                                   DBSCAN_ALGO_FDBSCAN, s);
 }
 
 cudaError_t launch_tile_leaves64(const uint64_t* keys, int64_t n, const DenseBoxTemps& t, int2* leafr,
                                  uint64_t* lkey, uint32_t* ctrl, cudaStream_t s)
 {
-    const unsigned g = grid_for(n, 256, 152 * 16);
-    cudaError_t e;
-    const int A = DBSCAN_ALGO_FDBSCAN;
-    if ((e = launch_leaf_starts<uint64_t>(keys, nullptr, nullptr, n, 64, t, ctrl, A, s)) != cudaSuccess) return e;
-    k_leaf_records<uint64_t><<<g, 256, 0, s>>>(t.lstart, nullptr, keys, ctrl, 64, leafr, lkey, nullptr, A);
-    note_launches(3);
-    return cudaGetLastError();
+    return launch_leaves<uint64_t>(keys, nullptr, nullptr, n, 64, t, leafr, lkey, nullptr, ctrl, DBSCAN_ALGO_FDBSCAN,
+                                   s);
 }
 
 void launch_lbvh(const void* sp, int dim, const int2* leafr, const uint64_t* lkey, const void* dbox, int64_t m_cap,

@@ -100,14 +100,15 @@ cudaError_t launch_density_estimate(const float* points, int64_t n, int dim, con
                                    float auto_fraction, float auto_occupancy, const EstBuffers& eb, uint32_t* ctrl,
                                    cudaStream_t s);
 
+// blocks of 8 warps of the leaf kernels, at most
+constexpr int LEAF_BLOCKS = 1216;
+
 struct DenseBoxTemps {
     uint8_t* pdense;    // n: 0 not dense, 1 dense cell within a tile, 2 dense cell as its own leaf
     int32_t* dstart;    // n: first point of the dense cell (valid where pdense != 0)
     void* dbox;         // n / 32 + 1 boxes: of the dense cells larger than a tile, at their first point / 32
-    int32_t* lf;        // n + 64: leaf-start flags as bit words (n / 32), then their counts
-    int32_t* lidx;      // n: the counts' exclusive scan
-    int32_t* lstart;    // n + 1
-    int32_t* scan_temp; // scan_temp_words(n)
+    uint32_t* lf;       // n / 32 + 1: leaf-start flags, one bit per position
+    uint32_t* lfc;      // LEAF_BLOCKS * 8: starts per warp of the leaf kernels
 };
 
 // ---------------------------------------------------------------------------

@@ -286,10 +286,8 @@ size_t carve_plan(Plan& p, void* base, int64_t n, int dim, int algo, int lcap, b
     } else {
         p.db = DenseBoxTemps{};
     }
-    p.db.lf = c.take<int32_t>(n + 64);
-    p.db.lidx = c.take<int32_t>(n);
-    p.db.lstart = c.take<int32_t>(n + 1);
-    p.db.scan_temp = c.take<int32_t>(scan_temp_words(n));
+    p.db.lf = c.take<uint32_t>(n / 32 + 1);
+    p.db.lfc = c.take<uint32_t>(LEAF_BLOCKS * 8);
     p.leafr = c.take<int2>(mc);
     p.lkey = c.take<uint64_t>(mc);
     p.nodebox = c.take<char>(box * (size_t)(2 * mc));

@@ -664,10 +664,4 @@ cudaError_t sort_pairs_u64(uint64_t* keys, uint32_t* vals, int64_t n, int bits, 
 cudaError_t sort_keys_u64(uint64_t* keys, int64_t n, int shift0, int bits, const SortBuffers& sb, cudaStream_t s,
                           bool* in_alt);
 
-// scan.cu: out[i] = op(in[0..i]) (inclusive) or op(in[0..i-1]) (exclusive, out[0] = identity)
-enum ScanOp { SCAN_ADD = 0, SCAN_MAX = 1 };
-size_t scan_temp_words(int64_t n);
-cudaError_t scan_i32(const int32_t* in, int32_t* out, int64_t n, ScanOp op, bool inclusive, int32_t* temp,
-                     cudaStream_t s);
-
 }  // namespace gbd
