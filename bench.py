@@ -65,8 +65,7 @@ def bytes_model(n: int, d: int, m: int, key_bytes: int, packed: bool = False) ->
 
 
 TRAFFIC_JSON = os.path.join(ROOT, "profiles", "traversal_traffic_densebox_halos.json")
-STAGE_KERNELS = {"preprocess": ("k_pre", "k_list_claims"), "main": ("k_intra", "k_kinds_count", "k_kinds_write",
-                                                                     "k_main")}
+STAGE_KERNELS = {"preprocess": ("k_pre", "k_list_claims"), "main": ("k_intra", "k_kinds", "k_main")}
 
 
 def measured_traffic(n: int, stage: str) -> float | None:

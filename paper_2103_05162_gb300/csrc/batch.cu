@@ -292,7 +292,7 @@ size_t carve_batch(BatchPlan& p, void* base, int64_t n, int count, int algo, int
     p.nsum = c.take<Traits<3>::Box>((size_t)sum_levels_entries(n));
     p.range = c.take<int2>(n);
     p.lsolid = c.take<uint8_t>(n);
-    p.klist = c.take<int32_t>(n);
+    p.klist = c.take<int32_t>(3 * n);
     p.tstart = c.take<int32_t>(n);
     p.tsib = c.take<int2>(n * TRAVERSAL_SIBCAP);
     p.tnsib = c.take<int8_t>(n);
@@ -383,6 +383,8 @@ cudaError_t enqueue_batch_stages(const BatchPlan& p, int64_t n, int count, int m
     if ((e = cudaMemsetAsync(p.ctrl + CTRL_WORK_PRE, 0, (CTRL_WORK_END - CTRL_WORK_PRE) * sizeof(uint32_t), s)) !=
         cudaSuccess)
         return e;
+    // points that keep no list (instances with minPts <= 2) read 0
+    if ((e = cudaMemsetAsync(p.nbr, 0, (size_t)n, s)) != cudaSuccess) return e;
     k_binit<<<grid_n(n), 256, 0, s>>>(keys, lb, p.inst, p.db.pdense, p.db.dstart, n, p.labels, p.core, p.ctrl);
     note_launches(1);
     if ((e = cudaMemsetAsync(p.canon, 0x7f, sizeof(int32_t) * (size_t)n, s)) != cudaSuccess) return e;

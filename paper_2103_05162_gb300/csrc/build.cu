@@ -5,26 +5,74 @@
 
 namespace gbd {
 
+// DenseBox grid (Sec. 4.2) from the bounds, in double precision: cell side
+// h = f * eps / sqrt(D) (computed by the host), enlarged when the widest axis
+// would need more than 2^max_axis_bits - 2 cells (the per-cell guard keeps
+// the result exact for any cell size, reading of Sec. 4.2); cmax_k = the
+// cell index of hi_k (plus one spare cell for rounding at the top); the key
+// interleaves `bits` bits per axis, enough for every cmax_k.
+template <int D>
+__device__ void make_grid(uint32_t* ctrl, const GridRequest& q)
+{
+    GridParams g{};
+    double h = q.side;
+    const double maxcells = (double)(1ull << q.max_axis_bits);
+    float lo[D], hi[D];
+    double ext_max = 0.0;
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+        lo[k] = ord2f(__ldcg(&ctrl[CTRL_LO + k]));
+        hi[k] = ord2f(__ldcg(&ctrl[CTRL_HI + k]));
+        ext_max = fmax(ext_max, (double)hi[k] - (double)lo[k]);
+    }
+    if (!(ext_max >= 0.0) || isinf(ext_max)) ext_max = 0.0;  // non-finite input: the run is aborted anyway
+    if (ext_max / h >= maxcells - 2.0) h = ext_max / (maxcells - 2.0);
+    const float inv_h = (float)(1.0 / h);
+    int bits = 1;
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+        g.lo[k] = lo[k];
+        double c = floor(((double)hi[k] - (double)lo[k]) * (double)inv_h) + 1.0;
+        if (!(c >= 1.0)) c = 1.0;
+        if (c > maxcells - 1.0) c = maxcells - 1.0;
+        g.cmax[k] = (uint32_t)c;
+        bits = max(bits, 32 - __clz((int)g.cmax[k]));
+    }
+    if (bits > q.max_axis_bits) bits = q.max_axis_bits;
+    g.inv_h = inv_h;
+    g.bits = bits;
+    g.morton = 1;
+    *q.gp = g;
+    ctrl[CTRL_KEYBITS] = (uint32_t)(bits * D);
+}
+
 // ---------------------------------------------------------------------------
 // K1: exact fp32 bounding box of the points, plus a flag for NaN/Inf.
 // Each thread strides over the flat coordinate array with a stride that is a
-// multiple of D, so it always sees the same axis.
+// multiple of D, so it always sees the same axis. The kernel also clears the
+// scratch that the stages after it find zeroed, and its last block computes
+// the DenseBox grids: a memset or a one-thread kernel of its own cost 2 to 7 us
+// of a small run each.
 // ---------------------------------------------------------------------------
 template <int D, int BT = bounds_threads<D>()>
 __global__ void __launch_bounds__(BT) k_bounds(const float* __restrict__ pts, int64_t n,
-                                               uint32_t* __restrict__ ctrl)
+                                               uint32_t* __restrict__ ctrl, BoundsExtra x)
 {
     __shared__ uint32_t s_lo[D], s_hi[D];
-    __shared__ int s_bad;
+    __shared__ int s_bad, s_last;
     if (threadIdx.x < D) { s_lo[threadIdx.x] = 0xffffffffu; s_hi[threadIdx.x] = 0u; }
     if (threadIdx.x == 0) s_bad = 0;
     __syncthreads();
     const int64_t total = n * D;
     const int64_t stride = (int64_t)gridDim.x * BT;
+    const int64_t first = blockIdx.x * (int64_t)BT + threadIdx.x;
+#pragma unroll
+    for (int z = 0; z < 2; ++z)
+        for (int64_t i = first; i < x.zero16[z]; i += stride) x.zero[z][i] = make_uint4(0u, 0u, 0u, 0u);
     const int axis = threadIdx.x % D;
     float lo = INFINITY, hi = -INFINITY;
     bool bad = false;
-    for (int64_t i = blockIdx.x * (int64_t)BT + threadIdx.x; i < total; i += stride) {
+    for (int64_t i = first; i < total; i += stride) {
         float v = __ldcs(pts + i);
         bad |= !isfinite(v);
         lo = fminf(lo, v);
@@ -39,60 +87,36 @@ __global__ void __launch_bounds__(BT) k_bounds(const float* __restrict__ pts, in
     if (threadIdx.x < D) {
         atomicMin(&ctrl[CTRL_LO + threadIdx.x], s_lo[threadIdx.x]);
         atomicMax(&ctrl[CTRL_HI + threadIdx.x], s_hi[threadIdx.x]);
+        __threadfence();
     }
     if (threadIdx.x == 0 && s_bad) atomicOr(&ctrl[CTRL_ABORT], ERR_NONFINITE);
+    if (x.grids == 0) return;
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&ctrl[CTRL_TICKET], 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last || threadIdx.x != 0) return;
+    __threadfence();
+    // (the run's own grid last: CTRL_KEYBITS is its)
+    for (int q = 0; q < x.grids; ++q) make_grid<D>(ctrl, x.grid[q]);
 }
 
 // the run's first kernel (see launch_run_begin)
 __global__ void k_run_begin(uint32_t* ctrl, int algo)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
+    const int t = threadIdx.x;
+    if (t == 0) {
         const uint32_t a = ctrl[CTRL_ABORT];
         if (a) ctrl[CTRL_ERR] |= a;
         ctrl[CTRL_ABORT] = 0u;
         ctrl[CTRL_ALGO] = (uint32_t)algo;
+        ctrl[CTRL_M] = 0u;
+        ctrl[CTRL_NCELLS] = 0u;
+        ctrl[CTRL_TICKET] = 0u;
     }
-}
-
-// DenseBox grid (Sec. 4.2) from the bounds on the device, in double
-// precision: cell side h = f * eps / sqrt(D), enlarged when the widest axis
-// would need more than 2^max_axis_bits - 2 cells (the per-cell guard keeps
-// the result exact for any cell size, reading of Sec. 4.2); cmax_k = the
-// cell index of hi_k (plus one spare cell for rounding at the top); the key
-// interleaves `bits` bits per axis, enough for every cmax_k.
-template <int D>
-__global__ void k_grid(uint32_t* ctrl, float eps, float factor, int max_axis_bits, GridParams* gp)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    GridParams g{};
-    double h = (double)factor * (double)eps / sqrt((double)D);
-    const double maxcells = ldexp(1.0, max_axis_bits);
-    float lo[D], hi[D];
-    double ext_max = 0.0;
-#pragma unroll
-    for (int k = 0; k < D; ++k) {
-        lo[k] = ord2f(ctrl[CTRL_LO + k]);
-        hi[k] = ord2f(ctrl[CTRL_HI + k]);
-        ext_max = fmax(ext_max, (double)hi[k] - (double)lo[k]);
+    if (t < MAX_DIM) {
+        ctrl[CTRL_LO + t] = 0xffffffffu;
+        ctrl[CTRL_HI + t] = 0u;
     }
-    if (!(ext_max >= 0.0) || isinf(ext_max)) ext_max = 0.0;  // non-finite input: the run is aborted anyway
-    if (ext_max / h >= maxcells - 2.0) h = ext_max / (maxcells - 2.0);
-    const float inv_h = (float)(1.0 / h);
-    int bits = 1;
-#pragma unroll
-    for (int k = 0; k < D; ++k) {
-        g.lo[k] = lo[k];
-        double c = floor(((double)hi[k] - (double)lo[k]) * (double)inv_h) + 1.0;
-        if (!(c >= 1.0)) c = 1.0;
-        if (c > maxcells - 1.0) c = maxcells - 1.0;
-        g.cmax[k] = (uint32_t)c;
-        while (bits < max_axis_bits && (ldexp(1.0, bits) - 1.0) < (double)g.cmax[k]) ++bits;
-    }
-    g.inv_h = inv_h;
-    g.bits = bits;
-    g.morton = 1;
-    *gp = g;
-    ctrl[CTRL_KEYBITS] = (uint32_t)(bits * D);
 }
 
 // ---------------------------------------------------------------------------
@@ -780,61 +804,6 @@ __global__ void __launch_bounds__(LF_THREADS)
     }
 }
 
-// ---------------------------------------------------------------------------
-// Leaf boxes: exact min/max of each leaf's points, stored at unified index
-// (m-1) + l of the node-box array. A thread takes a leaf of at most TILE
-// points (reading its contiguous points in turn: few instructions per point,
-// and consecutive threads' ranges share cache lines); the boxes of the leaves
-// larger than that (dense cells) come from the classification (dbox).
-// Each warp also writes the union of its 32 leaves' boxes, the first level of
-// the block summaries that the refit reads (sum1[w]: leaves 32 w .. 32 w + 31).
-// ---------------------------------------------------------------------------
-template <int D>
-__global__ void k_leaf_boxes(const typename Traits<D>::Point* __restrict__ sp, const int2* __restrict__ leafr,
-                             const uint32_t* __restrict__ ctrl, const typename Traits<D>::Box* __restrict__ dbox,
-                             typename Traits<D>::Box* __restrict__ nodebox, typename Traits<D>::Box* __restrict__ sum1)
-{
-    using T = Traits<D>;
-    const int lane = threadIdx.x & 31;
-    const int64_t m = ctrl[CTRL_M];
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; base < m; base += stride) {
-        const int64_t l = base + lane;
-        int s = 0, e = 0;
-        if (l < m) {
-            const int2 r = leafr[l];
-            s = r.x;
-            e = r.y & 0x7fffffff;
-        }
-        const bool small = l < m && e - s <= TILE;
-        typename T::Box mine = T::empty_box();
-        if (small) {
-            typename T::Box b = T::empty_box();
-            int j = s;
-            if constexpr (D == 3) {
-                // two 16-byte points per 256-bit load from an even index on
-                if ((j & 1) && j < e) T::grow(b, sp[j++]);
-                for (; j + 1 < e; j += 2) {
-                    float4 p0, p1;
-                    ldg256(&sp[j], p0, p1);
-                    T::grow(b, p0);
-                    T::grow(b, p1);
-                }
-            }
-            for (; j < e; ++j) T::grow(b, sp[j]);
-            nodebox[(m - 1) + l] = b;
-            mine = b;
-        }
-        if (l < m && !small) {
-            mine = dbox[s >> 5];
-            nodebox[(m - 1) + l] = mine;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) T::merge(mine, T::shfl_xor(mine, o));
-        if (lane == 0) sum1[base >> 5] = mine;
-    }
-}
-
 // Higher block summaries: level k (k >= 2) entry j is the union of level-1
 // entries [32^(k-1) j, 32^(k-1) (j + 1)), i.e. of 32^k consecutive leaves;
 // the levels follow each other in `sum` (level 1 first; sizes and count as
@@ -879,11 +848,10 @@ __device__ __forceinline__ int kdelta(const uint64_t* __restrict__ k, int64_t m,
     return 64 + __clz((int)((uint32_t)i ^ (uint32_t)j));
 }
 
-__global__ void k_karras(const uint64_t* __restrict__ lkey, const uint32_t* __restrict__ ctrl, int64_t m_host,
-                         int4* __restrict__ nmeta, int32_t* __restrict__ parent, int2* __restrict__ child_out,
-                         int2* __restrict__ range_out, int32_t* __restrict__ first_out)
+__device__ __forceinline__ void karras(const uint64_t* __restrict__ lkey, int64_t m, int4* __restrict__ nmeta,
+                                       int32_t* __restrict__ parent, int2* __restrict__ child_out,
+                                       int2* __restrict__ range_out, int32_t* __restrict__ first_out)
 {
-    const int64_t m = m_host >= 0 ? m_host : (int64_t)ctrl[CTRL_M];
     if (blockIdx.x == 0 && threadIdx.x == 0) parent[0] = -1;  // root (or the single leaf when m == 1)
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m - 1; i += (int64_t)gridDim.x * blockDim.x) {
         const int d = (kdelta(lkey, m, i, i + 1) - kdelta(lkey, m, i, i - 1)) > 0 ? 1 : -1;
@@ -911,6 +879,72 @@ __global__ void k_karras(const uint64_t* __restrict__ lkey, const uint32_t* __re
         if (range_out) range_out[i] = make_int2((int32_t)first, (int32_t)last);
         if (first_out) first_out[i] = (int32_t)first;
     }
+}
+
+// the topology alone (component entry point)
+__global__ void k_karras(const uint64_t* __restrict__ lkey, int64_t m, int4* __restrict__ nmeta,
+                         int32_t* __restrict__ parent, int2* __restrict__ child_out, int2* __restrict__ range_out)
+{
+    karras(lkey, m, nmeta, parent, child_out, range_out, nullptr);
+}
+
+// ---------------------------------------------------------------------------
+// Leaf boxes: exact min/max of each leaf's points, stored at unified index
+// (m-1) + l of the node-box array. A thread takes a leaf of at most TILE
+// points (reading its contiguous points in turn: few instructions per point,
+// and consecutive threads' ranges share cache lines); the boxes of the leaves
+// larger than that (dense cells) come from the classification (dbox).
+// The topology (K7) needs nothing of them, nor they of it: it shares the
+// launch. Each warp also writes the union of its 32 leaves' boxes, the first level of
+// the block summaries that the refit reads (sum1[w]: leaves 32 w .. 32 w + 31).
+// ---------------------------------------------------------------------------
+template <int D>
+__global__ void k_leaf_boxes(const typename Traits<D>::Point* __restrict__ sp, const int2* __restrict__ leafr,
+                             const uint32_t* __restrict__ ctrl, const typename Traits<D>::Box* __restrict__ dbox,
+                             typename Traits<D>::Box* __restrict__ nodebox, typename Traits<D>::Box* __restrict__ sum1,
+                             const uint64_t* __restrict__ lkey, int4* __restrict__ nmeta, int32_t* __restrict__ parent,
+                             int2* __restrict__ range_out, int32_t* __restrict__ first_out)
+{
+    using T = Traits<D>;
+    const int lane = threadIdx.x & 31;
+    const int64_t m = ctrl[CTRL_M];
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t base = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; base < m; base += stride) {
+        const int64_t l = base + lane;
+        int s = 0, e = 0;
+        if (l < m) {
+            const int2 r = leafr[l];
+            s = r.x;
+            e = r.y & 0x7fffffff;
+        }
+        const bool small = l < m && e - s <= TILE;
+        typename T::Box mine = T::empty_box();
+        if (small) {
+            typename T::Box b = T::empty_box();
+            int j = s;
+            if constexpr (D == 3) {
+                // two 16-byte points per 256-bit load from an even index on
+                if ((j & 1) && j < e) T::grow(b, sp[j++]);
+                for (; j + 1 < e; j += 2) {
+                    float4 p0, p1;
+                    ldg256(&sp[j], p0, p1);
+                    T::grow(b, p0);
+                    T::grow(b, p1);
+                }
+            }
+            for (; j < e; ++j) T::grow(b, sp[j]);
+            nodebox[(m - 1) + l] = b;
+            mine = b;
+        }
+        if (l < m && !small) {
+            mine = dbox[s >> 5];
+            nodebox[(m - 1) + l] = mine;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) T::merge(mine, T::shfl_xor(mine, o));
+        if (lane == 0) sum1[base >> 5] = mine;
+    }
+    karras(lkey, m, nmeta, parent, nullptr, range_out, first_out);
 }
 
 // ---------------------------------------------------------------------------
@@ -1059,10 +1093,10 @@ static inline unsigned grid_for(int64_t work, int threads, int max_blocks)
     return (unsigned)b;
 }
 
-void launch_bounds(const float* pts, int64_t n, int dim, uint32_t* ctrl, cudaStream_t s)
+void launch_bounds(const float* pts, int64_t n, int dim, uint32_t* ctrl, const BoundsExtra& x, cudaStream_t s)
 {
 #define BOUNDS_LAUNCH(D)                                                                            \
-    k_bounds<D><<<grid_for(n * D, bounds_threads<D>(), 152 * 8), bounds_threads<D>(), 0, s>>>(pts, n, ctrl)
+    k_bounds<D><<<grid_for(n * D, bounds_threads<D>(), 152 * 8), bounds_threads<D>(), 0, s>>>(pts, n, ctrl, x)
     GBD_DIM_SWITCH(dim, BOUNDS_LAUNCH)
 #undef BOUNDS_LAUNCH
     note_launches(1);
@@ -1071,15 +1105,6 @@ void launch_bounds(const float* pts, int64_t n, int dim, uint32_t* ctrl, cudaStr
 void launch_run_begin(uint32_t* ctrl, int algo, cudaStream_t s)
 {
     k_run_begin<<<1, 32, 0, s>>>(ctrl, algo);
-    note_launches(1);
-}
-
-void launch_grid(uint32_t* ctrl, int dim, float eps, float factor, int max_axis_bits, GridParams* gp,
-                 cudaStream_t s)
-{
-#define GRID_LAUNCH(D) k_grid<D><<<1, 32, 0, s>>>(ctrl, eps, factor, max_axis_bits, gp)
-    GBD_DIM_SWITCH(dim, GRID_LAUNCH)
-#undef GRID_LAUNCH
     note_launches(1);
 }
 
@@ -1187,9 +1212,6 @@ cudaError_t launch_densebox_leaves(const uint64_t* keys, const void* sp, int64_t
                                    const DenseBoxTemps& t, int2* leafr, uint64_t* lkey, uint32_t* ctrl,
                                    cudaStream_t s)
 {
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(t.pdense, 0, (size_t)n, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(ctrl + CTRL_NCELLS, 0, sizeof(uint32_t), s)) != cudaSuccess) return e;
     const int A = DBSCAN_ALGO_DENSEBOX;
     launch_dense_classify(keys, sp, n, dim, min_pts, e2, nullptr, nullptr, 64, t, ctrl, A, s);
     return launch_leaves<uint64_t>(keys, t.dstart, t.pdense, n, 64, t, leafr, lkey, nullptr, ctrl, A, s);
@@ -1224,30 +1246,31 @@ void launch_lbvh(const void* sp, int dim, const int2* leafr, const uint64_t* lke
 {
     const unsigned g = grid_for(m_cap, 256, 152 * 16);
     const unsigned gl = grid_for(sum_levels_entries(m_cap) * 32, 256, 152 * 4);
-#define LB_LAUNCH(D)                                                                                           \
-    do {                                                                                                       \
-        using Bx = typename Traits<D>::Box;                                                                    \
-        k_leaf_boxes<D><<<g, 256, 0, s>>>(static_cast<const typename Traits<D>::Point*>(sp), leafr, ctrl,       \
-                                           static_cast<const Bx*>(dbox), static_cast<Bx*>(nodebox), static_cast<Bx*>(nsum));                  \
-        k_box_levels<D><<<gl, 256, 0, s>>>(ctrl, static_cast<Bx*>(nsum));                                       \
+    // (the levels from 2 on: none while level 1 is read directly)
+    const bool levels = sum_level_size(m_cap, 1) > SUM_DIRECT;
+#define LB_LAUNCH(D)                                                                                                  \
+    do {                                                                                                              \
+        using Bx = typename Traits<D>::Box;                                                                           \
+        k_leaf_boxes<D><<<g, 256, 0, s>>>(static_cast<const typename Traits<D>::Point*>(sp), leafr, ctrl,              \
+                                          static_cast<const Bx*>(dbox), static_cast<Bx*>(nodebox),                    \
+                                          static_cast<Bx*>(nsum), lkey, nmeta, parent, range_out, nfirst);            \
+        if (levels) k_box_levels<D><<<gl, 256, 0, s>>>(ctrl, static_cast<Bx*>(nsum));                                 \
     } while (0)
     GBD_DIM_SWITCH(dim, LB_LAUNCH)
 #undef LB_LAUNCH
-    k_karras<<<g, 256, 0, s>>>(lkey, ctrl, -1, nmeta, parent, nullptr, range_out, nfirst);
 #define RF_LAUNCH(D)                                                                                         \
     k_refit<D><<<g, 256, 0, s>>>(ctrl, nmeta, nfirst, static_cast<typename Traits<D>::Box*>(nodebox),          \
                                  static_cast<const typename Traits<D>::Box*>(nsum),                            \
                                  static_cast<typename Traits<D>::Node*>(nodes))
     GBD_DIM_SWITCH(dim, RF_LAUNCH)
 #undef RF_LAUNCH
-    note_launches(4);
+    note_launches(levels ? 3 : 2);
 }
 
 void launch_karras_only(const uint64_t* lkey, int64_t m, int4* nmeta, int32_t* parent, int2* child_out,
                         int2* range_out, cudaStream_t s)
 {
-    k_karras<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(lkey, nullptr, m, nmeta, parent, child_out, range_out,
-                                                        nullptr);
+    k_karras<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(lkey, m, nmeta, parent, child_out, range_out);
     note_launches(1);
 }
 

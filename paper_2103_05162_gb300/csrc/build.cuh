@@ -48,6 +48,7 @@ enum : int {
     CTRL_WORK_END = 25,    // end of the per-phase counters (cleared before each phase)
     CTRL_ABORT = 26,       // error bits of the current run (ERR_*): set, every later stage does nothing
     CTRL_ALGO = 27,        // the algorithm the current run uses (DBSCAN_ALGO_FDBSCAN / _DENSEBOX)
+    CTRL_TICKET = 15,      // blocks of the bounds kernel that are done
     CTRL_KEYBITS = 28,     // DenseBox: cell-key bits of the current run's grid
     CTRL_EST_FRAC = 29,    // automatic choice: estimated dense-point share (float bits)
     CTRL_EST_OCC = 30,     // automatic choice: estimated mean cell occupancy (float bits)
@@ -156,15 +157,26 @@ __device__ __forceinline__ uint64_t interleave(const uint32_t* c)
     return key;
 }
 
-void launch_bounds(const float* pts, int64_t n, int dim, uint32_t* ctrl, cudaStream_t s);
+// a DenseBox grid from the device-side bounds: cell side f * eps / sqrt(dim)
+// (Sec. 4.2), coarsened until every axis fits max_axis_bits; goes to *gp, its
+// key width to CTRL_KEYBITS
+struct GridRequest {
+    double side;
+    int max_axis_bits;
+    GridParams* gp;
+};
+// what the bounds kernel does besides: scratch to clear (16-byte units), grids
+struct BoundsExtra {
+    uint4* zero[2] = {nullptr, nullptr};
+    int64_t zero16[2] = {0, 0};
+    int grids = 0;
+    GridRequest grid[2] = {};
+};
+void launch_bounds(const float* pts, int64_t n, int dim, uint32_t* ctrl, const BoundsExtra& x, cudaStream_t s);
 // the run's first kernel: moves CTRL_ABORT's bits into CTRL_ERR (kept for
-// the next host sync point), clears CTRL_ABORT and sets CTRL_ALGO
+// the next host sync point), clears CTRL_ABORT, the bounds and the counts, and
+// sets CTRL_ALGO
 void launch_run_begin(uint32_t* ctrl, int algo, cudaStream_t s);
-// DenseBox grid from the device-side bounds: cell side f * eps / sqrt(dim)
-// (Sec. 4.2), coarsened until every axis fits max_axis_bits; writes *gp and
-// CTRL_KEYBITS
-void launch_grid(uint32_t* ctrl, int dim, float eps, float factor, int max_axis_bits, GridParams* gp,
-                 cudaStream_t s);
 // FDbscan keys (gated on CTRL_ALGO == FDBSCAN): 32-bit Morton codes in 2D/3D
 void launch_morton32(const float* pts, int64_t n, int dim, const uint32_t* ctrl, int bits, uint32_t* keys,
                      uint32_t* vals, cudaStream_t s);
@@ -239,7 +251,7 @@ struct ClusterArgs {
     const void* nodebox;   // 2m-1 boxes (leaf boxes at m-1+l)
     const int2* leafr;     // m leaf records
     uint8_t* lsolid;       // m: the leaf's flag (nothing to do, all points core and in one set, neither)
-    int32_t* klist;        // m: leaf indices grouped by kind
+    int32_t* klist;        // 3 * m_cap: leaf indices by kind
     const uint8_t* pdense; // n or null: dense-cell flags per sorted point (DenseBox)
     const int32_t* dstart; // n or null: first point of each point's dense cell
     const uint32_t* perm;  // sorted position -> input index

@@ -297,7 +297,7 @@ size_t carve_plan(Plan& p, void* base, int64_t n, int dim, int algo, int lcap, b
     p.nfirst = c.take<int32_t>(mc);
     p.nsum = c.take<char>(box * (size_t)sum_levels_entries(mc));
     p.lsolid = c.take<uint8_t>(mc);
-    p.klist = c.take<int32_t>(mc);
+    p.klist = c.take<int32_t>(3 * mc);
     p.tstart = c.take<int32_t>(mc);
     p.tsib = c.take<int2>(mc * TRAVERSAL_SIBCAP);
     p.tnsib = c.take<int8_t>(mc);
@@ -474,27 +474,34 @@ dbscan_status build_index(Workspace* w, const Plan& p, StageTimer& T, const floa
                           float eps, int dense_mp, int algo, ClusterArgs& a, cudaStream_t s)
 {
     w->last_algo = algo == DBSCAN_ALGO_AUTO ? -2 : algo;  // -2: chosen on the device
-    TRY_CUDA(cudaMemsetAsync(p.ctrl + CTRL_LO, 0xff, MAX_DIM * sizeof(uint32_t), s));
-    TRY_CUDA(cudaMemsetAsync(p.ctrl + CTRL_HI, 0, MAX_DIM * sizeof(uint32_t), s));
-    TRY_CUDA(cudaMemsetAsync(p.ctrl + CTRL_M, 0, 2 * sizeof(uint32_t), s));
     launch_run_begin(p.ctrl, algo, s);
-    T.begin(ST_BOUNDS);
-    launch_bounds(points, n, dim, p.ctrl, s);
-    T.end();
-    TRY_CUDA(cudaGetLastError());
     const float e2 = eps * eps;
     const bool fd = algo != DBSCAN_ALGO_DENSEBOX, db = algo != DBSCAN_ALGO_FDBSCAN;
     const int idx_bits = index_bits(n);
     const int db_axis_bits = densebox_axis_bits(dim, idx_bits);
     const int db_key_bits = db_axis_bits * dim;
-    if (algo == DBSCAN_ALGO_AUTO) {
+    const int fd_key_bits = fdbscan_bits(dim) * dim;
+    // the bounds kernel clears the sort's scratch (histograms, counters and
+    // the status words of the widest key) and the dense-cell flags
+    BoundsExtra x;
+    const int sort_bits = fd && db ? (fd_key_bits > db_key_bits ? fd_key_bits : db_key_bits) : (fd ? fd_key_bits : db_key_bits);
+    x.zero[0] = reinterpret_cast<uint4*>(p.hist);
+    x.zero16[0] = (reinterpret_cast<char*>(p.status + sort_status_words(n, 8, sort_bits)) - reinterpret_cast<char*>(p.hist)) / 16;
+    if (db) {
+        x.zero[1] = reinterpret_cast<uint4*>(p.db.pdense);
+        x.zero16[1] = (n + 15) / 16;
         // the estimate's thresholds belong to the cells of Sec. 4.2 (f = 1)
-        launch_grid(p.ctrl, dim, eps, 1.0f, db_axis_bits, p.grid_est, s);
+        const double cell = (double)eps / std::sqrt((double)dim);
+        if (algo == DBSCAN_ALGO_AUTO) x.grid[x.grids++] = GridRequest{cell, db_axis_bits, p.grid_est};
+        x.grid[x.grids++] = GridRequest{(double)t_run.cell_factor * (double)eps / std::sqrt((double)dim), db_axis_bits, p.grid};
+    }
+    T.begin(ST_BOUNDS);
+    launch_bounds(points, n, dim, p.ctrl, x, s);
+    T.end();
+    TRY_CUDA(cudaGetLastError());
+    if (algo == DBSCAN_ALGO_AUTO)
         TRY_CUDA(launch_density_estimate(points, n, dim, p.grid_est, dense_mp, g_tuning.auto_fraction[dim],
                                          g_tuning.auto_occupancy[dim], p.est, p.ctrl, s));
-    }
-    // (after the estimate's grid: CTRL_KEYBITS is this grid's)
-    if (db) launch_grid(p.ctrl, dim, eps, t_run.cell_factor, db_axis_bits, p.grid, s);
 
     SortBuffers sb;
     sb.keys_alt = p.keys_alt;
@@ -504,6 +511,7 @@ dbscan_status build_index(Workspace* w, const Plan& p, StageTimer& T, const floa
     sb.counters = p.counters;
     sb.err = p.ctrl + CTRL_ABORT;  // a wait that runs out stops every later stage
     sb.ctl.abort = p.ctrl + CTRL_ABORT;
+    sb.cleared = true;
     sb.ctl.gate = p.ctrl + CTRL_ALGO;
     bool in_alt = false;
     const int64_t m_cap = leaf_cap(n, algo);

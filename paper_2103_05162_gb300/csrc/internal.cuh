@@ -643,6 +643,7 @@ struct SortBuffers {
     uint32_t* counters;    // SORT_MAX_PASSES
     uint32_t* err;         // device error word (ERR_SORT_TIMEOUT)
     SortCtl ctl;           // device-side control (pipeline sorts only)
+    bool cleared = false;  // hist, counters and status are zero already
 };
 // Test hooks of the look-back wait: the wait limit of every later sort
 // (spins; negative restores SPIN_LIMIT) and, if stall_first_tile, tile 0 of

@@ -339,10 +339,12 @@ cudaError_t sort_pairs(K* keys, uint32_t* vals, int64_t n, int shift0, int bits,
     const int passes = sort_passes(bits);
     const int64_t tiles = (n + TILE_ITEMS - 1) / TILE_ITEMS;
     cudaError_t e;
-    if ((e = cudaMemsetAsync(sb.hist, 0, sizeof(uint32_t) * RADIX * passes, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(sb.counters, 0, sizeof(uint32_t) * passes, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(sb.status, 0, sizeof(uint32_t) * RADIX * (size_t)tiles * passes, s)) != cudaSuccess)
-        return e;
+    if (!sb.cleared) {
+        if ((e = cudaMemsetAsync(sb.hist, 0, sizeof(uint32_t) * RADIX * passes, s)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(sb.counters, 0, sizeof(uint32_t) * passes, s)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(sb.status, 0, sizeof(uint32_t) * RADIX * (size_t)tiles * passes, s)) != cudaSuccess)
+            return e;
+    }
     K* k_alt = static_cast<K*>(sb.keys_alt);
     // once a wait has run out, no later pass may run: its input holds slots
     // the timed-out tiles never wrote, and ranks computed from them could

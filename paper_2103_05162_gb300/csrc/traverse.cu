@@ -409,12 +409,14 @@ struct DevArgs {
     const typename Traits<D>::Box* nodebox;
     const int2* leafr;
     uint8_t* lsolid;
-    int32_t* klist;
+    int32_t* klist;  // m_cap entries per leaf kind
+    int64_t m_cap;
     int32_t* labels;
     uint8_t* core;
     uint8_t* nbr;
     int32_t* nlist;
     int lcap;
+    bool whole_intra;  // k_intra also makes the lists' claims and groups the leaves by kind
     uint32_t* ctrl;
     float e2;
     int min_pts;
@@ -979,25 +981,36 @@ __global__ void __maxnreg__(traversal_regs<D>()) k_pre(const __grid_constant__ D
     }
 }
 
-// Border claims from preprocessing's lists (DBSCAN mode): a non-core point
-// holds all its neighbours outside its tile; it joins the cluster of the
-// first core one (Algorithm 3's claim of a border point, Sec. 3.2, made here
-// from the border's side). Neighbours inside the tile are k_intra's.
-__global__ void k_list_claims(const int32_t* __restrict__ nlist, int lcap, const uint8_t* __restrict__ nbr,
-                              const uint8_t* __restrict__ core, int32_t* labels, int64_t n)
+// A border claim from preprocessing's list (DBSCAN mode): a non-core point q
+// holds all its neighbours outside its tile; it joins the cluster of the first
+// core one (Algorithm 3's claim of a border point, Sec. 3.2, made here from the
+// border's side). Neighbours inside the tile are k_intra's, afterwards.
+__device__ __forceinline__ void list_claim(const int32_t* __restrict__ nlist, int lcap, const uint8_t* __restrict__ nbr,
+                                           const uint8_t* core, int32_t* labels, int64_t q)
 {
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
-        if (core[q]) continue;
-        const int k = nbr[q];
-        const int32_t* row = nlist + q * lcap;
-        for (int j = 0; j < k; ++j) {
-            const int y = row[j];
-            if (core[y]) {
-                uf_claim(labels, (int)q, y);
-                break;
-            }
+    const int k = nbr[q];
+    const int32_t* row = nlist + q * lcap;
+    for (int j = 0; j < k; ++j) {
+        const int y = row[j];
+        if (core[y]) {
+            uf_claim(labels, (int)q, y);
+            break;
         }
     }
+}
+
+// In small runs k_intra also makes the lists' claims and groups the leaves by
+// kind, which saves two launches of 5 us each. From SPLIT_INTRA points on both
+// are kernels of their own: a thread per point has more of the lists' scattered
+// reads in flight, and k_intra's warps take their leaves one by one, far apart,
+// instead of consecutive ones of alike cost (16.8M halos: 247 + 80 + 19 us
+// against 415; 512K road points: 36 against 30 + 10 + 11).
+constexpr int64_t SPLIT_INTRA = 1 << 22;
+__global__ void k_list_claims(const int32_t* __restrict__ nlist, int lcap, const uint8_t* __restrict__ nbr,
+                              const uint8_t* core, int32_t* labels, int64_t n)
+{
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
+        if (!core[q]) list_claim(nlist, lcap, nbr, core, labels, q);
 }
 
 // Each tile resolves its own pairs (q, q') with q' > q. Every lane builds the
@@ -1060,6 +1073,22 @@ __device__ __forceinline__ void link_next(const DevArgs<D>& a, const SoA<D>& soa
     }
 }
 
+// The lanes' leaves go to the lists of their kinds (0 a tile that is not solid,
+// 1 a solid tile, 2 a dense cell larger than a tile, -1 nothing to do), in lane
+// order, with one atomic per kind.
+__device__ __forceinline__ void append_kinds(uint32_t* ctrl, int32_t* klist, int64_t m_cap, int kind, int64_t L, int lane)
+{
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+        const unsigned b = __ballot_sync(FULL, kind == t);
+        if (!b) continue;
+        uint32_t at = 0;
+        if (lane == 0) at = atomicAdd(&ctrl[CTRL_KIND_COUNT + t], (uint32_t)__popc(b));
+        at = __shfl_sync(FULL, at, 0);
+        if (kind == t) klist[t * m_cap + at + __popc(b & ((1u << lane) - 1u))] = (int32_t)L;
+    }
+}
+
 template <int D>
 __global__ void __launch_bounds__(INTRA_THREADS) k_intra(DevArgs<D> a)
 {
@@ -1070,135 +1099,112 @@ __global__ void __launch_bounds__(INTRA_THREADS) k_intra(DevArgs<D> a)
     const int64_t m = a.ctrl[CTRL_M];
     const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t L = wid; L < m; L += nw) {
-        const int2 r = a.leafr[L];
-        if (r.y < 0) {
-            if (lane == 0) a.lsolid[L] = LEAF_SOLID;
-            const int n = (r.y & 0x7fffffff) - r.x;
-            soa.put(lane, a.sp[r.x + (int)((int64_t)n * lane / 32)]);
-            __syncwarp();
-            link_next<D>(a, soa, L, m, tile_params(a, (int)L), 32, FULL, r.x, 0, lane);
-            __syncwarp();
-            continue;
-        }
-        const int s = r.x, k = r.y - r.x;
-        const TileParams tp = tile_params(a, (int)L);
-        const bool valid = lane < k;
-        bool c = valid && a.core[s + lane];
-        if (tp.min_pts > 2 && !__any_sync(FULL, c)) {
-            // core flags known and none in the tile: no pair inside it
-            // unites or claims anything; the main phase needs the tile only
-            // where it claims border points
-            if (lane == 0) a.lsolid[L] = a.lcap > 0 || a.mode != DBSCAN_MODE_DBSCAN ? LEAF_IDLE : LEAF_MIXED;
-            continue;
-        }
-        const P p = a.sp[valid ? s + lane : s];
-        // the tile's adjacency, two points at a time (packed)
-        soa.put(lane, p);
-        __syncwarp();
-        unsigned adj = 0;
-        if (valid) {
-            const typename NB<D>::PP pp = NB<D>::pack(p);
-            int j = 0;
-            for (; j + 1 < k; j += 2) {
-                float d0, d1;
-                soa.d2pair(pp, j, d0, d1);
-                adj |= (d0 <= tp.e2 ? 1u : 0u) << j;
-                adj |= (d1 <= tp.e2 ? 2u : 0u) << j;
+    // up to 16 consecutive leaves per warp and round: their kinds go to the
+    // main phase's lists with one atomic per kind
+    const int64_t per = a.whole_intra ? max((int64_t)1, min((int64_t)16, (m + nw - 1) / nw)) : 1;
+    for (int64_t L0 = wid * per; L0 < m; L0 += nw * per) {
+        int kinds = -1;  // lane j: the kind of leaf L0 + j
+        for (int j = 0; j < per && L0 + j < m; ++j) {
+            const int64_t L = L0 + j;
+            const int2 r = a.leafr[L];
+            if (r.y < 0) {
+                if (lane == j) kinds = 2;
+                if (lane == 0) a.lsolid[L] = LEAF_SOLID;
+                const int n = (r.y & 0x7fffffff) - r.x;
+                soa.put(lane, a.sp[r.x + (int)((int64_t)n * lane / 32)]);
+                __syncwarp();
+                link_next<D>(a, soa, L, m, tile_params(a, (int)L), 32, FULL, r.x, 0, lane);
+                __syncwarp();
+                continue;
             }
-            if (j < k && soa.d2(p, j) <= tp.e2) adj |= 1u << j;
-            adj &= ~(1u << lane);
+            const int s = r.x, k = r.y - r.x;
+            const TileParams tp = tile_params(a, (int)L);
+            const bool valid = lane < k;
+            bool c = valid && a.core[s + lane];
+            if (a.whole_intra && a.lcap > 0 && tp.min_pts > 2 && valid && !c)
+                list_claim(a.nlist, a.lcap, a.nbr, a.core, a.labels, s + lane);
+            if (tp.min_pts > 2 && !__any_sync(FULL, c)) {
+                // core flags known and none in the tile: no pair inside it
+                // unites or claims anything; the main phase needs the tile only
+                // where it claims border points
+                const bool idle = a.lcap > 0 || a.mode != DBSCAN_MODE_DBSCAN;
+                if (lane == 0) a.lsolid[L] = idle ? LEAF_IDLE : LEAF_MIXED;
+                if (lane == j) kinds = idle ? -1 : 0;
+                continue;
+            }
+            const P p = a.sp[valid ? s + lane : s];
+            // the tile's adjacency, two points at a time (packed)
+            soa.put(lane, p);
+            __syncwarp();
+            unsigned adj = 0;
+            if (valid) {
+                const typename NB<D>::PP pp = NB<D>::pack(p);
+                int j = 0;
+                for (; j + 1 < k; j += 2) {
+                    float d0, d1;
+                    soa.d2pair(pp, j, d0, d1);
+                    adj |= (d0 <= tp.e2 ? 1u : 0u) << j;
+                    adj |= (d1 <= tp.e2 ? 2u : 0u) << j;
+                }
+                if (j < k && soa.d2(p, j) <= tp.e2) adj |= 1u << j;
+                adj &= ~(1u << lane);
+            }
+            __syncwarp();
+            if (tp.min_pts == 2) {
+                // no preprocessing: a neighbour inside the tile makes a point core
+                // (neighbours in other tiles are found by the main phase)
+                c = valid && (c || adj != 0);
+                if (c) a.core[s + lane] = 1;
+            }
+            const unsigned cm = __ballot_sync(FULL, c);
+            if (tp.min_pts > 2 && a.mode == DBSCAN_MODE_DBSCAN && valid && !c && (adj & cm))
+                uf_claim(a.labels, s + lane, s + __ffs(adj & cm) - 1);
+            // the components, each grown from its first point by one reduction
+            // over the lanes already in it per step
+            const unsigned near = c ? adj & cm : 0u;
+            unsigned reach = 1u << lane;
+            unsigned left = __ballot_sync(FULL, near != 0);
+            const bool pairs = left != 0;
+            while (left) {
+                unsigned grown = left & (0u - left), set;
+                do {
+                    set = grown;
+                    grown |= __reduce_or_sync(FULL, ((set >> lane) & 1u) ? near : 0u);
+                } while (grown != set);
+                if ((set >> lane) & 1u) reach = set;
+                left &= ~set;
+            }
+            if (c) {
+                const int lr = __ffs(reach) - 1;
+                if (lr != lane) uf_union(a.labels, s + lane, s + lr);
+            }
+            __syncwarp();
+            const int root = c ? uf_find(a.labels, s + lane) : -1;
+            const int root0 = __shfl_sync(FULL, root, 0);
+            const bool solid = __all_sync(FULL, !valid || (c && root == root0));
+            if (lane == 0) a.lsolid[L] = solid ? LEAF_SOLID : LEAF_MIXED;
+            if (lane == j) kinds = solid ? 1 : 0;
+            if (pairs) link_next<D>(a, soa, L, m, tp, k, tp.min_pts <= 2 ? tile_lanes(k) : cm, s, 1, lane);
+            __syncwarp();
         }
-        __syncwarp();
-        if (tp.min_pts == 2) {
-            // no preprocessing: a neighbour inside the tile makes a point core
-            // (neighbours in other tiles are found by the main phase)
-            c = valid && (c || adj != 0);
-            if (c) a.core[s + lane] = 1;
-        }
-        const unsigned cm = __ballot_sync(FULL, c);
-        if (tp.min_pts > 2 && a.mode == DBSCAN_MODE_DBSCAN && valid && !c && (adj & cm))
-            uf_claim(a.labels, s + lane, s + __ffs(adj & cm) - 1);
-        // the components, each grown from its first point by one reduction
-        // over the lanes already in it per step
-        const unsigned near = c ? adj & cm : 0u;
-        unsigned reach = 1u << lane;
-        unsigned left = __ballot_sync(FULL, near != 0);
-        const bool pairs = left != 0;
-        while (left) {
-            unsigned grown = left & (0u - left), set;
-            do {
-                set = grown;
-                grown |= __reduce_or_sync(FULL, ((set >> lane) & 1u) ? near : 0u);
-            } while (grown != set);
-            if ((set >> lane) & 1u) reach = set;
-            left &= ~set;
-        }
-        if (c) {
-            const int lr = __ffs(reach) - 1;
-            if (lr != lane) uf_union(a.labels, s + lane, s + lr);
-        }
-        __syncwarp();
-        const int root = c ? uf_find(a.labels, s + lane) : -1;
-        const int root0 = __shfl_sync(FULL, root, 0);
-        const bool solid = __all_sync(FULL, !valid || (c && root == root0));
-        if (lane == 0) a.lsolid[L] = solid ? LEAF_SOLID : LEAF_MIXED;
-        if (pairs) link_next<D>(a, soa, L, m, tp, k, tp.min_pts <= 2 ? tile_lanes(k) : cm, s, 1, lane);
-        __syncwarp();
+        if (a.whole_intra) append_kinds(a.ctrl, a.klist, a.m_cap, kinds, L0 + lane, lane);
     }
 }
 
-// Leaf kinds for the main phase: 0 a tile that is not solid, 1 a solid tile,
-// 2 a dense cell larger than a tile, -1 a tile with nothing to do. Lists are
-// grouped by kind; within a warp (32 consecutive leaves) the order is kept.
-__device__ __forceinline__ int leaf_kind(const int2* leafr, const uint8_t* lsolid, int64_t L)
-{
-    if (leafr[L].y < 0) return 2;
-    const uint8_t f = lsolid[L];
-    return f == LEAF_IDLE ? -1 : (f == LEAF_SOLID ? 1 : 0);
-}
-
-// (the links between consecutive leaves leave chains of sets as long as a
-// stretch of the curve; every leaf's thread shortens its own here, all of
-// them at once, so that the chains shrink by doubling)
-__global__ void k_kinds_count(const int2* __restrict__ leafr, const uint8_t* __restrict__ lsolid, uint32_t* ctrl,
-                              int32_t* labels)
+__global__ void k_kinds(const int2* __restrict__ leafr, const uint8_t* __restrict__ lsolid, uint32_t* ctrl,
+                        int32_t* __restrict__ klist, int64_t m_cap)
 {
     const int lane = threadIdx.x & 31;
     const int64_t m = ctrl[CTRL_M];
     for (int64_t base = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; base < m;
          base += (int64_t)gridDim.x * blockDim.x) {
         const int64_t L = base + lane;
-        const int kind = L < m ? leaf_kind(leafr, lsolid, L) : -1;
-#pragma unroll
-        for (int t = 0; t < 3; ++t) {
-            const unsigned b = __ballot_sync(FULL, kind == t);
-            if (lane == 0 && b) atomicAdd(&ctrl[CTRL_KIND_COUNT + t], (uint32_t)__popc(b));
+        int kind = -1;
+        if (L < m) {
+            const uint8_t f = lsolid[L];
+            kind = leafr[L].y < 0 ? 2 : (f == LEAF_IDLE ? -1 : (f == LEAF_SOLID ? 1 : 0));
         }
-        if (kind > 0) uf_find(labels, leafr[L].x);
-    }
-}
-
-__global__ void k_kinds_write(const int2* __restrict__ leafr, const uint8_t* __restrict__ lsolid, uint32_t* ctrl,
-                              int32_t* __restrict__ klist)
-{
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    const int64_t m = ctrl[CTRL_M];
-    const uint32_t off[3] = {0u, ctrl[CTRL_KIND_COUNT], ctrl[CTRL_KIND_COUNT] + ctrl[CTRL_KIND_COUNT + 1]};
-    for (int64_t base = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; base < m;
-         base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t L = base + lane;
-        const int kind = L < m ? leaf_kind(leafr, lsolid, L) : -1;
-#pragma unroll
-        for (int t = 0; t < 3; ++t) {
-            const unsigned b = __ballot_sync(FULL, kind == t);
-            if (!b) continue;
-            uint32_t at = 0;
-            if (lane == 0) at = atomicAdd(&ctrl[CTRL_KIND_FILL + t], (uint32_t)__popc(b));
-            at = __shfl_sync(FULL, at, 0);
-            if (kind == t) klist[off[t] + at + __popc(b & lt)] = (int32_t)L;
-        }
+        append_kinds(ctrl, klist, m_cap, kind, L, lane);
     }
 }
 
@@ -1709,10 +1715,10 @@ __global__ void __maxnreg__(main_regs<D>()) k_main(const __grid_constant__ DevAr
     // together with the leaf's own points.
     int L;
     auto resolve = [&](int64_t idx) {
-        // the list holds kind 0, then 1, then 2; taken as 2, 1, 0
+        // (a list per kind, taken as 2, 1, 0)
         if (idx >= total) L = -1;
-        else if (idx < c2) L = __ldg(&a.klist[c0 + c1 + idx]);
-        else L = __ldg(&a.klist[idx < c2 + c1 ? c0 + (idx - c2) : idx - c2 - c1]);
+        else if (idx < c2) L = __ldg(&a.klist[2 * a.m_cap + idx]);
+        else L = __ldg(&a.klist[idx < c2 + c1 ? a.m_cap + (idx - c2) : idx - c2 - c1]);
     };
     int pend = 0;
     if (lane == 0) pend = (int)atomicAdd(&a.ctrl[CTRL_KIND_WORK], 1u);
@@ -1770,13 +1776,22 @@ __global__ void __maxnreg__(main_regs<D>()) k_main(const __grid_constant__ DevAr
     }
 }
 
-// The same for one minPts of a multi-minPts run, with core flags from the
+// the work counters of the phases that follow
+__device__ __forceinline__ void clear_work(uint32_t* ctrl)
+{
+    if (blockIdx.x == 0 && threadIdx.x < CTRL_WORK_END - CTRL_WORK_PRE) ctrl[CTRL_WORK_PRE + threadIdx.x] = 0u;
+}
+constexpr int32_t CANON_NONE = 0x7f7f7f7f;  // above every index
+
+// k_init for one minPts of a multi-minPts run, with core flags from the
 // neighbour counts (capped at the largest minPts, which decides every smaller
 // one); points of dense cells are core for every minPts of the run.
 __global__ void k_init_from_counts(const uint8_t* __restrict__ pdense, const int32_t* __restrict__ dstart,
                                    const int32_t* __restrict__ ncount, int64_t n, int min_pts,
-                                   int32_t* __restrict__ labels, uint8_t* __restrict__ core)
+                                   int32_t* __restrict__ labels, uint8_t* __restrict__ core,
+                                   int32_t* __restrict__ canon, uint32_t* __restrict__ ctrl)
 {
+    clear_work(ctrl);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         if (pdense && pdense[i]) {
             labels[i] = dstart[i];
@@ -1785,6 +1800,7 @@ __global__ void k_init_from_counts(const uint8_t* __restrict__ pdense, const int
             labels[i] = (int32_t)i;
             core[i] = (min_pts <= 1 || ncount[i] >= min_pts) ? 1 : 0;
         }
+        canon[i] = CANON_NONE;
     }
 }
 
@@ -1802,10 +1818,13 @@ __global__ void k_core_from_input(const uint32_t* __restrict__ perm, const uint8
 }
 
 // labels[i] = i, or the first point of its dense cell (pre-united, Sec. 4.2);
-// core = 1 in dense cells (and everywhere when minPts == 1)
+// core = 1 in dense cells (and everywhere when minPts == 1); no list entries,
+// no smallest index, the phases' work counters at 0
 __global__ void k_init(const uint8_t* __restrict__ pdense, const int32_t* __restrict__ dstart, int64_t n,
-                       int min_pts, int32_t* __restrict__ labels, uint8_t* __restrict__ core)
+                       int min_pts, int32_t* __restrict__ labels, uint8_t* __restrict__ core,
+                       uint8_t* __restrict__ nbr, int32_t* __restrict__ canon, uint32_t* __restrict__ ctrl)
 {
+    clear_work(ctrl);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         if (pdense && pdense[i]) {
             labels[i] = dstart[i];
@@ -1814,6 +1833,8 @@ __global__ void k_init(const uint8_t* __restrict__ pdense, const int32_t* __rest
             labels[i] = (int32_t)i;
             core[i] = min_pts == 1 ? 1 : 0;
         }
+        nbr[i] = 0;
+        canon[i] = CANON_NONE;
     }
 }
 
@@ -1893,9 +1914,11 @@ DevArgs<D> dev_args(const ClusterArgs& a)
     d.leafr = a.leafr;
     d.lsolid = a.lsolid;
     d.klist = a.klist;
+    d.m_cap = a.m_cap;
     d.nbr = a.nbr;
     d.nlist = a.nlist;
     d.lcap = a.lcap;
+    d.whole_intra = a.n < SPLIT_INTRA;
     d.labels = a.labels;
     d.core = a.core;
     d.ctrl = a.ctrl;
@@ -1938,13 +1961,20 @@ void run_main_walk(const ClusterArgs& a, cudaStream_t s)
 template <int D>
 void run_main(const ClusterArgs& a, cudaStream_t s)
 {
+    const bool split = a.n >= SPLIT_INTRA;
+    if (split && a.lcap > 0) {
+        k_list_claims<<<152 * 16, 256, 0, s>>>(a.nlist, a.lcap, a.nbr, a.core, a.labels, a.n);
+        note_launches(1);
+    }
     int64_t gw = (a.m_cap * 32 + INTRA_THREADS - 1) / INTRA_THREADS;
     if (gw > 152 * 16) gw = 152 * 16;
     k_intra<D><<<(unsigned)gw, INTRA_THREADS, 0, s>>>(dev_args<D>(a));
-    int64_t gk = (a.m_cap + 255) / 256;
-    if (gk > 152 * 8) gk = 152 * 8;
-    k_kinds_count<<<(unsigned)gk, 256, 0, s>>>(a.leafr, a.lsolid, a.ctrl, a.labels);
-    k_kinds_write<<<(unsigned)gk, 256, 0, s>>>(a.leafr, a.lsolid, a.ctrl, a.klist);
+    if (split) {
+        int64_t gk = (a.m_cap + 255) / 256;
+        if (gk > 152 * 8) gk = 152 * 8;
+        k_kinds<<<(unsigned)gk, 256, 0, s>>>(a.leafr, a.lsolid, a.ctrl, a.klist, a.m_cap);
+        note_launches(1);
+    }
     run_main_walk<D>(a, s);
 }
 
@@ -1952,33 +1982,20 @@ void run_main(const ClusterArgs& a, cudaStream_t s)
 
 cudaError_t launch_cluster_init(const ClusterArgs& a, cudaStream_t s)
 {
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(a.ctrl + CTRL_WORK_PRE, 0, (CTRL_WORK_END - CTRL_WORK_PRE) * sizeof(uint32_t), s)) !=
-        cudaSuccess)
-        return e;
     int64_t gn = (a.n + 255) / 256;
     if (gn > 152 * 16) gn = 152 * 16;
-    k_init<<<(unsigned)gn, 256, 0, s>>>(a.pdense, a.dstart, a.n, a.min_pts, a.labels, a.core);
+    k_init<<<(unsigned)gn, 256, 0, s>>>(a.pdense, a.dstart, a.n, a.min_pts, a.labels, a.core, a.nbr, a.canon, a.ctrl);
     note_launches(1);
-    if ((e = cudaMemsetAsync(a.canon, 0x7f, sizeof(int32_t) * (size_t)a.n, s)) != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
 cudaError_t launch_cluster_from_counts(const ClusterArgs& a, int min_pts, cudaStream_t s)
 {
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(a.ctrl + CTRL_WORK_PRE, 0, (CTRL_WORK_END - CTRL_WORK_PRE) * sizeof(uint32_t), s)) !=
-        cudaSuccess)
-        return e;
     int64_t gn = (a.n + 255) / 256;
     if (gn > 152 * 16) gn = 152 * 16;
-    k_init_from_counts<<<(unsigned)gn, 256, 0, s>>>(a.pdense, a.dstart, a.ncount, a.n, min_pts, a.labels, a.core);
+    k_init_from_counts<<<(unsigned)gn, 256, 0, s>>>(a.pdense, a.dstart, a.ncount, a.n, min_pts, a.labels, a.core,
+                                                    a.canon, a.ctrl);
     note_launches(1);
-    if ((e = cudaMemsetAsync(a.canon, 0x7f, sizeof(int32_t) * (size_t)a.n, s)) != cudaSuccess) return e;
-    if (a.lcap > 0 && a.mode == DBSCAN_MODE_DBSCAN) {
-        k_list_claims<<<(unsigned)gn, 256, 0, s>>>(a.nlist, a.lcap, a.nbr, a.core, a.labels, a.n);
-        note_launches(1);
-    }
     return cudaGetLastError();
 }
 
@@ -2000,19 +2017,10 @@ cudaError_t launch_cluster_pre(const ClusterArgs& a, cudaStream_t s)
     // are always taken)
     if (a.min_pts <= 2 && !a.ncount) return cudaSuccess;
     count_phase(1, s);
-    cudaError_t e;
-    // points that keep no list (instances of a batch with minPts <= 2) read 0
-    if (a.lcap > 0 && (e = cudaMemsetAsync(a.nbr, 0, (size_t)a.n, s)) != cudaSuccess) return e;
 #define PRE_RUN(D) run_pre<D>(a, s)
     GBD_DIM_SWITCH(a.dim, PRE_RUN)
 #undef PRE_RUN
     note_launches(1);
-    if (a.lcap > 0 && !a.ncount) {  // (several minPts: claims per minPts)
-        int64_t gn = (a.n + 255) / 256;
-        if (gn > 152 * 16) gn = 152 * 16;
-        k_list_claims<<<(unsigned)gn, 256, 0, s>>>(a.nlist, a.lcap, a.nbr, a.core, a.labels, a.n);
-        note_launches(1);
-    }
     return cudaGetLastError();
 }
 
@@ -2022,7 +2030,7 @@ cudaError_t launch_cluster_main(const ClusterArgs& a, cudaStream_t s)
 #define MAIN_RUN(D) run_main<D>(a, s)
     GBD_DIM_SWITCH(a.dim, MAIN_RUN)
 #undef MAIN_RUN
-    note_launches(4);
+    note_launches(2);
     return cudaGetLastError();
 }
 
