@@ -60,6 +60,7 @@ __global__ void k_bbounds(const int64_t* __restrict__ offs,
                           const InstDev* __restrict__ inst, int count, int64_t n, uint32_t* __restrict__ bounds,
                           uint32_t* __restrict__ nonfinite)
 {
+    stage_begin(offs, inst);
     const int lane = threadIdx.x & 31;
     for (int64_t base = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; base < n;
          base += (int64_t)gridDim.x * blockDim.x) {
@@ -102,6 +103,7 @@ __global__ void k_bkeys(const int64_t* __restrict__ offs,
                         const InstDev* __restrict__ inst, int count, int64_t n, int lb, uint64_t* __restrict__ keys,
                         uint32_t* __restrict__ vals)
 {
+    stage_begin(offs, inst);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int b = find_inst(offs, count, i);
         const InstDev in = inst[b];
@@ -119,6 +121,7 @@ __global__ void k_bgather(const int64_t* __restrict__ offs,
                           const InstDev* __restrict__ inst, int count, const uint32_t* __restrict__ perm, int64_t n,
                           float4* __restrict__ sp, const uint32_t* __restrict__ ctrl)
 {
+    stage_begin(offs, inst, perm, ctrl);
     if (!stage_on(ctrl, -1)) return;  // a sort that gave up: stale permutation words
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t row = perm[i];
@@ -131,6 +134,7 @@ __global__ void k_bgather(const int64_t* __restrict__ offs,
 __global__ void k_inst_roots(const int2* __restrict__ range, const int32_t* __restrict__ linst,
                              const uint32_t* __restrict__ ctrl, int32_t* __restrict__ iroot)
 {
+    stage_begin(range, linst, ctrl);
     const int64_t m = ctrl[CTRL_M];
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < 2 * m - 1;
          x += (int64_t)gridDim.x * blockDim.x) {
@@ -151,6 +155,7 @@ __global__ void k_binit(const uint64_t* __restrict__ keys, int lb, const InstDev
                         const uint8_t* __restrict__ pdense, const int32_t* __restrict__ dstart, int64_t n,
                         int32_t* __restrict__ labels, uint8_t* __restrict__ core, const uint32_t* __restrict__ ctrl)
 {
+    stage_begin(keys, inst, pdense, dstart, ctrl);
     if (!stage_on(ctrl, -1)) return;  // a sort that gave up: stale keys would index past the instances
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         if (pdense && pdense[i]) {
@@ -169,6 +174,7 @@ __global__ void k_bfinalize(int32_t* labels, const uint8_t* __restrict__ core, c
                             const uint64_t* __restrict__ keys, int lb, const InstDev* __restrict__ inst, int64_t n,
                             int32_t* __restrict__ canon, const uint32_t* __restrict__ ctrl)
 {
+    stage_begin(core, perm, keys, inst, ctrl);
     if (!stage_on(ctrl, -1)) return;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
@@ -185,6 +191,7 @@ __global__ void k_brelabel(const int32_t* labels, const uint8_t* __restrict__ co
                            const uint64_t* __restrict__ keys, int lb, const InstDev* __restrict__ inst, int64_t n,
                            int mode, const int32_t* __restrict__ canon, const uint32_t* __restrict__ ctrl)
 {
+    stage_begin(labels, core, perm, keys, inst, canon, ctrl);
     if (!stage_on(ctrl, -1)) return;  // aborted batch: nothing is written
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const bool c = core[i] != 0;
@@ -354,7 +361,7 @@ cudaError_t enqueue_batch_stages(const BatchPlan& p, int64_t n, int count, int m
 {
     cudaError_t e;
     if ((e = cudaMemsetAsync(p.ctrl + CTRL_M, 0, 2 * sizeof(uint32_t), s)) != cudaSuccess) return e;
-    k_bkeys<<<grid_n(n), 256, 0, s>>>(p.offs, p.inst, count, n, lb, p.keys, p.vals);
+    launch(k_bkeys, grid_n(n), 256, 0, s, p.offs, p.inst, count, n, lb, p.keys, p.vals);
     note_launches(1);
     SortBuffers sb;
     sb.keys_alt = p.keys_alt;
@@ -368,7 +375,7 @@ cudaError_t enqueue_batch_stages(const BatchPlan& p, int64_t n, int count, int m
     if ((e = sort_pairs_u64(p.keys, p.vals, n, key_bits, sb, s, &in_alt)) != cudaSuccess) return e;
     const uint64_t* keys = in_alt ? p.keys_alt : p.keys;
     const uint32_t* perm = in_alt ? p.vals_alt : p.vals;
-    k_bgather<<<grid_n(n), 256, 0, s>>>(p.offs, p.inst, count, perm, n, p.sp, p.ctrl);
+    launch(k_bgather, grid_n(n), 256, 0, s, p.offs, p.inst, count, perm, n, p.sp, p.ctrl);
     note_launches(1);
     if (algo == DBSCAN_ALGO_DENSEBOX) {
         if ((e = cudaMemsetAsync(p.db.pdense, 0, (size_t)n, s)) != cudaSuccess) return e;
@@ -377,7 +384,7 @@ cudaError_t enqueue_batch_stages(const BatchPlan& p, int64_t n, int count, int m
     if ((e = launch_batch_leaves(keys, n, lb, p.db, p.leafr, p.lkey, p.linst, p.ctrl, s)) != cudaSuccess) return e;
     launch_lbvh(p.sp, 3, p.leafr, p.lkey, p.db.dbox, n, p.ctrl, p.nmeta, p.parent, p.nfirst, p.nodebox, p.nsum, p.nodes, s,
                 p.range);
-    k_inst_roots<<<grid_n(2 * n), 256, 0, s>>>(p.range, p.linst, p.ctrl, p.iroot);
+    launch(k_inst_roots, grid_n(2 * n), 256, 0, s, p.range, p.linst, p.ctrl, p.iroot);
     note_launches(1);
     // union-find init (per point instance parameters)
     if ((e = cudaMemsetAsync(p.ctrl + CTRL_WORK_PRE, 0, (CTRL_WORK_END - CTRL_WORK_PRE) * sizeof(uint32_t), s)) !=
@@ -385,7 +392,7 @@ cudaError_t enqueue_batch_stages(const BatchPlan& p, int64_t n, int count, int m
         return e;
     // points that keep no list (instances with minPts <= 2) read 0
     if ((e = cudaMemsetAsync(p.nbr, 0, (size_t)n, s)) != cudaSuccess) return e;
-    k_binit<<<grid_n(n), 256, 0, s>>>(keys, lb, p.inst, p.db.pdense, p.db.dstart, n, p.labels, p.core, p.ctrl);
+    launch(k_binit, grid_n(n), 256, 0, s, keys, lb, p.inst, p.db.pdense, p.db.dstart, n, p.labels, p.core, p.ctrl);
     note_launches(1);
     if ((e = cudaMemsetAsync(p.canon, 0x7f, sizeof(int32_t) * (size_t)n, s)) != cudaSuccess) return e;
     ClusterArgs a;
@@ -426,8 +433,8 @@ cudaError_t enqueue_batch_stages(const BatchPlan& p, int64_t n, int count, int m
     if ((e = launch_cluster_starts(a, s)) != cudaSuccess) return e;
     if ((e = launch_cluster_pre(a, s)) != cudaSuccess) return e;
     if ((e = launch_cluster_main(a, s)) != cudaSuccess) return e;
-    k_bfinalize<<<grid_n(n), 256, 0, s>>>(p.labels, p.core, perm, keys, lb, p.inst, n, p.canon, p.ctrl);
-    k_brelabel<<<grid_n(n), 256, 0, s>>>(p.labels, p.core, perm, keys, lb, p.inst, n, mode, p.canon, p.ctrl);
+    launch(k_bfinalize, grid_n(n), 256, 0, s, p.labels, p.core, perm, keys, lb, p.inst, n, p.canon, p.ctrl);
+    launch(k_brelabel, grid_n(n), 256, 0, s, p.labels, p.core, perm, keys, lb, p.inst, n, mode, p.canon, p.ctrl);
     note_launches(2);
     return cudaGetLastError();
 }
@@ -443,6 +450,7 @@ dbscan_status run_batch(Workspace* w, int32_t count, const int64_t* offsets, con
         return set_error(DBSCAN_ERR_INVALID_ARG, "batches take an explicit algorithm (FDBSCAN or DENSEBOX)");
     const int64_t n = offsets[count];
     if (n == 0) return DBSCAN_OK;
+    t_overlap = n <= OVERLAP_POINTS;
     int max_mp = 1;
     for (int b = 0; b < count; ++b)
         if (min_pts[b] > max_mp) max_mp = min_pts[b];
@@ -485,7 +493,7 @@ dbscan_status run_batch(Workspace* w, int32_t count, const int64_t* offsets, con
     BTRY(cudaMemcpyAsync(p.bounds, hb.data(), sizeof(uint32_t) * hb.size(), cudaMemcpyHostToDevice, s));
     // fold the last run's abort bits into the error word and clear them
     launch_run_begin(p.ctrl, algo, s);
-    k_bbounds<<<grid_n(n), 256, 0, s>>>(p.offs, p.inst, count, n, p.bounds, p.bounds + 6 * (size_t)count);
+    launch(k_bbounds, grid_n(n), 256, 0, s, p.offs, p.inst, count, n, p.bounds, p.bounds + 6 * (size_t)count);
     note_launches(1);
     uint32_t err = 0;
     BTRY(cudaMemcpyAsync(hb.data(), p.bounds, sizeof(uint32_t) * hb.size(), cudaMemcpyDeviceToHost, s));

@@ -58,6 +58,7 @@ template <int D, int BT = bounds_threads<D>()>
 __global__ void __launch_bounds__(BT) k_bounds(const float* __restrict__ pts, int64_t n,
                                                uint32_t* __restrict__ ctrl, BoundsExtra x)
 {
+    stage_begin(pts);
     __shared__ uint32_t s_lo[D], s_hi[D];
     __shared__ int s_bad, s_last;
     if (threadIdx.x < D) { s_lo[threadIdx.x] = 0xffffffffu; s_hi[threadIdx.x] = 0u; }
@@ -103,6 +104,7 @@ __global__ void __launch_bounds__(BT) k_bounds(const float* __restrict__ pts, in
 // the run's first kernel (see launch_run_begin)
 __global__ void k_run_begin(uint32_t* ctrl, int algo)
 {
+    stage_begin();
     const int t = threadIdx.x;
     if (t == 0) {
         const uint32_t a = ctrl[CTRL_ABORT];
@@ -128,6 +130,7 @@ template <int D>
 __global__ void k_morton32(const float* __restrict__ pts, int64_t n, const uint32_t* __restrict__ ctrl, int bits,
                            uint32_t* __restrict__ keys, uint32_t* __restrict__ vals)
 {
+    stage_begin(pts, ctrl);
     if (!stage_on(ctrl, DBSCAN_ALGO_FDBSCAN)) return;
     float lo[D], scale[D];
     const float cells = (float)(1u << bits);
@@ -154,6 +157,7 @@ template <int D>
 __global__ void k_morton64(const float* __restrict__ pts, int64_t n, const uint32_t* __restrict__ ctrl, int bits,
                            uint64_t* __restrict__ keys, uint32_t* __restrict__ vals)
 {
+    stage_begin(pts, ctrl);
     if (!stage_on(ctrl, DBSCAN_ALGO_FDBSCAN)) return;
     float lo[D], scale[D];
     const float cells = (float)(1u << bits);
@@ -203,6 +207,7 @@ __global__ void k_cellkey_packed(const float* __restrict__ pts, int64_t n, const
                                  const uint32_t* __restrict__ ctrl, int idx_bits, int host_passes,
                                  uint64_t* __restrict__ words0, uint64_t* __restrict__ words1)
 {
+    stage_begin(pts, gp, ctrl);
     if (!stage_on(ctrl, DBSCAN_ALGO_DENSEBOX)) return;
     const GridParams g = *gp;
     // (host_passes 0: no sort runs, n <= 1, and the words stay in words0)
@@ -235,6 +240,7 @@ __global__ void k_est_insert(const float* __restrict__ pts, int64_t n, int s, co
                              const uint32_t* __restrict__ ctrl, unsigned long long* __restrict__ table,
                              int32_t* __restrict__ slot)
 {
+    stage_begin(pts, gp, ctrl);
     if (!stage_on(ctrl, -1)) return;
     const GridParams g = *gp;
     for (int j = threadIdx.x; j < s; j += blockDim.x) {
@@ -258,6 +264,7 @@ __global__ void k_est_count(const float* __restrict__ pts, int64_t n, int64_t st
                             const GridParams* __restrict__ gp, const uint32_t* __restrict__ ctrl,
                             const unsigned long long* __restrict__ table, uint32_t* __restrict__ counts)
 {
+    stage_begin(pts, gp, ctrl, table);
     if (!stage_on(ctrl, -1)) return;
     const GridParams g = *gp;
     __shared__ uint32_t sc[EST_SLOTS];
@@ -291,6 +298,7 @@ __global__ void k_est_result(const int32_t* __restrict__ slot, int s, const uint
                              int64_t n, int64_t stride, int min_pts, float auto_fraction, float auto_occupancy,
                              uint32_t* __restrict__ out, uint32_t* __restrict__ ctrl)
 {
+    stage_begin(slot, counts);
     if (!stage_on(ctrl, -1)) return;
     uint32_t c = 0;
     unsigned long long occ = 0;
@@ -326,6 +334,7 @@ __global__ void k_est_result(const int32_t* __restrict__ slot, int s, const uint
 template <int D>
 __global__ void k_morton_generic(const float* __restrict__ pts, int64_t n, GridParams g, uint64_t* __restrict__ out)
 {
+    stage_begin(pts);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         uint32_t c[D];
 #pragma unroll
@@ -347,6 +356,7 @@ template <int D>
 __global__ void k_gather(const float* __restrict__ pts, const uint32_t* __restrict__ perm, int64_t n,
                          typename Traits<D>::Point* __restrict__ sp, const uint32_t* __restrict__ ctrl, int algo)
 {
+    stage_begin(pts, perm, ctrl);
     // a sort that gave up leaves stale words in perm: never index with them
     if (!stage_on(ctrl, algo)) return;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -392,6 +402,7 @@ __global__ void k_gather_packed(const float* __restrict__ pts, const uint64_t* _
                                 uint32_t* __restrict__ perm, uint64_t* __restrict__ keys,
                                 const uint32_t* __restrict__ ctrl)
 {
+    stage_begin(pts, words, ctrl);
     using P = typename Traits<D>::Point;
     if (!stage_on(ctrl, DBSCAN_ALGO_DENSEBOX)) return;  // (a sort that gave up: stale index bits)
     const uint64_t mask = (1ull << idx_bits) - 1ull;
@@ -464,6 +475,7 @@ __global__ void __launch_bounds__(CELL_THREADS)
                      uint8_t* __restrict__ pdense, int32_t* __restrict__ dstart,
                      typename Traits<D>::Box* __restrict__ dbox, uint32_t* __restrict__ ctrl, int algo, int steps)
 {
+    stage_begin(keys, sp, mps, e2s);
     using T = Traits<D>;
     using Box = typename T::Box;
     if (!stage_on(ctrl, algo)) return;
@@ -682,6 +694,7 @@ __global__ void __launch_bounds__(LF_THREADS)
                  int64_t n, int windows, int id_shift, uint32_t* __restrict__ words, uint32_t* __restrict__ counts,
                  const uint32_t* __restrict__ ctrl, int algo)
 {
+    stage_begin(keys, dstart, pdense, ctrl);
     if (!stage_on(ctrl, algo)) return;
     const int lane = threadIdx.x & 31;
     const int warp = blockIdx.x * LF_WARPS + (threadIdx.x >> 5);
@@ -760,6 +773,7 @@ __global__ void __launch_bounds__(LF_THREADS)
                    const uint32_t* __restrict__ words, const uint32_t* __restrict__ counts, int2* __restrict__ leafr,
                    uint64_t* __restrict__ lkey, int32_t* __restrict__ linst, uint32_t* __restrict__ ctrl, int algo)
 {
+    stage_begin(keys, pdense, words, counts);
     // (skipped -- aborted run, or the other algorithm's chain --: m stays 0
     // and every later stage finds no leaves)
     if (!stage_on(ctrl, algo)) return;
@@ -812,6 +826,7 @@ __global__ void __launch_bounds__(LF_THREADS)
 template <int D>
 __global__ void k_box_levels(const uint32_t* __restrict__ ctrl, typename Traits<D>::Box* __restrict__ sum)
 {
+    stage_begin(ctrl);
     using T = Traits<D>;
     const int lane = threadIdx.x & 31;
     const int64_t m = ctrl[CTRL_M];
@@ -885,6 +900,7 @@ __device__ __forceinline__ void karras(const uint64_t* __restrict__ lkey, int64_
 __global__ void k_karras(const uint64_t* __restrict__ lkey, int64_t m, int4* __restrict__ nmeta,
                          int32_t* __restrict__ parent, int2* __restrict__ child_out, int2* __restrict__ range_out)
 {
+    stage_begin(lkey);
     karras(lkey, m, nmeta, parent, child_out, range_out, nullptr);
 }
 
@@ -905,6 +921,7 @@ __global__ void k_leaf_boxes(const typename Traits<D>::Point* __restrict__ sp, c
                              const uint64_t* __restrict__ lkey, int4* __restrict__ nmeta, int32_t* __restrict__ parent,
                              int2* __restrict__ range_out, int32_t* __restrict__ first_out)
 {
+    stage_begin(sp, leafr, ctrl, dbox, lkey);
     using T = Traits<D>;
     const int lane = threadIdx.x & 31;
     const int64_t m = ctrl[CTRL_M];
@@ -1006,6 +1023,7 @@ __global__ void k_refit(uint32_t* __restrict__ ctrl, const int4* __restrict__ nm
                         const int32_t* __restrict__ nfirst, typename Traits<D>::Box* __restrict__ nodebox,
                         const typename Traits<D>::Box* __restrict__ sum, typename Traits<D>::Node* __restrict__ nodes)
 {
+    stage_begin(nmeta, nfirst, sum);
     using T = Traits<D>;
     using Box = typename T::Box;
     const int lane = threadIdx.x & 31;
@@ -1074,12 +1092,12 @@ cudaError_t launch_density_estimate(const float* points, int64_t n, int dim, con
     if (gb > 152 * 4) gb = 152 * 4;
 #define EST_LAUNCH(D)                                                                      \
     do {                                                                                   \
-        k_est_insert<D><<<1, 1024, 0, s>>>(points, n, smp, g, ctrl, eb.table, eb.slot);   \
-        k_est_count<D><<<(unsigned)gb, 256, 0, s>>>(points, n, stride, g, ctrl, eb.table, eb.counts); \
+        launch(k_est_insert<D>, 1, 1024, 0, s, points, n, smp, g, ctrl, eb.table, eb.slot);   \
+        launch(k_est_count<D>, (unsigned)gb, 256, 0, s, points, n, stride, g, ctrl, eb.table, eb.counts); \
     } while (0)
     GBD_DIM_SWITCH(dim, EST_LAUNCH)
 #undef EST_LAUNCH
-    k_est_result<<<1, 1024, 0, s>>>(eb.slot, smp, eb.counts, n, stride, min_pts, auto_fraction, auto_occupancy,
+    launch(k_est_result, 1, 1024, 0, s, eb.slot, smp, eb.counts, n, stride, min_pts, auto_fraction, auto_occupancy,
                                     eb.result, ctrl);
     note_launches(3);
     return cudaGetLastError();
@@ -1096,7 +1114,7 @@ static inline unsigned grid_for(int64_t work, int threads, int max_blocks)
 void launch_bounds(const float* pts, int64_t n, int dim, uint32_t* ctrl, const BoundsExtra& x, cudaStream_t s)
 {
 #define BOUNDS_LAUNCH(D)                                                                            \
-    k_bounds<D><<<grid_for(n * D, bounds_threads<D>(), 152 * 8), bounds_threads<D>(), 0, s>>>(pts, n, ctrl, x)
+    launch(k_bounds<D>, grid_for(n * D, bounds_threads<D>(), 152 * 8), bounds_threads<D>(), 0, s, pts, n, ctrl, x)
     GBD_DIM_SWITCH(dim, BOUNDS_LAUNCH)
 #undef BOUNDS_LAUNCH
     note_launches(1);
@@ -1104,7 +1122,7 @@ void launch_bounds(const float* pts, int64_t n, int dim, uint32_t* ctrl, const B
 
 void launch_run_begin(uint32_t* ctrl, int algo, cudaStream_t s)
 {
-    k_run_begin<<<1, 32, 0, s>>>(ctrl, algo);
+    launch(k_run_begin, 1, 32, 0, s, ctrl, algo);
     note_launches(1);
 }
 
@@ -1112,8 +1130,8 @@ void launch_morton32(const float* pts, int64_t n, int dim, const uint32_t* ctrl,
                      uint32_t* vals, cudaStream_t s)
 {
     const unsigned g = grid_for(n, 256, 152 * 16);
-    if (dim == 3) k_morton32<3><<<g, 256, 0, s>>>(pts, n, ctrl, bits, keys, vals);
-    else k_morton32<2><<<g, 256, 0, s>>>(pts, n, ctrl, bits, keys, vals);
+    if (dim == 3) launch(k_morton32<3>, g, 256, 0, s, pts, n, ctrl, bits, keys, vals);
+    else launch(k_morton32<2>, g, 256, 0, s, pts, n, ctrl, bits, keys, vals);
     note_launches(1);
 }
 
@@ -1121,7 +1139,7 @@ void launch_morton64(const float* pts, int64_t n, int dim, const uint32_t* ctrl,
                      uint32_t* vals, cudaStream_t s)
 {
     const unsigned g = grid_for(n, 256, 152 * 16);
-#define M64_LAUNCH(D) k_morton64<D><<<g, 256, 0, s>>>(pts, n, ctrl, bits, keys, vals)
+#define M64_LAUNCH(D) launch(k_morton64<D>, g, 256, 0, s, pts, n, ctrl, bits, keys, vals)
     GBD_DIM_SWITCH(dim, M64_LAUNCH)
 #undef M64_LAUNCH
     note_launches(1);
@@ -1132,7 +1150,7 @@ void launch_cellkey_packed(const float* pts, int64_t n, int dim, const GridParam
 {
     const unsigned g = grid_for(n, 256, 152 * 16);
 #define CKP_LAUNCH(D) \
-    k_cellkey_packed<D><<<g, 256, 0, s>>>(pts, n, gp, ctrl, idx_bits, host_passes, words0, words1)
+    launch(k_cellkey_packed<D>, g, 256, 0, s, pts, n, gp, ctrl, idx_bits, host_passes, words0, words1)
     GBD_DIM_SWITCH(dim, CKP_LAUNCH)
 #undef CKP_LAUNCH
     note_launches(1);
@@ -1146,8 +1164,8 @@ void launch_gather_packed(const float* pts, const uint64_t* words, int64_t n, in
 #define GP_LAUNCH(D)                                                                                          \
     do {                                                                                                      \
         auto* spd = static_cast<typename Traits<D>::Point*>(sp);                                              \
-        if (a16) k_gather_packed<D, true><<<g, 256, 0, s>>>(pts, words, n, idx_bits, spd, perm, keys, ctrl);  \
-        else k_gather_packed<D, false><<<g, 256, 0, s>>>(pts, words, n, idx_bits, spd, perm, keys, ctrl);    \
+        if (a16) launch(k_gather_packed<D, true>, g, 256, 0, s, pts, words, n, idx_bits, spd, perm, keys, ctrl);  \
+        else launch(k_gather_packed<D, false>, g, 256, 0, s, pts, words, n, idx_bits, spd, perm, keys, ctrl);    \
     } while (0)
     GBD_DIM_SWITCH(dim, GP_LAUNCH)
 #undef GP_LAUNCH
@@ -1157,8 +1175,8 @@ void launch_gather_packed(const float* pts, const uint64_t* words, int64_t n, in
 void launch_morton_generic(const float* pts, int64_t n, int dim, const GridParams& gp, uint64_t* out, cudaStream_t s)
 {
     const unsigned g = grid_for(n, 256, 152 * 16);
-    if (dim == 3) k_morton_generic<3><<<g, 256, 0, s>>>(pts, n, gp, out);
-    else k_morton_generic<2><<<g, 256, 0, s>>>(pts, n, gp, out);
+    if (dim == 3) launch(k_morton_generic<3>, g, 256, 0, s, pts, n, gp, out);
+    else launch(k_morton_generic<2>, g, 256, 0, s, pts, n, gp, out);
     note_launches(1);
 }
 
@@ -1167,7 +1185,7 @@ void launch_gather(const float* pts, const uint32_t* perm, int64_t n, int dim, v
 {
     const unsigned g = grid_for(n, 256, 152 * 16);
 #define GATHER_LAUNCH(D) \
-    k_gather<D><<<g, 256, 0, s>>>(pts, perm, n, static_cast<typename Traits<D>::Point*>(sp), ctrl, algo)
+    launch(k_gather<D>, g, 256, 0, s, pts, perm, n, static_cast<typename Traits<D>::Point*>(sp), ctrl, algo)
     GBD_DIM_SWITCH(dim, GATHER_LAUNCH)
 #undef GATHER_LAUNCH
     note_launches(1);
@@ -1184,8 +1202,8 @@ cudaError_t launch_leaves(const K* keys, const int32_t* dstart, const uint8_t* p
     if (w2 < LF_MIN_WINDOWS / 2) w2 = LF_MIN_WINDOWS / 2;
     const int windows = (int)(2 * w2);
     const unsigned g = (unsigned)((n + (int64_t)LF_THREADS * windows - 1) / ((int64_t)LF_THREADS * windows));
-    k_leaf_flags<K><<<g, LF_THREADS, 0, s>>>(keys, dstart, pdense, n, windows, id_shift, t.lf, t.lfc, ctrl, algo);
-    k_leaf_records<K><<<g, LF_THREADS, 0, s>>>(keys, pdense, n, windows, id_shift, t.lf, t.lfc, leafr, lkey, linst, ctrl,
+    launch(k_leaf_flags<K>, g, LF_THREADS, 0, s, keys, dstart, pdense, n, windows, id_shift, t.lf, t.lfc, ctrl, algo);
+    launch(k_leaf_records<K>, g, LF_THREADS, 0, s, keys, pdense, n, windows, id_shift, t.lf, t.lfc, leafr, lkey, linst, ctrl,
                                                algo);
     note_launches(2);
     return cudaGetLastError();
@@ -1199,7 +1217,7 @@ void launch_dense_classify(const uint64_t* keys, const void* sp, int64_t n, int 
     if (steps > CELL_STEPS) steps = CELL_STEPS;
     const unsigned g = grid_for(n, (int)steps * CELL_THREADS, 152 * 16);
 #define DC_LAUNCH(D)                                                                                              \
-    k_dense_classify<D><<<g, CELL_THREADS, 0, s>>>(keys, static_cast<const typename Traits<D>::Point*>(sp), n,     \
+    launch(k_dense_classify<D>, g, CELL_THREADS, 0, s, keys, static_cast<const typename Traits<D>::Point*>(sp), n,     \
                                                    min_pts, e2, mps, e2s, lb, t.pdense, t.dstart,                  \
                                                    static_cast<typename Traits<D>::Box*>(t.dbox), ctrl, algo,       \
                                                    (int)steps)
@@ -1251,15 +1269,15 @@ void launch_lbvh(const void* sp, int dim, const int2* leafr, const uint64_t* lke
 #define LB_LAUNCH(D)                                                                                                  \
     do {                                                                                                              \
         using Bx = typename Traits<D>::Box;                                                                           \
-        k_leaf_boxes<D><<<g, 256, 0, s>>>(static_cast<const typename Traits<D>::Point*>(sp), leafr, ctrl,              \
+        launch(k_leaf_boxes<D>, g, 256, 0, s, static_cast<const typename Traits<D>::Point*>(sp), leafr, ctrl,              \
                                           static_cast<const Bx*>(dbox), static_cast<Bx*>(nodebox),                    \
                                           static_cast<Bx*>(nsum), lkey, nmeta, parent, range_out, nfirst);            \
-        if (levels) k_box_levels<D><<<gl, 256, 0, s>>>(ctrl, static_cast<Bx*>(nsum));                                 \
+        if (levels) launch(k_box_levels<D>, gl, 256, 0, s, ctrl, static_cast<Bx*>(nsum));                                 \
     } while (0)
     GBD_DIM_SWITCH(dim, LB_LAUNCH)
 #undef LB_LAUNCH
 #define RF_LAUNCH(D)                                                                                         \
-    k_refit<D><<<g, 256, 0, s>>>(ctrl, nmeta, nfirst, static_cast<typename Traits<D>::Box*>(nodebox),          \
+    launch(k_refit<D>, g, 256, 0, s, ctrl, nmeta, nfirst, static_cast<typename Traits<D>::Box*>(nodebox),          \
                                  static_cast<const typename Traits<D>::Box*>(nsum),                            \
                                  static_cast<typename Traits<D>::Node*>(nodes))
     GBD_DIM_SWITCH(dim, RF_LAUNCH)
@@ -1270,7 +1288,7 @@ void launch_lbvh(const void* sp, int dim, const int2* leafr, const uint64_t* lke
 void launch_karras_only(const uint64_t* lkey, int64_t m, int4* nmeta, int32_t* parent, int2* child_out,
                         int2* range_out, cudaStream_t s)
 {
-    k_karras<<<grid_for(m, 256, 152 * 16), 256, 0, s>>>(lkey, m, nmeta, parent, child_out, range_out);
+    launch(k_karras, grid_for(m, 256, 152 * 16), 256, 0, s, lkey, m, nmeta, parent, child_out, range_out);
     note_launches(1);
 }
 

@@ -20,6 +20,7 @@
 namespace gbd {
 
 thread_local std::string t_err;
+thread_local bool t_overlap = false;
 
 dbscan_status set_error(dbscan_status st, const char* fmt, ...)
 {
@@ -474,6 +475,7 @@ dbscan_status build_index(Workspace* w, const Plan& p, StageTimer& T, const floa
                           float eps, int dense_mp, int algo, ClusterArgs& a, cudaStream_t s)
 {
     w->last_algo = algo == DBSCAN_ALGO_AUTO ? -2 : algo;  // -2: chosen on the device
+    t_overlap = n <= OVERLAP_POINTS;
     launch_run_begin(p.ctrl, algo, s);
     const float e2 = eps * eps;
     const bool fd = algo != DBSCAN_ALGO_DENSEBOX, db = algo != DBSCAN_ALGO_FDBSCAN;

@@ -64,6 +64,7 @@ template <typename K>
 __global__ void __launch_bounds__(THREADS) k_hist(const K* __restrict__ k0, const K* __restrict__ k1, int64_t n,
                                                   int shift0, int passes, SortCtl ctl, uint32_t* __restrict__ hist)
 {
+    stage_begin(k0, k1);
     __shared__ uint32_t sh[SORT_MAX_PASSES * RADIX];
     __shared__ int s_dec;
     const int pd = sort_block_passes(ctl, passes, &s_dec);
@@ -154,6 +155,7 @@ __global__ void __launch_bounds__(THREADS, VALS ? 3 : 4)
                const uint32_t* __restrict__ hist, uint32_t* __restrict__ status, uint32_t* tile_counter,
                uint32_t* err, int wait_limit, int stall_first_tile)
 {
+    stage_begin(hist);
     extern __shared__ __align__(16) unsigned char smem[];
     K* keys_s = reinterpret_cast<K*>(smem);
     uint32_t* vals_s = reinterpret_cast<uint32_t*>(smem + TILE_ITEMS * sizeof(K));
@@ -352,7 +354,7 @@ cudaError_t sort_pairs(K* keys, uint32_t* vals, int64_t n, int shift0, int bits,
     SortCtl ctl = sb.ctl;
     if (!ctl.abort) ctl.abort = sb.err;
     const int hist_blocks = (int)(tiles < 1216 ? tiles : 1216);
-    k_hist<K><<<hist_blocks, THREADS, 0, s>>>(keys, k_alt, n, shift0, passes, ctl, sb.hist);
+    launch(k_hist<K>, hist_blocks, THREADS, 0, s, keys, k_alt, n, shift0, passes, ctl, sb.hist);
     note_launches(1);
     const bool with_vals = vals != nullptr;
     const size_t smem = TILE_ITEMS * (sizeof(K) + (with_vals ? sizeof(uint32_t) : 0));
@@ -364,12 +366,10 @@ cudaError_t sort_pairs(K* keys, uint32_t* vals, int64_t n, int shift0, int bits,
     const int stall = g_stall_first_tile.load(std::memory_order_relaxed);
     for (int p = 0; p < passes; ++p) {
         if (with_vals)
-            k_onesweep<K, true><<<(unsigned)tiles, THREADS, smem, s>>>(
-                keys, vals, k_alt, sb.vals_alt, n, shift0, p, passes, ctl, sb.hist + RADIX * p,
+            launch(k_onesweep<K, true>, (unsigned)tiles, THREADS, smem, s, keys, vals, k_alt, sb.vals_alt, n, shift0, p, passes, ctl, sb.hist + RADIX * p,
                 sb.status + (size_t)RADIX * tiles * p, sb.counters + p, sb.err, limit, stall);
         else
-            k_onesweep<K, false><<<(unsigned)tiles, THREADS, smem, s>>>(
-                keys, nullptr, k_alt, nullptr, n, shift0, p, passes, ctl, sb.hist + RADIX * p,
+            launch(k_onesweep<K, false>, (unsigned)tiles, THREADS, smem, s, keys, nullptr, k_alt, nullptr, n, shift0, p, passes, ctl, sb.hist + RADIX * p,
                 sb.status + (size_t)RADIX * tiles * p, sb.counters + p, sb.err, limit, stall);
         note_launches(1);
     }

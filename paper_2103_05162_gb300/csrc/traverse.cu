@@ -532,6 +532,7 @@ template <int D>
 __global__ void __launch_bounds__(LL_THREADS)
     k_leaf_lists(const __grid_constant__ DevArgs<D> a, const int32_t* __restrict__ parent, const int4* __restrict__ nmeta)
 {
+    stage_begin(parent, nmeta);
     using T = Traits<D>;
     const int64_t m = a.ctrl[CTRL_M];
     const int leaf0 = (int)(m - 1);
@@ -919,6 +920,7 @@ struct PreWarp {
 template <int D>
 __global__ void __maxnreg__(traversal_regs<D>()) k_pre(const __grid_constant__ DevArgs<D> a)
 {
+    stage_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     WarpMem<D>* wm = reinterpret_cast<WarpMem<D>*>(smem) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
@@ -1009,6 +1011,7 @@ constexpr int64_t SPLIT_INTRA = 1 << 22;
 __global__ void k_list_claims(const int32_t* __restrict__ nlist, int lcap, const uint8_t* __restrict__ nbr,
                               const uint8_t* core, int32_t* labels, int64_t n)
 {
+    stage_begin(nlist, nbr, core);
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
         if (!core[q]) list_claim(nlist, lcap, nbr, core, labels, q);
 }
@@ -1092,6 +1095,7 @@ __device__ __forceinline__ void append_kinds(uint32_t* ctrl, int32_t* klist, int
 template <int D>
 __global__ void __launch_bounds__(INTRA_THREADS) k_intra(DevArgs<D> a)
 {
+    stage_begin();
     using P = typename Traits<D>::Point;
     __shared__ SoA<D> soa_s[INTRA_THREADS / 32];
     SoA<D>& soa = soa_s[threadIdx.x >> 5];
@@ -1194,6 +1198,7 @@ __global__ void __launch_bounds__(INTRA_THREADS) k_intra(DevArgs<D> a)
 __global__ void k_kinds(const int2* __restrict__ leafr, const uint8_t* __restrict__ lsolid, uint32_t* ctrl,
                         int32_t* __restrict__ klist, int64_t m_cap)
 {
+    stage_begin(leafr, lsolid);
     const int lane = threadIdx.x & 31;
     const int64_t m = ctrl[CTRL_M];
     for (int64_t base = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; base < m;
@@ -1699,6 +1704,7 @@ struct MainWarp {
 template <int D>
 __global__ void __maxnreg__(main_regs<D>()) k_main(const __grid_constant__ DevArgs<D> a)
 {
+    stage_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     WarpMem<D>* wm = reinterpret_cast<WarpMem<D>*>(smem) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
@@ -1791,6 +1797,7 @@ __global__ void k_init_from_counts(const uint8_t* __restrict__ pdense, const int
                                    int32_t* __restrict__ labels, uint8_t* __restrict__ core,
                                    int32_t* __restrict__ canon, uint32_t* __restrict__ ctrl)
 {
+    stage_begin(pdense, dstart, ncount);
     clear_work(ctrl);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         if (pdense && pdense[i]) {
@@ -1812,6 +1819,7 @@ __global__ void k_core_from_input(const uint32_t* __restrict__ perm, const uint8
                                   const uint8_t* __restrict__ pdense, int64_t n, uint8_t* __restrict__ core,
                                   const uint32_t* __restrict__ ctrl)
 {
+    stage_begin(perm, core_in, pdense, ctrl);
     if (!stage_on(ctrl, -1)) return;  // aborted run: perm may hold stale words
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         core[i] = ((pdense && pdense[i]) || core_in[perm[i]]) ? 1 : 0;
@@ -1824,6 +1832,7 @@ __global__ void k_init(const uint8_t* __restrict__ pdense, const int32_t* __rest
                        int min_pts, int32_t* __restrict__ labels, uint8_t* __restrict__ core,
                        uint8_t* __restrict__ nbr, int32_t* __restrict__ canon, uint32_t* __restrict__ ctrl)
 {
+    stage_begin(pdense, dstart);
     clear_work(ctrl);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         if (pdense && pdense[i]) {
@@ -1842,6 +1851,7 @@ __global__ void k_init(const uint8_t* __restrict__ pdense, const int32_t* __rest
 __global__ void k_finalize(int32_t* labels, const uint8_t* __restrict__ core, const uint32_t* __restrict__ perm,
                            int64_t n, int32_t* __restrict__ canon, const uint32_t* __restrict__ ctrl)
 {
+    stage_begin(core, perm, ctrl);
     if (!stage_on(ctrl, -1)) return;
     // warp-uniform trip count: warp_atomic_min needs all 32 lanes
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -1859,6 +1869,7 @@ __global__ void k_relabel(const int32_t* labels, const uint8_t* __restrict__ cor
                           int64_t n, int mode, const int32_t* __restrict__ canon, int32_t* __restrict__ out,
                           uint8_t* __restrict__ core_out, const uint32_t* __restrict__ ctrl)
 {
+    stage_begin(labels, core, perm, canon, ctrl);
     // aborted run (non-finite input, a sort that gave up): perm may hold
     // stale words, so nothing is written; the error is reported at the next
     // host sync point
@@ -1945,7 +1956,7 @@ void run_pre(const ClusterArgs& a, cudaStream_t s)
     const size_t smem = sizeof(WarpMem<D>) * (size_t)(a.block / 32);
     int& g = blocks[a.block / 32];
     if (!g) g = persistent_blocks((const void*)k_pre<D>, a.block, smem);
-    k_pre<D><<<g, a.block, smem, s>>>(dev_args<D>(a));
+    launch(k_pre<D>, g, a.block, smem, s, dev_args<D>(a));
 }
 
 template <int D>
@@ -1955,7 +1966,7 @@ void run_main_walk(const ClusterArgs& a, cudaStream_t s)
     const size_t smem = sizeof(WarpMem<D>) * (size_t)(a.block / 32);
     int& g = blocks[a.block / 32];
     if (!g) g = persistent_blocks((const void*)k_main<D>, a.block, smem);
-    k_main<D><<<g, a.block, smem, s>>>(dev_args<D>(a));
+    launch(k_main<D>, g, a.block, smem, s, dev_args<D>(a));
 }
 
 template <int D>
@@ -1963,16 +1974,16 @@ void run_main(const ClusterArgs& a, cudaStream_t s)
 {
     const bool split = a.n >= SPLIT_INTRA;
     if (split && a.lcap > 0) {
-        k_list_claims<<<152 * 16, 256, 0, s>>>(a.nlist, a.lcap, a.nbr, a.core, a.labels, a.n);
+        launch(k_list_claims, 152 * 16, 256, 0, s, a.nlist, a.lcap, a.nbr, a.core, a.labels, a.n);
         note_launches(1);
     }
     int64_t gw = (a.m_cap * 32 + INTRA_THREADS - 1) / INTRA_THREADS;
     if (gw > 152 * 16) gw = 152 * 16;
-    k_intra<D><<<(unsigned)gw, INTRA_THREADS, 0, s>>>(dev_args<D>(a));
+    launch(k_intra<D>, (unsigned)gw, INTRA_THREADS, 0, s, dev_args<D>(a));
     if (split) {
         int64_t gk = (a.m_cap + 255) / 256;
         if (gk > 152 * 8) gk = 152 * 8;
-        k_kinds<<<(unsigned)gk, 256, 0, s>>>(a.leafr, a.lsolid, a.ctrl, a.klist, a.m_cap);
+        launch(k_kinds, (unsigned)gk, 256, 0, s, a.leafr, a.lsolid, a.ctrl, a.klist, a.m_cap);
         note_launches(1);
     }
     run_main_walk<D>(a, s);
@@ -1984,7 +1995,7 @@ cudaError_t launch_cluster_init(const ClusterArgs& a, cudaStream_t s)
 {
     int64_t gn = (a.n + 255) / 256;
     if (gn > 152 * 16) gn = 152 * 16;
-    k_init<<<(unsigned)gn, 256, 0, s>>>(a.pdense, a.dstart, a.n, a.min_pts, a.labels, a.core, a.nbr, a.canon, a.ctrl);
+    launch(k_init, (unsigned)gn, 256, 0, s, a.pdense, a.dstart, a.n, a.min_pts, a.labels, a.core, a.nbr, a.canon, a.ctrl);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -1993,7 +2004,7 @@ cudaError_t launch_cluster_from_counts(const ClusterArgs& a, int min_pts, cudaSt
 {
     int64_t gn = (a.n + 255) / 256;
     if (gn > 152 * 16) gn = 152 * 16;
-    k_init_from_counts<<<(unsigned)gn, 256, 0, s>>>(a.pdense, a.dstart, a.ncount, a.n, min_pts, a.labels, a.core,
+    launch(k_init_from_counts, (unsigned)gn, 256, 0, s, a.pdense, a.dstart, a.ncount, a.n, min_pts, a.labels, a.core,
                                                     a.canon, a.ctrl);
     note_launches(1);
     return cudaGetLastError();
@@ -2004,7 +2015,7 @@ cudaError_t launch_cluster_starts(const ClusterArgs& a, cudaStream_t s)
     count_phase(0, s);
     int64_t gm = (a.m_cap + 255) / 256;
     if (gm > 152 * 8) gm = 152 * 8;
-#define LL_LAUNCH(D) k_leaf_lists<D><<<(unsigned)gm, LL_THREADS, 0, s>>>(dev_args<D>(a), a.parent, a.nmeta)
+#define LL_LAUNCH(D) launch(k_leaf_lists<D>, (unsigned)gm, LL_THREADS, 0, s, dev_args<D>(a), a.parent, a.nmeta)
     GBD_DIM_SWITCH(a.dim, LL_LAUNCH)
 #undef LL_LAUNCH
     note_launches(1);
@@ -2038,7 +2049,7 @@ cudaError_t launch_cluster_core_from_input(const ClusterArgs& a, const uint8_t* 
 {
     int64_t gn = (a.n + 255) / 256;
     if (gn > 152 * 16) gn = 152 * 16;
-    k_core_from_input<<<(unsigned)gn, 256, 0, s>>>(a.perm, core_in, a.pdense, a.n, a.core, a.ctrl);
+    launch(k_core_from_input, (unsigned)gn, 256, 0, s, a.perm, core_in, a.pdense, a.n, a.core, a.ctrl);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -2047,8 +2058,8 @@ cudaError_t launch_cluster_final(const ClusterArgs& a, int32_t* labels_out, uint
 {
     int64_t gn = (a.n + 255) / 256;
     if (gn > 152 * 16) gn = 152 * 16;
-    k_finalize<<<(unsigned)gn, 256, 0, s>>>(a.labels, a.core, a.perm, a.n, a.canon, a.ctrl);
-    k_relabel<<<(unsigned)gn, 256, 0, s>>>(a.labels, a.core, a.perm, a.n, a.mode, a.canon, labels_out, core_out,
+    launch(k_finalize, (unsigned)gn, 256, 0, s, a.labels, a.core, a.perm, a.n, a.canon, a.ctrl);
+    launch(k_relabel, (unsigned)gn, 256, 0, s, a.labels, a.core, a.perm, a.n, a.mode, a.canon, labels_out, core_out,
                                            a.ctrl);
     note_launches(2);
     return cudaGetLastError();
