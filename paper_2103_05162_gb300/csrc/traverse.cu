@@ -856,6 +856,7 @@ struct PreWarp {
             }
             if (!__any_sync(FULL, act)) return false;
             if (__any_sync(FULL, act != was)) qbox = warp_box<D>(p, act);
+            if (!__any_sync(FULL, cand)) return true;  // no leaf is left to stream
         }
         // few queries: their box says little, so each of them is tested against
         // the lanes' leaves

@@ -58,3 +58,18 @@ def test_clumps_in_a_batch():
     for b, (x, e, m) in enumerate(inst):
         s = slice(int(offs[b]), int(offs[b + 1]))
         assert_matches_oracle(x, float(np.float32(e)), m, gb.MODE_DBSCAN, lab[s].cpu().numpy(), core[s].cpu().numpy())
+
+
+@pytest.mark.parametrize("d", [2, 3, 5])
+def test_cell_near_the_box_of_a_tile_but_near_none_of_its_points(d):
+    # two arms of isolated points whose box reaches a dense cell larger than a
+    # tile: preprocessing's only candidate leaf, and it drops out for every query
+    w = 1.0 / np.sqrt(d)  # cells of eps 1
+    X = np.zeros((22 + 40, d))
+    X[:11, 0] = X[11:22, 1] = 31.8 * w
+    X[:11, 1] = X[11:22, 0] = 1.1 * np.arange(11)
+    X[22:, :2] = 32.3 * w + np.random.default_rng(d).uniform(-0.1 * w, 0.1 * w, size=(40, 2))
+    X = X.astype(np.float32)
+    lab, core = gb.dbscan_run(torch.from_numpy(X).cuda(), 1.0, 5, algo="densebox", want_core=True, sync=True)
+    assert_matches_oracle(X, 1.0, 5, gb.MODE_DBSCAN, lab.cpu().numpy(), core.cpu().numpy())
+    assert (lab[:22] == -1).all() and (lab[22:] == 22).all()
