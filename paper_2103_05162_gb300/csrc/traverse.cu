@@ -306,8 +306,7 @@ __device__ __forceinline__ typename Traits<D>::Box load_box(const typename Trait
 // cost a chain of dependent loads for each, with a third of the lanes idle.
 // (PointStream needs a leaf with `on` in some lane.)
 struct StreamMem {
-    int us[32];
-    int off[32];
+    int first[32];  // per leaf of the stream: its first point less its first position
 };
 
 template <int D>
@@ -315,7 +314,7 @@ struct PointStream {
     using P = typename Traits<D>::Point;
     const P* __restrict__ sp;
     StreamMem& st;
-    int off;       // first position of this lane's leaf in the stream (no leaf: past its end)
+    int off;       // first position of this lane's leaf in the stream (no leaf: beyond any)
     int total;
     int before;    // leaves that start before the current 32 positions, less one
     int b;         // the step's first position
@@ -341,10 +340,9 @@ struct PointStream {
         __syncwarp();
         if (on) {
             const int r = __popc(om & ((1u << lane) - 1u));
-            st.us[r] = us;
-            st.off[r] = off;
+            st.first[r] = us - off;
         } else {
-            off = total;
+            off = INT_MAX;
         }
         __syncwarp();
         before = -1;
@@ -353,10 +351,11 @@ struct PointStream {
     }
     __device__ __forceinline__ void load(int at)
     {
-        const unsigned sm = __reduce_or_sync(FULL, (unsigned)(off - at) < 32u && off < total ? 1u << (off - at) : 0u);
+        const unsigned t = (unsigned)(off - at);
+        const unsigned sm = __reduce_or_sync(FULL, t < 32u ? 1u << t : 0u);
         const int r = before + __popc(sm & (0xffffffffu >> (31 - lane)));
         before += __popc(sm);
-        jn = at + lane < total ? st.us[r] + (at + lane - st.off[r]) : st.us[0];
+        jn = st.first[r] + min(at + lane, total - 1);  // (past the end: the last point)
         pn = sp[jn];
     }
     __device__ __forceinline__ bool next()
@@ -704,13 +703,13 @@ __device__ __forceinline__ int next_leaf(uint32_t* ctr)
     return __shfl_sync(FULL, L, 0);
 }
 
-// Register caps of the traversal kernels: 56 in 2D and 3D (nine 128-thread
-// blocks per SM, measured fastest on the 16M halo workload); more above 3D,
-// where a point and its packed copy take 3 D registers
+// Register caps of the preprocessing kernel, the fastest measured: 48 in 3D
+// (16.8M halos 1356 us, 56: 1397), 56 in 2D (4.2M road points 314, 48: 328), 80 in
+// 5D (400K points 239, 96: 252)
 template <int D>
 constexpr int traversal_regs()
 {
-    return D <= 3 ? 56 : (D <= 5 ? 96 : 128);
+    return D == 2 ? 56 : (D == 3 ? 48 : (D <= 5 ? 80 : 112));
 }
 
 // (the main phase holds more state per lane and waits on union-find chains)
@@ -731,7 +730,7 @@ constexpr int main_regs()
 // Issue-bound (75% of the slots; 1700 instructions per tile on 16.8M halos,
 // a quarter of them the tile's own pairs): visiting leaf by leaf, with a test
 // of each query against each leaf's box, took 1580 us there and 338 us on 400K
-// 5D points, this takes 1460 and 263 us.
+// 5D points, this takes 1350 and 239 us.
 constexpr int FEW_QUERIES = 8;
 
 template <int D>
@@ -761,8 +760,10 @@ struct PreWarp {
         const unsigned am0 = am;
         const bool list = a.lcap > 0;
         int32_t* row = a.nlist + (int64_t)(qs + lane) * a.lcap;
-        if (__popc(am) < n) {
-            // lane per staged point, looping over the queries
+        if (2 * __popc(am) < n) {
+            // lane per staged point, looping over the queries: a step of it
+            // costs as much as a step of the other loop, which takes two
+            // staged points (16.8M halos 1397 us, 1461 without the factor)
             const bool in = lane < n;
             const P rp = wm.soa.get(lane);
             const int ri = wm.idx[lane];
@@ -954,6 +955,7 @@ __global__ void __maxnreg__(traversal_regs<D>()) k_pre(const __grid_constant__ D
         if (counts) {
             const typename NB<D>::PP pp = NB<D>::pack(w.p);
             int u = 0;
+#pragma unroll 2
             for (; u + 1 < k && cnt < tp.min_pts; u += 2) {
                 float d0, d1;
                 wm->soa.d2pair(pp, u, d0, d1);
