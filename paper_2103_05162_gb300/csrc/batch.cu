@@ -241,10 +241,9 @@ struct BatchPlan {
     int2* leafr;
     uint64_t* lkey;
     int32_t* linst;
-    void* nodebox;
+    void* leafbox;
     void* nodes;
     int4* nmeta;
-    int32_t* parent;
     int32_t* nfirst;  // first leaf of each internal node
     void* nsum;       // block summaries of the leaf boxes
     int2* range;
@@ -291,10 +290,9 @@ size_t carve_batch(BatchPlan& p, void* base, int64_t n, int count, int algo, int
     p.leafr = c.take<int2>(n);
     p.lkey = c.take<uint64_t>(n);
     p.linst = c.take<int32_t>(n);
-    p.nodebox = c.take<Traits<3>::Box>(2 * n);
+    p.leafbox = c.take<Traits<3>::Box>(n);
     p.nodes = c.take<Traits<3>::Node>(n);
     p.nmeta = c.take<int4>(n);
-    p.parent = c.take<int32_t>(2 * n);
     p.nfirst = c.take<int32_t>(n);
     p.nsum = c.take<Traits<3>::Box>((size_t)sum_levels_entries(n));
     p.range = c.take<int2>(n);
@@ -382,7 +380,7 @@ cudaError_t enqueue_batch_stages(const BatchPlan& p, int64_t n, int count, int m
         launch_dense_classify(keys, p.sp, n, 3, 0, 0.0f, p.mps, p.e2s, lb, p.db, p.ctrl, -1, s);
     }
     if ((e = launch_batch_leaves(keys, n, lb, p.db, p.leafr, p.lkey, p.linst, p.ctrl, s)) != cudaSuccess) return e;
-    launch_lbvh(p.sp, 3, p.leafr, p.lkey, p.db.dbox, n, p.ctrl, p.nmeta, p.parent, p.nfirst, p.nodebox, p.nsum, p.nodes, s,
+    launch_lbvh(p.sp, 3, p.leafr, p.lkey, p.db.dbox, n, p.ctrl, p.nmeta, p.nfirst, p.leafbox, p.nsum, p.nodes, s,
                 p.range);
     launch(k_inst_roots, grid_n(2 * n), 256, 0, s, p.range, p.linst, p.ctrl, p.iroot);
     note_launches(1);
@@ -398,7 +396,7 @@ cudaError_t enqueue_batch_stages(const BatchPlan& p, int64_t n, int count, int m
     ClusterArgs a;
     a.sp = p.sp;
     a.nodes = p.nodes;
-    a.nodebox = p.nodebox;
+    a.leafbox = p.leafbox;
     a.leafr = p.leafr;
     a.lsolid = p.lsolid;
     a.klist = p.klist;
@@ -407,8 +405,6 @@ cudaError_t enqueue_batch_stages(const BatchPlan& p, int64_t n, int count, int m
     a.tnsib = p.tnsib;
     a.llist = p.llist;
     a.lcount = p.lcount;
-    a.parent = p.parent;
-    a.nmeta = p.nmeta;
     a.pdense = p.db.pdense;
     a.dstart = p.db.dstart;
     a.perm = perm;

@@ -1,6 +1,6 @@
 // Index construction: bounds, space-filling-curve keys, gather into sorted
 // order, DenseBox cell classification and leaf layout, Karras LBVH topology
-// and the atomic bottom-up refit (Sec. 4.1, 4.2).
+// and the node boxes (Sec. 4.1, 4.2).
 #include "build.cuh"
 
 namespace gbd {
@@ -864,10 +864,9 @@ __device__ __forceinline__ int kdelta(const uint64_t* __restrict__ k, int64_t m,
 }
 
 __device__ __forceinline__ void karras(const uint64_t* __restrict__ lkey, int64_t m, int4* __restrict__ nmeta,
-                                       int32_t* __restrict__ parent, int2* __restrict__ child_out,
-                                       int2* __restrict__ range_out, int32_t* __restrict__ first_out)
+                                       int2* __restrict__ child_out, int2* __restrict__ range_out,
+                                       int32_t* __restrict__ first_out)
 {
-    if (blockIdx.x == 0 && threadIdx.x == 0) parent[0] = -1;  // root (or the single leaf when m == 1)
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m - 1; i += (int64_t)gridDim.x * blockDim.x) {
         const int d = (kdelta(lkey, m, i, i + 1) - kdelta(lkey, m, i, i - 1)) > 0 ? 1 : -1;
         const int dmin = kdelta(lkey, m, i, i - d);
@@ -888,8 +887,6 @@ __device__ __forceinline__ void karras(const uint64_t* __restrict__ lkey, int64_
         const int32_t left = (int32_t)(first == gamma ? (m - 1) + gamma : gamma);
         const int32_t right = (int32_t)(last == gamma + 1 ? (m - 1) + gamma + 1 : gamma + 1);
         nmeta[i] = make_int4(left, right, (int32_t)gamma, (int32_t)last);
-        parent[left] = (int32_t)i;
-        parent[right] = (int32_t)i;
         if (child_out) child_out[i] = make_int2(left, right);
         if (range_out) range_out[i] = make_int2((int32_t)first, (int32_t)last);
         if (first_out) first_out[i] = (int32_t)first;
@@ -898,15 +895,14 @@ __device__ __forceinline__ void karras(const uint64_t* __restrict__ lkey, int64_
 
 // the topology alone (component entry point)
 __global__ void k_karras(const uint64_t* __restrict__ lkey, int64_t m, int4* __restrict__ nmeta,
-                         int32_t* __restrict__ parent, int2* __restrict__ child_out, int2* __restrict__ range_out)
+                         int2* __restrict__ child_out, int2* __restrict__ range_out)
 {
     stage_begin(lkey);
-    karras(lkey, m, nmeta, parent, child_out, range_out, nullptr);
+    karras(lkey, m, nmeta, child_out, range_out, nullptr);
 }
 
 // ---------------------------------------------------------------------------
-// Leaf boxes: exact min/max of each leaf's points, stored at unified index
-// (m-1) + l of the node-box array. A thread takes a leaf of at most TILE
+// Leaf boxes: exact min/max of each leaf's points. A thread takes a leaf of at most TILE
 // points (reading its contiguous points in turn: few instructions per point,
 // and consecutive threads' ranges share cache lines); the boxes of the leaves
 // larger than that (dense cells) come from the classification (dbox).
@@ -917,8 +913,8 @@ __global__ void k_karras(const uint64_t* __restrict__ lkey, int64_t m, int4* __r
 template <int D>
 __global__ void k_leaf_boxes(const typename Traits<D>::Point* __restrict__ sp, const int2* __restrict__ leafr,
                              const uint32_t* __restrict__ ctrl, const typename Traits<D>::Box* __restrict__ dbox,
-                             typename Traits<D>::Box* __restrict__ nodebox, typename Traits<D>::Box* __restrict__ sum1,
-                             const uint64_t* __restrict__ lkey, int4* __restrict__ nmeta, int32_t* __restrict__ parent,
+                             typename Traits<D>::Box* __restrict__ leafbox, typename Traits<D>::Box* __restrict__ sum1,
+                             const uint64_t* __restrict__ lkey, int4* __restrict__ nmeta,
                              int2* __restrict__ range_out, int32_t* __restrict__ first_out)
 {
     stage_begin(sp, leafr, ctrl, dbox, lkey);
@@ -950,18 +946,18 @@ __global__ void k_leaf_boxes(const typename Traits<D>::Point* __restrict__ sp, c
                 }
             }
             for (; j < e; ++j) T::grow(b, sp[j]);
-            nodebox[(m - 1) + l] = b;
+            leafbox[l] = b;
             mine = b;
         }
         if (l < m && !small) {
             mine = dbox[s >> 5];
-            nodebox[(m - 1) + l] = mine;
+            leafbox[l] = mine;
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) T::merge(mine, T::shfl_xor(mine, o));
         if (lane == 0) sum1[base >> 5] = mine;
     }
-    karras(lkey, m, nmeta, parent, nullptr, range_out, first_out);
+    karras(lkey, m, nmeta, nullptr, range_out, first_out);
 }
 
 // ---------------------------------------------------------------------------
@@ -1020,7 +1016,7 @@ __device__ typename Traits<D>::Box range_box(const typename Traits<D>::Box* __re
 
 template <int D>
 __global__ void k_refit(uint32_t* __restrict__ ctrl, const int4* __restrict__ nmeta,
-                        const int32_t* __restrict__ nfirst, typename Traits<D>::Box* __restrict__ nodebox,
+                        const int32_t* __restrict__ nfirst, const typename Traits<D>::Box* __restrict__ leafbox,
                         const typename Traits<D>::Box* __restrict__ sum, typename Traits<D>::Node* __restrict__ nodes)
 {
     stage_begin(nmeta, nfirst, sum);
@@ -1029,7 +1025,6 @@ __global__ void k_refit(uint32_t* __restrict__ ctrl, const int4* __restrict__ nm
     const int lane = threadIdx.x & 31;
     const int64_t m = ctrl[CTRL_M];
     if (m <= 1) return;
-    const Box* leafbox = nodebox + (m - 1);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     // whole warps iterate together (the long ranges take all lanes)
     for (int64_t base = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; base < m - 1; base += stride) {
@@ -1052,9 +1047,6 @@ __global__ void k_refit(uint32_t* __restrict__ ctrl, const int4* __restrict__ nm
             for (; j <= mt.z; ++j) T::merge(L, ld_box<D>(leafbox + j));
 #pragma unroll 4
             for (; j <= mt.w; ++j) T::merge(R, ld_box<D>(leafbox + j));
-            Box U = L;
-            T::merge(U, R);
-            nodebox[p] = U;
             nodes[p] = T::make_node(L, R, mt.x, mt.y, mt.z, mt.w);
         }
         unsigned big = __ballot_sync(FULL, ok && !small);
@@ -1065,12 +1057,7 @@ __global__ void k_refit(uint32_t* __restrict__ ctrl, const int4* __restrict__ nm
                       w = __shfl_sync(FULL, mt.w, src);
             const Box L = range_box<D>(leafbox, sum, m, f, g, lane);
             const Box R = range_box<D>(leafbox, sum, m, (int64_t)g + 1, w, lane);
-            if (lane == src) {
-                Box U = L;
-                T::merge(U, R);
-                nodebox[p] = U;
-                nodes[p] = T::make_node(L, R, mt.x, mt.y, mt.z, mt.w);
-            }
+            if (lane == src) nodes[p] = T::make_node(L, R, mt.x, mt.y, mt.z, mt.w);
         }
     }
 }
@@ -1259,7 +1246,7 @@ cudaError_t launch_tile_leaves64(const uint64_t* keys, int64_t n, const DenseBox
 }
 
 void launch_lbvh(const void* sp, int dim, const int2* leafr, const uint64_t* lkey, const void* dbox, int64_t m_cap,
-                 uint32_t* ctrl, int4* nmeta, int32_t* parent, int32_t* nfirst, void* nodebox, void* nsum, void* nodes, cudaStream_t s,
+                 uint32_t* ctrl, int4* nmeta, int32_t* nfirst, void* leafbox, void* nsum, void* nodes, cudaStream_t s,
                  int2* range_out)
 {
     const unsigned g = grid_for(m_cap, 256, 152 * 16);
@@ -1270,14 +1257,14 @@ void launch_lbvh(const void* sp, int dim, const int2* leafr, const uint64_t* lke
     do {                                                                                                              \
         using Bx = typename Traits<D>::Box;                                                                           \
         launch(k_leaf_boxes<D>, g, 256, 0, s, static_cast<const typename Traits<D>::Point*>(sp), leafr, ctrl,              \
-                                          static_cast<const Bx*>(dbox), static_cast<Bx*>(nodebox),                    \
-                                          static_cast<Bx*>(nsum), lkey, nmeta, parent, range_out, nfirst);            \
+                                          static_cast<const Bx*>(dbox), static_cast<Bx*>(leafbox),                    \
+                                          static_cast<Bx*>(nsum), lkey, nmeta, range_out, nfirst);            \
         if (levels) launch(k_box_levels<D>, gl, 256, 0, s, ctrl, static_cast<Bx*>(nsum));                                 \
     } while (0)
     GBD_DIM_SWITCH(dim, LB_LAUNCH)
 #undef LB_LAUNCH
 #define RF_LAUNCH(D)                                                                                         \
-    launch(k_refit<D>, g, 256, 0, s, ctrl, nmeta, nfirst, static_cast<typename Traits<D>::Box*>(nodebox),          \
+    launch(k_refit<D>, g, 256, 0, s, ctrl, nmeta, nfirst, static_cast<typename Traits<D>::Box*>(leafbox),          \
                                  static_cast<const typename Traits<D>::Box*>(nsum),                            \
                                  static_cast<typename Traits<D>::Node*>(nodes))
     GBD_DIM_SWITCH(dim, RF_LAUNCH)
@@ -1285,10 +1272,10 @@ void launch_lbvh(const void* sp, int dim, const int2* leafr, const uint64_t* lke
     note_launches(levels ? 3 : 2);
 }
 
-void launch_karras_only(const uint64_t* lkey, int64_t m, int4* nmeta, int32_t* parent, int2* child_out,
+void launch_karras_only(const uint64_t* lkey, int64_t m, int4* nmeta, int2* child_out,
                         int2* range_out, cudaStream_t s)
 {
-    launch(k_karras, grid_for(m, 256, 152 * 16), 256, 0, s, lkey, m, nmeta, parent, child_out, range_out);
+    launch(k_karras, grid_for(m, 256, 152 * 16), 256, 0, s, lkey, m, nmeta, child_out, range_out);
     note_launches(1);
 }
 

@@ -234,11 +234,11 @@ __host__ __device__ inline int64_t sum_levels_entries(int64_t m)
 // leaf boxes, block summaries (nsum: sum_levels_entries(m_cap) boxes),
 // Karras topology (nfirst: the first leaf of each internal node) and refit
 void launch_lbvh(const void* sp, int dim, const int2* leafr, const uint64_t* lkey, const void* dbox, int64_t m_cap,
-                 uint32_t* ctrl, int4* nmeta, int32_t* parent, int32_t* nfirst, void* nodebox, void* nsum, void* nodes,
+                 uint32_t* ctrl, int4* nmeta, int32_t* nfirst, void* leafbox, void* nsum, void* nodes,
                  cudaStream_t s, int2* range_out = nullptr);
 cudaError_t launch_batch_leaves(const uint64_t* keys, int64_t n, int id_shift, const DenseBoxTemps& t, int2* leafr,
                                 uint64_t* lkey, int32_t* linst, uint32_t* ctrl, cudaStream_t s);
-void launch_karras_only(const uint64_t* lkey, int64_t m, int4* nmeta, int32_t* parent, int2* child_out,
+void launch_karras_only(const uint64_t* lkey, int64_t m, int4* nmeta, int2* child_out,
                         int2* range_out, cudaStream_t s);
 
 // traverse.cu
@@ -248,7 +248,7 @@ constexpr int TRAVERSAL_LEAFCAP = 48; // leaves within eps listed per leaf
 struct ClusterArgs {
     const void* sp;        // sorted points
     const void* nodes;     // m-1 node records
-    const void* nodebox;   // 2m-1 boxes (leaf boxes at m-1+l)
+    const void* leafbox;   // m boxes
     const int2* leafr;     // m leaf records
     uint8_t* lsolid;       // m: the leaf's flag (nothing to do, all points core and in one set, neither)
     int32_t* klist;        // 3 * m_cap: leaf indices by kind
@@ -277,10 +277,7 @@ struct ClusterArgs {
     const float* e2s = nullptr;
     const int32_t* mps = nullptr;
     const int32_t* iroot = nullptr;
-    // tree links (parent of every node, children of internal nodes) and the
-    // per-leaf traversal start written by launch_cluster_pre
-    const int32_t* parent = nullptr;
-    const int4* nmeta = nullptr;
+    // where the walks of a leaf without a list begin (launch_cluster_starts)
     int32_t* tstart = nullptr;
     int2* tsib = nullptr;    // m_cap * TRAVERSAL_SIBCAP: (node, last leaf) of the sibling subtrees within eps
     int8_t* tnsib = nullptr; // m_cap: how many (-1: more than TRAVERSAL_SIBCAP, use tstart)

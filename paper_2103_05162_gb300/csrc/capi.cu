@@ -222,10 +222,9 @@ struct Plan {
     DenseBoxTemps db;
     int2* leafr;
     uint64_t* lkey;
-    void* nodebox;
+    void* leafbox;
     void* nodes;
     int4* nmeta;
-    int32_t* parent;
     int32_t* nfirst;  // first leaf of each internal node
     void* nsum;       // block summaries of the leaf boxes
     uint8_t* lsolid;
@@ -291,10 +290,9 @@ size_t carve_plan(Plan& p, void* base, int64_t n, int dim, int algo, int lcap, b
     p.db.lfc = c.take<uint32_t>(LEAF_BLOCKS * 8);
     p.leafr = c.take<int2>(mc);
     p.lkey = c.take<uint64_t>(mc);
-    p.nodebox = c.take<char>(box * (size_t)(2 * mc));
+    p.leafbox = c.take<char>(box * (size_t)mc);
     p.nodes = c.take<char>(node * (size_t)mc);
     p.nmeta = c.take<int4>(mc);
-    p.parent = c.take<int32_t>(2 * mc);
     p.nfirst = c.take<int32_t>(mc);
     p.nsum = c.take<char>(box * (size_t)sum_levels_entries(mc));
     p.lsolid = c.take<uint8_t>(mc);
@@ -585,14 +583,14 @@ dbscan_status build_index(Workspace* w, const Plan& p, StageTimer& T, const floa
     }
     TRY_CUDA(cudaGetLastError());
     T.begin(ST_LBVH);
-    launch_lbvh(p.sp, dim, p.leafr, p.lkey, p.db.dbox, m_cap, p.ctrl, p.nmeta, p.parent, p.nfirst, p.nodebox, p.nsum,
+    launch_lbvh(p.sp, dim, p.leafr, p.lkey, p.db.dbox, m_cap, p.ctrl, p.nmeta, p.nfirst, p.leafbox, p.nsum,
                 p.nodes, s);
     T.end();
     TRY_CUDA(cudaGetLastError());
 
     a.sp = p.sp;
     a.nodes = p.nodes;
-    a.nodebox = p.nodebox;
+    a.leafbox = p.leafbox;
     a.leafr = p.leafr;
     a.lsolid = p.lsolid;
     a.klist = p.klist;
@@ -601,8 +599,6 @@ dbscan_status build_index(Workspace* w, const Plan& p, StageTimer& T, const floa
     a.tnsib = p.tnsib;
     a.llist = p.llist;
     a.lcount = p.lcount;
-    a.parent = p.parent;
-    a.nmeta = p.nmeta;
     // (automatic choice: the DenseBox flags are all zero when FDbscan ran)
     a.pdense = db ? p.db.pdense : nullptr;
     a.dstart = db ? p.db.dstart : nullptr;
@@ -1299,8 +1295,7 @@ dbscan_status dbscan_lbvh_topology(const uint64_t* leaf_keys, int64_t m, int32_t
     TRY_CUDA(ensure_arena(w->aux, c.off + 256, s));
     Carver d(w->aux.base);
     int4* nmeta = d.take<int4>(m);
-    int32_t* parent = d.take<int32_t>(2 * m);
-    launch_karras_only(leaf_keys, m, nmeta, parent, reinterpret_cast<int2*>(children_out),
+    launch_karras_only(leaf_keys, m, nmeta, reinterpret_cast<int2*>(children_out),
                        reinterpret_cast<int2*>(range_out), s);
     TRY_CUDA(cudaGetLastError());
     return DBSCAN_OK;

@@ -31,6 +31,7 @@
 // applies the rule of Algorithm 3 as it finds each pair, with no neighbour
 // list: core-core pairs are united, a core point claims a non-core neighbour
 // with one compare-and-swap (Sec. 3.2).
+#include <algorithm>
 #include <climits>
 
 #include "build.cuh"
@@ -290,12 +291,12 @@ template <> struct __align__(16) SoA<2> {
 
 // a node or leaf box: one 256-bit load where it is a 32-byte record (2D, 3D)
 template <int D>
-__device__ __forceinline__ typename Traits<D>::Box load_box(const typename Traits<D>::Box* __restrict__ nodebox,
+__device__ __forceinline__ typename Traits<D>::Box load_box(const typename Traits<D>::Box* __restrict__ boxes,
                                                             int64_t i)
 {
     typename Traits<D>::Box b;
-    if constexpr (sizeof(typename Traits<D>::Box) == 32) ldg256(&nodebox[i], b.lo, b.hi);
-    else b = nodebox[i];
+    if constexpr (sizeof(typename Traits<D>::Box) == 32) ldg256(&boxes[i], b.lo, b.hi);
+    else b = boxes[i];
     return b;
 }
 
@@ -405,7 +406,7 @@ template <int D>
 struct DevArgs {
     const typename Traits<D>::Point* sp;
     const typename Traits<D>::Node* nodes;
-    const typename Traits<D>::Box* nodebox;
+    const typename Traits<D>::Box* leafbox;
     const int2* leafr;
     uint8_t* lsolid;
     int32_t* klist;  // m_cap entries per leaf kind
@@ -426,8 +427,8 @@ struct DevArgs {
     const float* e2s;
     const int32_t* mps;
     const int32_t* iroot;
-    // per leaf: the node its traversals start at, and the sibling subtrees
-    // along the way that come within eps (tile_start)
+    // per leaf without a list: the node its traversals start at, and the
+    // sibling subtrees on the way down that come within eps (tile_start)
     int32_t* tstart;
     int2* tsib;
     int8_t* tnsib;
@@ -468,49 +469,153 @@ __device__ __forceinline__ TileParams tile_params(const DevArgs<D>& a, int L)
     return TileParams{a.e2s[b], a.mps[b], a.iroot[b]};
 }
 
-// The lowest ancestor A of each leaf such that no point outside A's subtree
-// is within eps of the leaf's box: walking up from the leaf, every sibling
-// subtree whose box is within eps of the leaf box (box-to-box distance, the
-// same exact pruning test as the traversal) moves the start up to the
-// sibling's parent. Traversals for the leaf's points (each within the leaf
-// box) then start at A instead of the root and skip the levels above it,
-// where only one path could lead to a neighbour.
-template <int D>
-__device__ __forceinline__ int tile_start(const DevArgs<D>& a, const int32_t* __restrict__ parent,
-                                          const int4* __restrict__ nmeta, int64_t L, int leaf0, const TileParams& tp,
-                                          const typename Traits<D>::Box& tb)
+// The lowest ancestor A of a leaf such that no point outside A's subtree is
+// within eps of the leaf's box, and the sibling subtrees on the way down from
+// A that come within eps of it: traversals for the leaf's points (each within
+// the leaf box) then start at A, or at those siblings, instead of the root and
+// skip the levels above, where only one path could lead to a neighbour. Found
+// from the top: one node record per level holds both children's boxes and
+// says on which side the leaf lies, so a level is one dependent load, and the
+// upper levels are the same for all lanes. Climbing from the leaf took three
+// per level (parent, its children, the sibling's box) and 409 us for the lists
+// of 16.8M halos, where this takes 366: most of it is the walk below the
+// siblings.
+//
+// Returns the number of siblings (-1: more than SIBCAP); the first SIBCAP go
+// to near(k, sibling, last leaf under it) from the top down.
+template <int D, typename Near>
+__device__ __forceinline__ int tile_start(const DevArgs<D>& a, int L, int leaf0, const TileParams& tp,
+                                          const typename Traits<D>::Box& q, int& start, Near near)
 {
-    int cur = leaf0 + (int)L;
-    int start = cur;
-    int ns = 0;  // siblings recorded (-1: more than SIBCAP)
-    int2* sib_out = a.tsib + L * SIBCAP;
-    // a longer climb than the tree is deep means a corrupt tree: start at the
-    // root
-    int steps = 0;
-    while (cur != tp.start) {
-        const int p = parent[cur];
-        if (p < 0 || ++steps > TREE_DEPTH) {
+    int cur = tp.start, ns = 0;
+    start = leaf0 + L;
+    // a longer way down than the tree is deep means a corrupt tree: start at
+    // the root
+#pragma unroll 1
+    for (int steps = 0; cur < leaf0; ++steps) {
+        if (steps > TREE_DEPTH) {
             start = tp.start;
-            ns = -1;
+            return -1;
+        }
+        const auto nd = NB<D>::load(a.nodes, cur);
+        float dl, dr;
+        NB<D>::bd2(nd, q, dl, dr);
+        const bool right = L > nd.m.z;
+        if ((right ? dl : dr) <= tp.e2) {
+            if (ns == 0) start = cur;
+            if (ns < SIBCAP) near(ns, right ? nd.m.x : nd.m.y, right ? nd.m.z : nd.m.w);
+            ++ns;
+        }
+        cur = right ? nd.m.y : nd.m.x;
+    }
+    return ns <= SIBCAP ? ns : -1;
+}
+
+// The roots of leaf L's walk onto an empty stack (the top is taken first):
+// its sibling leaves from the farthest ancestor down, then the sibling
+// subtrees from the nearest up, or the start node where there are more than
+// SIBCAP of them. Subtrees whose leaves all precede mask_lo are left out.
+template <int D>
+__device__ __forceinline__ int walk_roots(const DevArgs<D>& a, int L, int leaf0, int mask_lo, int* stack, int lane)
+{
+    const int ns = a.tnsib[L];
+    int item = -1;
+    if (ns >= 0) {
+        if (lane < ns) {
+            const int2 t = a.tsib[(int64_t)L * SIBCAP + ns - 1 - lane];
+            if (t.y >= mask_lo) item = t.x;
+        }
+    } else if (lane == 0) {
+        item = a.tstart[L];
+    }
+    const unsigned lm = __ballot_sync(FULL, item >= leaf0), im = __ballot_sync(FULL, item >= 0 && item < leaf0);
+    const int sp = __popc(lm) + __popc(im);
+    const int pos = item >= leaf0 ? __popc(lm >> lane) - 1 : __popc(lm) + __popc(im & ((1u << lane) - 1u));
+    if (item >= 0) stack[sp - 1 - pos] = item;
+    __syncwarp();
+    return sp;
+}
+
+// A node's children within eps of the box q, in the order they are taken:
+// leaves before subtrees, left before right (RIGHT: the right one of two
+// subtrees first; -1: none)
+template <int D, bool RIGHT = false>
+__device__ __forceinline__ int2 near_children(const DevArgs<D>& a, int node, const typename Traits<D>::Box& q, float e2,
+                                              int leaf0, int mask_lo)
+{
+    const auto nd = NB<D>::load(a.nodes, node);
+    float dl, dr;
+    NB<D>::bd2(nd, q, dl, dr);
+    int l = dl <= e2 && nd.m.z >= mask_lo ? nd.m.x : -1;
+    int r = dr <= e2 && nd.m.w >= mask_lo ? nd.m.y : -1;
+    if (l < 0 || (l < leaf0 && (r >= leaf0 || (RIGHT && r >= 0)))) { const int t = l; l = r; r = t; }
+    return make_int2(l, r);
+}
+
+// Where a leaf has no list (more than LEAFCAP leaves within eps): the next
+// leaves of its walk through the tree, up to 32 of them into wm.cand (mask_lo:
+// only leaves from there on). Up to 32 nodes from the top of the stack are
+// expanded a step, each in place, so that the leaves come out in the order of
+// a walk that takes one node at a time -- whose chain of dependent loads, one
+// per node, was a third of the main phase on dense data. Returns how many
+// (fewer than 32: the walk is over).
+template <int D, bool RIGHT = false>
+__device__ __forceinline__ int walk_next(const DevArgs<D>& a, WarpMem<D>& wm, int& sp, int& nc, int64_t& steps,
+                                         int64_t m, const typename Traits<D>::Box& q, float e2, int mask_lo, int lane)
+{
+    const int leaf0 = (int)(m - 1);
+    const unsigned lt = (1u << lane) - 1u;
+#pragma unroll 1
+    while (sp > 0 && nc < 32) {
+        // each step enters a node or emits a leaf, each at most once; more
+        // steps can only come from a corrupt tree: flag it and stop
+        if (++steps > 2 * m) {
+            if (lane == 0) atomicOr(&a.ctrl[CTRL_ERR], ERR_STACK);
+            sp = 0;
             break;
         }
-        const int4 nm = nmeta[p];
-        const int sib = nm.x == cur ? nm.y : nm.x;
-        const typename Traits<D>::Box sb = load_box<D>(a.nodebox, sib);
-        if (box_box<D>(tb, sb) <= tp.e2) {
-            start = p;
-            if (ns >= 0 && ns < SIBCAP) {
-                // the sibling and the last leaf under it
-                sib_out[ns++] = make_int2(sib, sib >= leaf0 ? sib - leaf0 : nmeta[sib].w);
-            } else {
-                ns = -1;
-            }
+        const int np = sp > STACK_WIDE ? 1 : min(sp, 32);
+        const int item = lane < np ? wm.stack[sp - 1 - lane] : -1;
+        __syncwarp();
+        // the leaves before the first subtree are next in order
+        const unsigned sub = __ballot_sync(FULL, item >= 0 && item < leaf0);
+        const int lead = sub ? __ffs(sub) - 1 : np;
+        const bool emit = lane < lead && item - leaf0 >= mask_lo;
+        const unsigned em = __ballot_sync(FULL, emit);
+        if (emit) wm.cand[nc + __popc(em & lt)] = item - leaf0;
+        nc += __popc(em);
+        // the others stay, subtrees replaced by their children
+        int2 c = make_int2(-1, -1);
+        if (lane >= lead && lane < np) {
+            GBD_COUNT(CNT_NODE, item < leaf0);
+            c = item >= leaf0 ? make_int2(item, -1) : near_children<D, RIGHT>(a, item, q, e2, leaf0, mask_lo);
         }
-        cur = p;
+        const unsigned c1 = __ballot_sync(FULL, c.x >= 0), c2 = __ballot_sync(FULL, c.y >= 0);
+        sp += __popc(c1) + __popc(c2) - np;
+        if (sp > STACK) {
+            if (lane == 0) atomicOr(&a.ctrl[CTRL_ERR], ERR_STACK);
+            sp = 0;
+            break;
+        }
+        const int pos = sp - 1 - __popc(c1 & lt) - __popc(c2 & lt);
+        if (c.x >= 0) wm.stack[pos] = c.x;
+        if (c.y >= 0) wm.stack[pos - 1] = c.y;
+        __syncwarp();
     }
-    a.tstart[L] = start;
-    a.tnsib[L] = (int8_t)ns;
-    return ns;
+    return min(nc, 32);
+}
+
+// the leaves handed out by walk_next are done with: the rest moves up
+template <int D>
+__device__ __forceinline__ int walk_take(WarpMem<D>& wm, int& nc, int lane)
+{
+    const int U = lane < nc ? wm.cand[lane] : -1;
+    const int V = lane + 32 < nc ? wm.cand[lane + 32] : -1;
+    __syncwarp();
+    if (V >= 0) wm.cand[lane] = V;
+    nc = max(nc - 32, 0);
+    __syncwarp();
+    return U;
 }
 
 // The leaves whose boxes come within eps of each leaf's box (itself
@@ -526,38 +631,94 @@ __device__ __forceinline__ int tile_start(const DevArgs<D>& a, const int32_t* __
 // a walk deeper than LL_STACK gives up its list as well)
 constexpr int LL_THREADS = 256;
 constexpr int LL_STACK = 48;
+// Up to so many leaves per warp of the launch, a warp makes a list: a
+// thread's walk is a chain of one load per node, a warp's of one per level or
+// so (16,384 blob points: 42 us by threads, 19 by warps). With more leaves
+// than the resident threads can take two each, threads do as well (262,144
+// halos, 4 leaves per warp: 57 us either way) or better (524,287 road points,
+// 6 per warp: 25 us by threads, 56 by warps).
+constexpr int LL_ROUNDS = 2;
+
+// Leaf L's list by a whole warp: the same list in the same order (the nearest
+// sibling leaves first, then the sibling subtrees from the farthest down, a
+// node's leaves before its subtrees, its right subtree first).
+template <int D>
+__device__ __forceinline__ void warp_list(const DevArgs<D>& a, int L, int64_t m, WarpMem<D>& wm, int lane)
+{
+    const int leaf0 = (int)(m - 1);
+    const TileParams tp = tile_params(a, L);
+    const typename Traits<D>::Box q = load_box<D>(a.leafbox, L);
+    int32_t* out = a.llist + (int64_t)L * LEAFCAP;
+    int2 mine = make_int2(-1, 0);  // lane k: sibling k from the top and the last leaf under it
+    int start, cnt = LEAFCAP + 1;
+    const int ns = tile_start<D>(a, L, leaf0, tp, q, start, [&](int k, int sib, int last) {
+        if (lane == k) mine = make_int2(sib, last);
+    });
+    if (ns >= 0) {
+        const unsigned lm = __ballot_sync(FULL, mine.x >= leaf0);
+        const unsigned im = __ballot_sync(FULL, mine.x >= 0 && mine.x < leaf0);
+        if (mine.x >= leaf0) out[__popc(lm >> lane) - 1] = mine.x - leaf0;
+        else if (mine.x >= 0) wm.stack[__popc(im >> lane) - 1] = mine.x;
+        __syncwarp();
+        cnt = __popc(lm);
+        int sp = __popc(im), nc = 0;
+        int64_t steps = 0;
+        while (cnt <= LEAFCAP) {
+            const int k = walk_next<D, true>(a, wm, sp, nc, steps, m, q, tp.e2, 0, lane);
+            if (k == 0) break;
+            const int U = walk_take<D>(wm, nc, lane);
+            if (U >= 0 && cnt + lane < LEAFCAP) out[cnt + lane] = U;
+            cnt += k;
+        }
+        __syncwarp();
+    }
+    if (lane == 0) a.lcount[L] = cnt <= LEAFCAP ? (int16_t)cnt : (int16_t)-1;
+    if (cnt > LEAFCAP) {  // walks of this leaf begin at its siblings or its start
+        if (lane < ns) a.tsib[(int64_t)L * SIBCAP + lane] = mine;
+        if (lane == 0) {
+            a.tnsib[L] = (int8_t)ns;
+            a.tstart[L] = start;
+        }
+    }
+}
 
 template <int D>
-__global__ void __launch_bounds__(LL_THREADS)
-    k_leaf_lists(const __grid_constant__ DevArgs<D> a, const int32_t* __restrict__ parent, const int4* __restrict__ nmeta)
+__global__ void __launch_bounds__(LL_THREADS) k_leaf_lists(const __grid_constant__ DevArgs<D> a)
 {
-    stage_begin(parent, nmeta);
+    stage_begin();
     using T = Traits<D>;
     const int64_t m = a.ctrl[CTRL_M];
     const int leaf0 = (int)(m - 1);
-    __shared__ int s_stk[LL_STACK][LL_THREADS];
+    __shared__ __align__(16) int s_stk[LL_STACK][LL_THREADS];
     int* const stk = &s_stk[0][threadIdx.x];  // stk[k * LL_THREADS]: entry k
+    static_assert(sizeof(WarpMem<D>) * (LL_THREADS / 32) <= sizeof(s_stk), "the warps' walks fit");
+    const int64_t warps = (int64_t)gridDim.x * (LL_THREADS / 32);
+    if (m <= LL_ROUNDS * warps) {
+        WarpMem<D>& wm = reinterpret_cast<WarpMem<D>*>(&s_stk[0][0])[threadIdx.x >> 5];
+        for (int64_t L = blockIdx.x * (int64_t)(LL_THREADS / 32) + (threadIdx.x >> 5); L < m; L += warps)
+            warp_list(a, (int)L, m, wm, threadIdx.x & 31);
+        return;
+    }
     for (int64_t L = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; L < m; L += (int64_t)gridDim.x * blockDim.x) {
         const TileParams tp = tile_params(a, (int)L);
         typename T::Box q;
-        q = load_box<D>(a.nodebox, leaf0 + L);
+        q = load_box<D>(a.leafbox, L);
         int32_t* out = a.llist + L * LEAFCAP;
-        int cnt = 0, sp = 0;
-        const int ns = tile_start<D>(a, parent, nmeta, L, leaf0, tp, q);
-        if (ns >= 0) {
-            for (int j = 0; j < ns; ++j) {
-                const int r = a.tsib[L * SIBCAP + j].x;
-                if (r >= leaf0) {  // a leaf sibling: within eps of the box by construction
-                    if (cnt < LEAFCAP) out[cnt] = r - leaf0;
-                    ++cnt;
-                } else if (sp < LL_STACK) {
-                    stk[LL_THREADS * sp++] = r;
-                } else {
-                    cnt = LEAFCAP + 1;
-                }
+        int cnt = 0, sp = 0, start;
+        // the siblings wait at the end of the stack, the nearest first, and
+        // are moved to its start (never past the next one to be read)
+        static_assert(SIBCAP <= LL_STACK, "siblings fit the stack");
+        const int ns = tile_start<D>(a, (int)L, leaf0, tp, q, start,
+                                     [&](int k, int sib, int) { stk[LL_THREADS * (LL_STACK - 1 - k)] = sib; });
+        if (ns < 0) cnt = LEAFCAP + 1;
+        for (int j = LL_STACK - ns; j < LL_STACK; ++j) {
+            const int r = stk[LL_THREADS * j];
+            if (r >= leaf0) {  // a leaf sibling: within eps of the box by construction
+                if (cnt < LEAFCAP) out[cnt] = r - leaf0;
+                ++cnt;
+            } else {
+                stk[LL_THREADS * sp++] = r;
             }
-        } else {
-            cnt = LEAFCAP + 1;
         }
         int64_t steps = 0;
         while (sp > 0 && cnt <= LEAFCAP) {
@@ -587,113 +748,13 @@ __global__ void __launch_bounds__(LL_THREADS)
             }
         }
         a.lcount[L] = cnt <= LEAFCAP ? (int16_t)cnt : (int16_t)-1;
+        if (cnt > LEAFCAP) {  // walks of this leaf begin at its siblings or its start
+            a.tnsib[L] = (int8_t)tile_start<D>(a, (int)L, leaf0, tp, q, start, [&](int k, int sib, int last) {
+                a.tsib[L * SIBCAP + k] = make_int2(sib, last);
+            });
+            a.tstart[L] = start;
+        }
     }
-}
-
-// The roots of leaf L's walk onto an empty stack (the top is taken first):
-// its sibling leaves from the farthest ancestor down, then the sibling
-// subtrees from the nearest up, or the start node where there are more than
-// SIBCAP of them. Subtrees whose leaves all precede mask_lo are left out.
-template <int D>
-__device__ __forceinline__ int walk_roots(const DevArgs<D>& a, int L, int leaf0, int mask_lo, int* stack, int lane)
-{
-    const int ns = a.tnsib[L];
-    int item = -1;
-    if (ns >= 0) {
-        if (lane < ns) {
-            const int2 t = a.tsib[(int64_t)L * SIBCAP + lane];
-            if (t.y >= mask_lo) item = t.x;
-        }
-    } else if (lane == 0) {
-        item = a.tstart[L];
-    }
-    const unsigned lm = __ballot_sync(FULL, item >= leaf0), im = __ballot_sync(FULL, item >= 0 && item < leaf0);
-    const int sp = __popc(lm) + __popc(im);
-    const int pos = item >= leaf0 ? __popc(lm >> lane) - 1 : __popc(lm) + __popc(im & ((1u << lane) - 1u));
-    if (item >= 0) stack[sp - 1 - pos] = item;
-    __syncwarp();
-    return sp;
-}
-
-// A node's children within eps of the box q, in the order they are taken:
-// leaves before subtrees, left before right (-1: none)
-template <int D>
-__device__ __forceinline__ int2 near_children(const DevArgs<D>& a, int node, const typename Traits<D>::Box& q, float e2,
-                                              int leaf0, int mask_lo)
-{
-    const auto nd = NB<D>::load(a.nodes, node);
-    float dl, dr;
-    NB<D>::bd2(nd, q, dl, dr);
-    int l = dl <= e2 && nd.m.z >= mask_lo ? nd.m.x : -1;
-    int r = dr <= e2 && nd.m.w >= mask_lo ? nd.m.y : -1;
-    if (l < 0 || (l < leaf0 && r >= leaf0)) { const int t = l; l = r; r = t; }
-    return make_int2(l, r);
-}
-
-// Where a leaf has no list (more than LEAFCAP leaves within eps): the next
-// leaves of its walk through the tree, up to 32 of them into wm.cand (mask_lo:
-// only leaves from there on). Up to 32 nodes from the top of the stack are
-// expanded a step, each in place, so that the leaves come out in the order of
-// a walk that takes one node at a time -- whose chain of dependent loads, one
-// per node, was a third of the main phase on dense data. Returns how many
-// (fewer than 32: the walk is over).
-template <int D>
-__device__ __forceinline__ int walk_next(const DevArgs<D>& a, WarpMem<D>& wm, int& sp, int& nc, int64_t& steps,
-                                         int64_t m, const typename Traits<D>::Box& q, float e2, int mask_lo, int lane)
-{
-    const int leaf0 = (int)(m - 1);
-    const unsigned lt = (1u << lane) - 1u;
-#pragma unroll 1
-    while (sp > 0 && nc < 32) {
-        // each step enters a node or emits a leaf, each at most once; more
-        // steps can only come from a corrupt tree: flag it and stop
-        if (++steps > 2 * m) {
-            if (lane == 0) atomicOr(&a.ctrl[CTRL_ERR], ERR_STACK);
-            sp = 0;
-            break;
-        }
-        const int np = sp > STACK_WIDE ? 1 : min(sp, 32);
-        const int item = lane < np ? wm.stack[sp - 1 - lane] : -1;
-        __syncwarp();
-        // the leaves before the first subtree are next in order
-        const unsigned sub = __ballot_sync(FULL, item >= 0 && item < leaf0);
-        const int lead = sub ? __ffs(sub) - 1 : np;
-        const bool emit = lane < lead && item - leaf0 >= mask_lo;
-        const unsigned em = __ballot_sync(FULL, emit);
-        if (emit) wm.cand[nc + __popc(em & lt)] = item - leaf0;
-        nc += __popc(em);
-        // the others stay, subtrees replaced by their children
-        int2 c = make_int2(-1, -1);
-        if (lane >= lead && lane < np) {
-            GBD_COUNT(CNT_NODE, item < leaf0);
-            c = item >= leaf0 ? make_int2(item, -1) : near_children<D>(a, item, q, e2, leaf0, mask_lo);
-        }
-        const unsigned c1 = __ballot_sync(FULL, c.x >= 0), c2 = __ballot_sync(FULL, c.y >= 0);
-        sp += __popc(c1) + __popc(c2) - np;
-        if (sp > STACK) {
-            if (lane == 0) atomicOr(&a.ctrl[CTRL_ERR], ERR_STACK);
-            sp = 0;
-            break;
-        }
-        const int pos = sp - 1 - __popc(c1 & lt) - __popc(c2 & lt);
-        if (c.x >= 0) wm.stack[pos] = c.x;
-        if (c.y >= 0) wm.stack[pos - 1] = c.y;
-        __syncwarp();
-    }
-    return min(nc, 32);
-}
-
-// the leaves handed out by walk_next are done with: the rest moves up
-template <int D>
-__device__ __forceinline__ int walk_take(WarpMem<D>& wm, int& nc, int lane)
-{
-    const int U = lane < nc ? wm.cand[lane] : -1;
-    const int V = lane + 32 < nc ? wm.cand[lane + 32] : -1;
-    __syncwarp();
-    if (V >= 0) wm.cand[lane] = V;
-    nc = max(nc - 32, 0);
-    __syncwarp();
-    return U;
 }
 
 __device__ __forceinline__ int next_leaf(uint32_t* ctr)
@@ -825,7 +886,7 @@ struct PreWarp {
             const int2 r = __ldg(&a.leafr[U]);
             us = r.x;
             ue = r.y & 0x7fffffff;
-            bx = load_box<D>(a.nodebox, (m - 1) + U);
+            bx = load_box<D>(a.leafbox, U);
             cand = NB<D>::bbox(qbox, bx) <= e2;
             whole = cand && ue - us >= min_pts && T::box_far2(qbox, bx) <= e2;
         }
@@ -846,7 +907,7 @@ struct PreWarp {
             while (bm) {
                 const int src = __ffs(bm) - 1;
                 bm &= bm - 1;
-                const typename T::Box big = load_box<D>(a.nodebox, (m - 1) + __shfl_sync(FULL, U, src));
+                const typename T::Box big = load_box<D>(a.leafbox, __shfl_sync(FULL, U, src));
                 const int size = __shfl_sync(FULL, ue - us, src);
                 if (act && size >= min_pts && T::far_dist2(p, big) <= e2) {
                     cnt = min_pts;
@@ -971,7 +1032,7 @@ __global__ void __maxnreg__(traversal_regs<D>()) k_pre(const __grid_constant__ D
         if (am) {
             // every point of the tile still counting: their box is the
             // leaf's own (exact min/max of the same points), no reduction
-            w.qbox = am == tile_lanes(k) ? load_box<D>(a.nodebox, (m - 1) + L) : warp_box<D>(w.p, w.act);
+            w.qbox = am == tile_lanes(k) ? load_box<D>(a.leafbox, L) : warp_box<D>(w.p, w.act);
             w.walk(L, m);
         }
         if (counts) {
@@ -1049,7 +1110,7 @@ __device__ __forceinline__ void link_next(const DevArgs<D>& a, const SoA<D>& soa
     const int n = (r.y & 0x7fffffff) - r.x;
     const int idx = r.x + (n <= 32 ? min(lane, n - 1) : (int)((int64_t)n * lane / 32));
     const P p = a.sp[idx];
-    const typename Traits<D>::Box box = load_box<D>(a.nodebox, (m - 1) + L);
+    const typename Traits<D>::Box box = load_box<D>(a.leafbox, L);
     const bool c = lane < n && (tp.min_pts <= 2 || r.y < 0 || a.core[idx]) && NB<D>::pbox(p, box) <= tp.e2;
     if (!__any_sync(FULL, c)) return;
     unsigned hit = 0;
@@ -1562,7 +1623,7 @@ struct MainWarp {
         if (U >= 0) {
             h.fl = *(volatile const uint8_t*)&a.lsolid[U];
             const int2 r = __ldg(&a.leafr[U]);
-            h.box = load_box<D>(a.nodebox, (m - 1) + U);
+            h.box = load_box<D>(a.leafbox, U);
             h.us = r.x;
             h.ue = r.y & 0x7fffffff;
         }
@@ -1648,7 +1709,7 @@ struct MainWarp {
                 const int Us = __shfl_sync(FULL, h.U, src);
                 const int vs = __shfl_sync(FULL, us, src), ve = __shfl_sync(FULL, ue, src);
                 const bool sol = __shfl_sync(FULL, (int)solid, src);
-                const B box = load_box<D>(a.nodebox, (m - 1) + Us);
+                const B box = load_box<D>(a.leafbox, Us);
                 GBD_COUNT(CNT_LEAF, lane == 0);
                 if (!sol) {
                     cell_mixed(vs, ve, box);
@@ -1759,7 +1820,7 @@ __global__ void __maxnreg__(main_regs<D>()) k_main(const __grid_constant__ DevAr
         const bool in = !w.cell && q < w.e;
         const bool c = in && a.core[q];
         w.p = a.sp[in ? q : w.s];
-        w.qbox = load_box<D>(a.nodebox, (m - 1) + L);
+        w.qbox = load_box<D>(a.leafbox, L);
         const typename MainWarp<D>::Head h = w.head(U);
         w.rq = CODE_DONE;
         w.uni = false;
@@ -1924,7 +1985,7 @@ DevArgs<D> dev_args(const ClusterArgs& a)
     DevArgs<D> d;
     d.sp = static_cast<const typename Traits<D>::Point*>(a.sp);
     d.nodes = static_cast<const typename Traits<D>::Node*>(a.nodes);
-    d.nodebox = static_cast<const typename Traits<D>::Box*>(a.nodebox);
+    d.leafbox = static_cast<const typename Traits<D>::Box*>(a.leafbox);
     d.leafr = a.leafr;
     d.lsolid = a.lsolid;
     d.klist = a.klist;
@@ -2016,9 +2077,11 @@ cudaError_t launch_cluster_from_counts(const ClusterArgs& a, int min_pts, cudaSt
 cudaError_t launch_cluster_starts(const ClusterArgs& a, cudaStream_t s)
 {
     count_phase(0, s);
-    int64_t gm = (a.m_cap + 255) / 256;
+    // (a thread per leaf, or up to the resident blocks a warp)
+    int64_t gm = std::max<int64_t>((a.m_cap + LL_THREADS - 1) / LL_THREADS,
+                                   std::min<int64_t>((a.m_cap + LL_THREADS / 32 - 1) / (LL_THREADS / 32), 152 * 4));
     if (gm > 152 * 8) gm = 152 * 8;
-#define LL_LAUNCH(D) launch(k_leaf_lists<D>, (unsigned)gm, LL_THREADS, 0, s, dev_args<D>(a), a.parent, a.nmeta)
+#define LL_LAUNCH(D) launch(k_leaf_lists<D>, (unsigned)gm, LL_THREADS, 0, s, dev_args<D>(a))
     GBD_DIM_SWITCH(a.dim, LL_LAUNCH)
 #undef LL_LAUNCH
     note_launches(1);
