@@ -1,6 +1,8 @@
 // Index construction: bounds, space-filling-curve keys, gather into sorted
 // order, DenseBox cell classification and leaf layout, Karras LBVH topology
 // and the node boxes (Sec. 4.1, 4.2).
+#include <algorithm>
+
 #include "build.cuh"
 
 namespace gbd {
@@ -865,9 +867,9 @@ __device__ __forceinline__ int kdelta(const uint64_t* __restrict__ k, int64_t m,
 
 __device__ __forceinline__ void karras(const uint64_t* __restrict__ lkey, int64_t m, int4* __restrict__ nmeta,
                                        int2* __restrict__ child_out, int2* __restrict__ range_out,
-                                       int32_t* __restrict__ first_out)
+                                       int32_t* __restrict__ first_out, unsigned block, unsigned blocks)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m - 1; i += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t i = block * (int64_t)blockDim.x + threadIdx.x; i < m - 1; i += (int64_t)blocks * blockDim.x) {
         const int d = (kdelta(lkey, m, i, i + 1) - kdelta(lkey, m, i, i - 1)) > 0 ? 1 : -1;
         const int dmin = kdelta(lkey, m, i, i - d);
         int64_t lmax = 2;
@@ -898,31 +900,50 @@ __global__ void k_karras(const uint64_t* __restrict__ lkey, int64_t m, int4* __r
                          int2* __restrict__ child_out, int2* __restrict__ range_out)
 {
     stage_begin(lkey);
-    karras(lkey, m, nmeta, child_out, range_out, nullptr);
+    karras(lkey, m, nmeta, child_out, range_out, nullptr, blockIdx.x, gridDim.x);
 }
 
 // ---------------------------------------------------------------------------
-// Leaf boxes: exact min/max of each leaf's points. A thread takes a leaf of at most TILE
-// points (reading its contiguous points in turn: few instructions per point,
-// and consecutive threads' ranges share cache lines); the boxes of the leaves
-// larger than that (dense cells) come from the classification (dbox).
-// The topology (K7) needs nothing of them, nor they of it: it shares the
-// launch. Each warp also writes the union of its 32 leaves' boxes, the first level of
-// the block summaries that the refit reads (sum1[w]: leaves 32 w .. 32 w + 31).
+// Leaf boxes: exact min/max of each leaf's points. A thread takes a leaf of
+// at most TILE points (reading its contiguous points, four loads in flight;
+// consecutive threads' ranges share cache lines); the boxes of the leaves
+// larger than that (dense cells) come from the classification (dbox). Each
+// warp also writes the union of its 32 leaves' boxes, the first level of the
+// block summaries that the refit reads (sum1[w]: leaves 32 w .. 32 w + 31).
+// The topology (K7) needs nothing of them, nor they of it: the odd blocks of
+// the same launch do it. Both are chains of loads: one after the other in the
+// same threads took 17 us on 16,384 blob points (12 on 1,000, 91 on 16.8M
+// halos), this takes 10 (7.5, 78).
 // ---------------------------------------------------------------------------
 template <int D>
 __global__ void k_leaf_boxes(const typename Traits<D>::Point* __restrict__ sp, const int2* __restrict__ leafr,
                              const uint32_t* __restrict__ ctrl, const typename Traits<D>::Box* __restrict__ dbox,
                              typename Traits<D>::Box* __restrict__ leafbox, typename Traits<D>::Box* __restrict__ sum1,
                              const uint64_t* __restrict__ lkey, int4* __restrict__ nmeta,
-                             int2* __restrict__ range_out, int32_t* __restrict__ first_out)
+                             int2* __restrict__ range_out, int32_t* __restrict__ first_out, int shared_keys)
 {
     stage_begin(sp, leafr, ctrl, dbox, lkey);
     using T = Traits<D>;
     const int lane = threadIdx.x & 31;
     const int64_t m = ctrl[CTRL_M];
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; base < m; base += stride) {
+    const unsigned block = blockIdx.x >> 1, blocks = gridDim.x >> 1;
+    if (blockIdx.x & 1) {
+        // the topology's searches are chains of dependent loads of keys: where all
+        // of them fit, they are read from shared memory
+        if (m <= shared_keys) {
+            extern __shared__ __align__(16) unsigned char smem[];
+            uint64_t* keys = reinterpret_cast<uint64_t*>(smem);
+            if ((int64_t)block * blockDim.x >= m - 1) return;  // no node for this block
+            for (int64_t i = threadIdx.x; i < m; i += blockDim.x) keys[i] = lkey[i];
+            __syncthreads();
+            karras(keys, m, nmeta, nullptr, range_out, first_out, block, blocks);
+        } else {
+            karras(lkey, m, nmeta, nullptr, range_out, first_out, block, blocks);
+        }
+        return;
+    }
+    const int64_t stride = (int64_t)blocks * blockDim.x;
+    for (int64_t base = block * (int64_t)blockDim.x + threadIdx.x - lane; base < m; base += stride) {
         const int64_t l = base + lane;
         int s = 0, e = 0;
         if (l < m) {
@@ -938,6 +959,7 @@ __global__ void k_leaf_boxes(const typename Traits<D>::Point* __restrict__ sp, c
             if constexpr (D == 3) {
                 // two 16-byte points per 256-bit load from an even index on
                 if ((j & 1) && j < e) T::grow(b, sp[j++]);
+#pragma unroll 4
                 for (; j + 1 < e; j += 2) {
                     float4 p0, p1;
                     ldg256(&sp[j], p0, p1);
@@ -945,6 +967,7 @@ __global__ void k_leaf_boxes(const typename Traits<D>::Point* __restrict__ sp, c
                     T::grow(b, p1);
                 }
             }
+#pragma unroll 4
             for (; j < e; ++j) T::grow(b, sp[j]);
             leafbox[l] = b;
             mine = b;
@@ -957,7 +980,6 @@ __global__ void k_leaf_boxes(const typename Traits<D>::Point* __restrict__ sp, c
         for (int o = 16; o > 0; o >>= 1) T::merge(mine, T::shfl_xor(mine, o));
         if (lane == 0) sum1[base >> 5] = mine;
     }
-    karras(lkey, m, nmeta, nullptr, range_out, first_out);
 }
 
 // ---------------------------------------------------------------------------
@@ -1251,14 +1273,18 @@ void launch_lbvh(const void* sp, int dim, const int2* leafr, const uint64_t* lke
 {
     const unsigned g = grid_for(m_cap, 256, 152 * 16);
     const unsigned gl = grid_for(sum_levels_entries(m_cap) * 32, 256, 152 * 4);
+    // leaf keys that a block of the topology takes into shared memory: in runs
+    // of up to 64K points, which seldom have more tiles than that; larger runs
+    // keep the shared memory free for more blocks
+    const int keys = m_cap <= (1 << 16) ? (int)std::min<int64_t>(m_cap, 4096) : 0;
     // (the levels from 2 on: none while level 1 is read directly)
     const bool levels = sum_level_size(m_cap, 1) > SUM_DIRECT;
 #define LB_LAUNCH(D)                                                                                                  \
     do {                                                                                                              \
         using Bx = typename Traits<D>::Box;                                                                           \
-        launch(k_leaf_boxes<D>, g, 256, 0, s, static_cast<const typename Traits<D>::Point*>(sp), leafr, ctrl,              \
+        launch(k_leaf_boxes<D>, 2 * g, 256, sizeof(uint64_t) * keys, s, static_cast<const typename Traits<D>::Point*>(sp), leafr, ctrl, \
                                           static_cast<const Bx*>(dbox), static_cast<Bx*>(leafbox),                    \
-                                          static_cast<Bx*>(nsum), lkey, nmeta, range_out, nfirst);            \
+                                          static_cast<Bx*>(nsum), lkey, nmeta, range_out, nfirst, keys);      \
         if (levels) launch(k_box_levels<D>, gl, 256, 0, s, ctrl, static_cast<Bx*>(nsum));                                 \
     } while (0)
     GBD_DIM_SWITCH(dim, LB_LAUNCH)
