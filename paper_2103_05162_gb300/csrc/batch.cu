@@ -61,7 +61,7 @@ __device__ __forceinline__ float4 load_row(const InstDev& in, int64_t row)
 // the same for all lanes. (A search per row, nine dependent loads for 512
 // instances, and six atomics per 32 rows were most of the kernels that use
 // this: with 20.6M rows the bounds took 399 us, now 52; keys 203, now 119;
-// gather 238, now 160.) Sorted positions keep
+// gather 238, now 160 (240 where it also splits words).) Sorted positions keep
 // the instances' rows, so it serves them as well.
 template <int U, typename F>
 __device__ __forceinline__ void rows_by_instance(const int64_t* __restrict__ offs, int count, int64_t n, F f)
@@ -132,10 +132,11 @@ __global__ void k_bbounds(const int64_t* __restrict__ offs,
     if (__any_sync(FULL, bad) && lane == 0) atomicOr(nonfinite, 1u);
 }
 
-// key = (instance << lb) | Morton code of the point's cell in its instance's grid
+// key = (instance << lb) | Morton code of the point's cell in its instance's
+// grid; above the row, in one word (idx_bits of it), where both fit
 __global__ void k_bkeys(const int64_t* __restrict__ offs,
-                        const InstDev* __restrict__ inst, int count, int64_t n, int lb, uint64_t* __restrict__ keys,
-                        uint32_t* __restrict__ vals)
+                        const InstDev* __restrict__ inst, int count, int64_t n, int lb, int idx_bits,
+                        uint64_t* __restrict__ keys, uint32_t* __restrict__ vals)
 {
     stage_begin(offs, inst);
     const int lane = threadIdx.x & 31;
@@ -152,24 +153,36 @@ __global__ void k_bkeys(const int64_t* __restrict__ offs,
             c[0] = cell_index(floorf(__fmul_rn(__fsub_rn(v[u].x, in.lo[0]), in.scale[0])), in.cmax[0]);
             c[1] = cell_index(floorf(__fmul_rn(__fsub_rn(v[u].y, in.lo[1]), in.scale[1])), in.cmax[1]);
             c[2] = cell_index(floorf(__fmul_rn(__fsub_rn(v[u].z, in.lo[2]), in.scale[2])), in.cmax[2]);
-            keys[i] = ((uint64_t)b << lb) | interleave<3>(c);
-            vals[i] = (uint32_t)i;
+            const uint64_t key = ((uint64_t)b << lb) | interleave<3>(c);
+            keys[i] = idx_bits ? (key << idx_bits) | (uint64_t)i : key;
+            if (!idx_bits) vals[i] = (uint32_t)i;
         }
     });
 }
 
 __global__ void k_bgather(const int64_t* __restrict__ offs,
-                          const InstDev* __restrict__ inst, int count, const uint32_t* __restrict__ perm, int64_t n,
-                          float4* __restrict__ sp, const uint32_t* __restrict__ ctrl)
+                          const InstDev* __restrict__ inst, int count, uint32_t* __restrict__ perm, int64_t n,
+                          float4* __restrict__ sp, const uint32_t* __restrict__ ctrl,
+                          const uint64_t* __restrict__ words, int idx_bits, uint64_t* __restrict__ keys)
 {
-    stage_begin(offs, inst, perm, ctrl);
+    stage_begin(offs, inst, perm, ctrl, words);
     if (!stage_on(ctrl, -1)) return;  // a sort that gave up: stale permutation words
     const int lane = threadIdx.x & 31;
     rows_by_instance<4>(offs, count, n, [&](int b, int64_t r, int64_t se) {
         uint32_t row[4];
         float4 v[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) row[u] = perm[min(r + 32 * u + lane, se - 1)];
+        for (int u = 0; u < 4; ++u) {
+            const int64_t i = min(r + 32 * u + lane, se - 1);
+            if (idx_bits) {  // the word is split into the key and the row
+                const uint64_t w = __ldcs(words + i);
+                row[u] = (uint32_t)(w & ((1ull << idx_bits) - 1ull));
+                keys[i] = w >> idx_bits;
+                __stcs(perm + i, row[u]);
+            } else {
+                row[u] = perm[i];
+            }
+        }
 #pragma unroll
         for (int u = 0; u < 4; ++u) v[u] = load_row(inst[b], row[u]);
 #pragma unroll
@@ -411,7 +424,13 @@ cudaError_t enqueue_batch_stages(const BatchPlan& p, int64_t n, int count, int m
 {
     cudaError_t e;
     if ((e = cudaMemsetAsync(p.ctrl + CTRL_M, 0, 2 * sizeof(uint32_t), s)) != cudaSuccess) return e;
-    launch(k_bkeys, grid_n(n), 256, 0, s, p.offs, p.inst, count, n, lb, p.keys, p.vals);
+    // Key and row in one word where they fit: the four passes of 512 instances
+    // take 577 us instead of 691 for keys with values, of which the gather,
+    // which then writes both, takes 80 back.
+    int idx_bits = 1;
+    while ((1ll << idx_bits) < n) ++idx_bits;
+    if (idx_bits + key_bits > 64) idx_bits = 0;
+    launch(k_bkeys, grid_n(n), 256, 0, s, p.offs, p.inst, count, n, lb, idx_bits, p.keys, p.vals);
     note_launches(1);
     SortBuffers sb;
     sb.keys_alt = p.keys_alt;
@@ -422,10 +441,13 @@ cudaError_t enqueue_batch_stages(const BatchPlan& p, int64_t n, int count, int m
     sb.err = p.ctrl + CTRL_ABORT;  // a wait that runs out stops every later stage
     sb.ctl.abort = p.ctrl + CTRL_ABORT;
     bool in_alt = false;
-    if ((e = sort_pairs_u64(p.keys, p.vals, n, key_bits, sb, s, &in_alt)) != cudaSuccess) return e;
-    const uint64_t* keys = in_alt ? p.keys_alt : p.keys;
-    const uint32_t* perm = in_alt ? p.vals_alt : p.vals;
-    launch(k_bgather, grid_n(n), 256, 0, s, p.offs, p.inst, count, perm, n, p.sp, p.ctrl);
+    e = idx_bits ? sort_keys_u64(p.keys, n, idx_bits, key_bits, sb, s, &in_alt)
+                 : sort_pairs_u64(p.keys, p.vals, n, key_bits, sb, s, &in_alt);
+    if (e != cudaSuccess) return e;
+    const uint64_t* words = in_alt ? p.keys_alt : p.keys;
+    uint64_t* keys = in_alt == (idx_bits != 0) ? p.keys : p.keys_alt;
+    uint32_t* perm = in_alt && !idx_bits ? p.vals_alt : p.vals;
+    launch(k_bgather, grid_n(n), 256, 0, s, p.offs, p.inst, count, perm, n, p.sp, p.ctrl, words, idx_bits, keys);
     note_launches(1);
     if (algo == DBSCAN_ALGO_DENSEBOX) {
         if ((e = cudaMemsetAsync(p.db.pdense, 0, (size_t)n, s)) != cudaSuccess) return e;
