@@ -407,7 +407,7 @@ def run_gb300(args, rank: int, world: int) -> None:
         traffic = measured_traffic(n, top)
         if traffic is not None:
             traffic /= 1.0  # bytes per launch of the stage (one launch per step)
-    kernels = {"preprocess": "k_pre + k_list_claims", "main": "k_intra + k_kinds_* + k_main x3"}
+    kernels = {"preprocess": "k_pre + k_list_claims", "main": "k_intra + k_kinds + k_main"}
     counts = traversal_counts(n) if (algo == gb.ALGO_DENSEBOX and args.min_pts == 10) else None
     stage_frac_hbm = {k: model[k] / (stage_ms[k] / 1e3) / 1e9 / peak for k in stage_ms}
     if top in ("preprocess", "main") and counts is not None:
