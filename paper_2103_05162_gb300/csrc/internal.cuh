@@ -136,10 +136,19 @@ __device__ __forceinline__ float gap2_rn(float alo, float ahi, float blo, float 
 // ---------------------------------------------------------------------------
 // Pairs of fp32 values in one 64-bit register, for the packed f32x2
 // arithmetic of sm_100-family GPUs: each half is rounded to nearest even on
-// its own, so sub2 / add2 / mul2 give exactly __fsub_rn / __fadd_rn /
+// its own, so sub2 / add2 / sqr2 give exactly __fsub_rn / __fadd_rn /
 // __fmul_rn per half, in half the instructions.
+//
+// add2 is a multiply-add by a 1 that the assembler cannot know (constant
+// memory, which the host may write): fl(1 b + a) is fl(a + b). ptxas 13.0
+// contracts add.rn.f32x2 of a mul.rn.f32x2 to one fused multiply-add, in spite
+// of both .rn and of --fmad=false (a product by a literal 1 or with a literal
+// -0 added it folds away first); the last bit was then another in 21% of random
+// 3D distances, and pairs at eps fell on the wrong side of it. Distances of 2,432
+// blocks from shared memory: 3.48e12 a second, contracted 4.08e12, scalar 2.69e12.
 // ---------------------------------------------------------------------------
 typedef unsigned long long f32x2;
+static __constant__ f32x2 c_ones = 0x3f8000003f800000ull;
 
 __device__ __forceinline__ f32x2 pk2(float a, float b)
 {
@@ -160,7 +169,7 @@ __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b)
 __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
 {
     f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(c_ones), "l"(a));
     return r;
 }
 __device__ __forceinline__ f32x2 sqr2(f32x2 a)
