@@ -277,7 +277,7 @@ __global__ void k_est_count(const float* __restrict__ pts, int64_t n, int64_t st
         const unsigned long long key = cell_key<D>(pts + j * stride * D, g);
         uint32_t h = est_hash(key);
         for (int probe = 0; probe < EST_SLOTS; ++probe) {
-            const unsigned long long k = __ldg(&table[h]);
+            const unsigned long long k = table[h];
             if (k == key) {
                 atomicAdd(&sc[h], 1u);
                 break;
@@ -1000,7 +1000,7 @@ template <int D>
 __device__ __forceinline__ typename Traits<D>::Box ld_box(const typename Traits<D>::Box* b)
 {
     typename Traits<D>::Box r;
-    if constexpr (sizeof(typename Traits<D>::Box) == 32) ldg256(b, r.lo, r.hi);
+    if constexpr (sizeof(typename Traits<D>::Box) == 32) ld256(b, r.lo, r.hi);
     else r = *b;
     return r;
 }
@@ -1041,7 +1041,7 @@ __global__ void k_refit(uint32_t* __restrict__ ctrl, const int4* __restrict__ nm
                         const int32_t* __restrict__ nfirst, const typename Traits<D>::Box* __restrict__ leafbox,
                         const typename Traits<D>::Box* __restrict__ sum, typename Traits<D>::Node* __restrict__ nodes)
 {
-    stage_begin(nmeta, nfirst, sum);
+    stage_begin(nmeta, nfirst, leafbox, sum);
     using T = Traits<D>;
     using Box = typename T::Box;
     const int lane = threadIdx.x & 31;

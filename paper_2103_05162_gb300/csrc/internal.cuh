@@ -382,12 +382,21 @@ template <> struct Traits<3> {
 
 // A 32-byte record (two float4) in one 256-bit read-only load (sm_100 and
 // later); the address must be 32-byte aligned and the data read-only for the
-// kernel's lifetime.
+// kernel's lifetime: not written by the kernel before it, which it may overlap.
 __device__ __forceinline__ void ldg256(const void* p, float4& x, float4& y)
 {
     asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
         : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w), "=f"(y.x), "=f"(y.y), "=f"(y.z), "=f"(y.w)
         : "l"(p));
+}
+
+// The same by an ordinary load, for what the kernel before this one writes
+// (volatile, so that it stays after the wait for that kernel).
+__device__ __forceinline__ void ld256(const void* p, float4& x, float4& y)
+{
+    asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w), "=f"(y.x), "=f"(y.y), "=f"(y.z), "=f"(y.w)
+                 : "l"(p));
 }
 
 // The same through L2 (ld.global.cg), for records that other threads of the
@@ -617,9 +626,21 @@ __host__ __device__ __forceinline__ float ord2f(uint32_t u)
 // next one be scheduled meanwhile. A small run is a chain of some 20 kernels of
 // 3 to 10 us, and each saves the part of its launch that overlaps (1,000
 // points: 164 -> 117 us per run, 16,384: 245 -> 190). A kernel must not return
-// before stage_begin(): the order would not reach the kernel after it. The
-// pointers pass through an empty assembly statement, so that no load through
-// them (a read-only one above all) can be moved ahead of the wait.
+// before stage_begin(): the order would not reach the kernel after it.
+//
+// An overlapped kernel exists while the one before it still writes, so what
+// that one writes may not be read by read-only loads (ld.global.nc: __ldg,
+// ldg256, and what the compiler makes of a const __restrict__ parameter), whose
+// data has to stay as it is for the kernel's lifetime. What any older kernel
+// wrote is complete before this one can start (the one before it has passed
+// its own wait) and may be read either way. Hence
+//  * every const __restrict__ parameter goes through stage_begin: it comes out
+//    of an empty assembly statement, a pointer of which the compiler knows
+//    nothing, so its loads are ordinary ones and stay after the wait;
+//  * the kernels that take a DevArgs read the control words first and all else
+//    at addresses that depend on them or on what their atomics return;
+//  * __ldg and ldg256 are left to the caller's points and offsets, sorted
+//    points, leaf records and boxes and nodes, where an older kernel wrote them.
 //
 // Runs of more than OVERLAP_POINTS points are launched one after the other, as
 // without the attribute: their kernels fill the GPU in several waves, and

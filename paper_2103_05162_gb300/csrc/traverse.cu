@@ -968,7 +968,7 @@ struct PreWarp {
             int U = -1;
             if (lc >= 0) {
                 if (j0 >= lc) return;
-                if (j0 + lane < lc) U = __ldg(a.llist + (int64_t)L * LEAFCAP + j0 + lane);
+                if (j0 + lane < lc) U = a.llist[(int64_t)L * LEAFCAP + j0 + lane];
                 j0 += 32;
             } else {
                 if (walk_next<D>(a, wm, sp, nc, steps, m, qbox, e2, 0, lane) == 0) return;
@@ -1752,7 +1752,7 @@ struct MainWarp {
             int U = -1;
             if (lc >= 0) {
                 if (j0 >= lc) return;
-                if (!have && j0 + lane < lc) U = __ldg(a.llist + (int64_t)L * LEAFCAP + j0 + lane);
+                if (!have && j0 + lane < lc) U = a.llist[(int64_t)L * LEAFCAP + j0 + lane];
                 j0 += 32;
             } else {
                 if (walk_next<D>(a, wm, sp, nc, steps, m, qbox, e2, L + 1, lane) == 0) return;
@@ -1787,8 +1787,8 @@ __global__ void __maxnreg__(main_regs<D>()) k_main(const __grid_constant__ DevAr
     auto resolve = [&](int64_t idx) {
         // (a list per kind, taken as 2, 1, 0)
         if (idx >= total) L = -1;
-        else if (idx < c2) L = __ldg(&a.klist[2 * a.m_cap + idx]);
-        else L = __ldg(&a.klist[idx < c2 + c1 ? a.m_cap + (idx - c2) : idx - c2 - c1]);
+        else if (idx < c2) L = a.klist[2 * a.m_cap + idx];
+        else L = a.klist[idx < c2 + c1 ? a.m_cap + (idx - c2) : idx - c2 - c1];
     };
     int pend = 0;
     if (lane == 0) pend = (int)atomicAdd(&a.ctrl[CTRL_KIND_WORK], 1u);
@@ -1810,7 +1810,7 @@ __global__ void __maxnreg__(main_regs<D>()) k_main(const __grid_constant__ DevAr
         w.e = r.y & 0x7fffffff;
         w.cell = r.y < 0;
         int U = -1;
-        if (lane < lc) U = __ldg(a.llist + (int64_t)L * LEAFCAP + lane);
+        if (lane < lc) U = a.llist[(int64_t)L * LEAFCAP + lane];
         if (U <= L) U = -1;
         // a tile's points that take part: after preprocessing a non-core
         // point with no other point within eps takes part in no pair, and in
