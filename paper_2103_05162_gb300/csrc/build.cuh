@@ -244,6 +244,7 @@ void launch_karras_only(const uint64_t* lkey, int64_t m, int4* nmeta, int2* chil
 // traverse.cu
 constexpr int TRAVERSAL_SIBCAP = 8;   // sibling subtrees recorded per leaf
 constexpr int TRAVERSAL_LEAFCAP = 48; // leaves within eps listed per leaf
+constexpr int MAX_BLOCK = 1024;       // threads of a traversal block, at most
 
 struct ClusterArgs {
     const void* sp;        // sorted points

@@ -1187,8 +1187,8 @@ int dbscan_border_lists(void) { return g_tuning.border_lists; }
 dbscan_status dbscan_set_tuning(int block_size, float cell_factor)
 {
     t_err.clear();
-    if (block_size != 0 && (block_size < 32 || block_size > 1024 || block_size % 32 != 0))
-        return set_error(DBSCAN_ERR_INVALID_ARG, "block size must be a multiple of 32 in [32, 1024]");
+    if (block_size != 0 && (block_size < 32 || block_size > MAX_BLOCK || block_size % 32 != 0))
+        return set_error(DBSCAN_ERR_INVALID_ARG, "block size must be a multiple of 32 in [32, %d]", MAX_BLOCK);
     if (cell_factor != 0.0f && !(cell_factor > 0.0f && cell_factor <= 1.0f))
         return set_error(DBSCAN_ERR_INVALID_ARG, "cell factor must be in (0, 1]");
     g_tuning.block = block_size;

@@ -33,6 +33,9 @@
 // with one compare-and-swap (Sec. 3.2).
 #include <algorithm>
 #include <climits>
+#include <map>
+#include <mutex>
+#include <tuple>
 
 #include "build.cuh"
 
@@ -1967,16 +1970,31 @@ void count_phase(int phase, cudaStream_t s)
 #endif
 }
 
-// blocks of a persistent launch: as many as fit on all SMs at once
-int persistent_blocks(const void* kernel, int block, size_t smem)
+// Blocks of a persistent launch (as many as fit on all SMs at once), kept per
+// kernel, device and block size. Blocks from some 600 threads on take more
+// shared memory than a launch gets by default; that limit belongs to the kernel
+// on its device, so it is set once, to what the largest block takes: set to each
+// size at its first use, a smaller block's would lower it under a larger one's.
+cudaError_t persistent_blocks(const void* kernel, int block, size_t warp_smem, unsigned* out)
 {
+    static std::mutex mu;
+    static std::map<std::tuple<const void*, int, int>, unsigned> known;
     int dev = 0, sms = 0, per = 0;
-    // (large blocks: more shared memory than a launch gets by default)
-    if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, block, smem);
-    return (per > 0 ? per : 1) * (sms > 0 ? sms : 1);
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(mu);
+    unsigned& g = known[std::make_tuple(kernel, dev, block)];
+    if (!g) {
+        if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(warp_smem * (MAX_BLOCK / 32)))) != cudaSuccess ||
+            (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+            (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, block, warp_smem * (block / 32))) !=
+                cudaSuccess)
+            return e;
+        g = (unsigned)((per > 0 ? per : 1) * sms);
+    }
+    *out = g;
+    return cudaSuccess;
 }
 
 template <int D>
@@ -2013,28 +2031,19 @@ DevArgs<D> dev_args(const ClusterArgs& a)
     return d;
 }
 
+// (launch errors: cudaGetLastError)
 template <int D>
-void run_pre(const ClusterArgs& a, cudaStream_t s)
+cudaError_t run_persistent(void (*kernel)(DevArgs<D>), const ClusterArgs& a, cudaStream_t s)
 {
-    static int blocks[33] = {};
-    const size_t smem = sizeof(WarpMem<D>) * (size_t)(a.block / 32);
-    int& g = blocks[a.block / 32];
-    if (!g) g = persistent_blocks((const void*)k_pre<D>, a.block, smem);
-    launch(k_pre<D>, g, a.block, smem, s, dev_args<D>(a));
+    unsigned g = 0;
+    const cudaError_t e = persistent_blocks((const void*)kernel, a.block, sizeof(WarpMem<D>), &g);
+    if (e != cudaSuccess) return e;
+    launch(kernel, g, a.block, sizeof(WarpMem<D>) * (size_t)(a.block / 32), s, dev_args<D>(a));
+    return cudaSuccess;
 }
 
 template <int D>
-void run_main_walk(const ClusterArgs& a, cudaStream_t s)
-{
-    static int blocks[33] = {};
-    const size_t smem = sizeof(WarpMem<D>) * (size_t)(a.block / 32);
-    int& g = blocks[a.block / 32];
-    if (!g) g = persistent_blocks((const void*)k_main<D>, a.block, smem);
-    launch(k_main<D>, g, a.block, smem, s, dev_args<D>(a));
-}
-
-template <int D>
-void run_main(const ClusterArgs& a, cudaStream_t s)
+cudaError_t run_main(const ClusterArgs& a, cudaStream_t s)
 {
     const bool split = a.n >= SPLIT_INTRA;
     if (split && a.lcap > 0) {
@@ -2050,7 +2059,7 @@ void run_main(const ClusterArgs& a, cudaStream_t s)
         launch(k_kinds, (unsigned)gk, 256, 0, s, a.leafr, a.lsolid, a.ctrl, a.klist, a.m_cap);
         note_launches(1);
     }
-    run_main_walk<D>(a, s);
+    return run_persistent<D>(k_main<D>, a, s);
 }
 
 }  // namespace
@@ -2094,9 +2103,11 @@ cudaError_t launch_cluster_pre(const ClusterArgs& a, cudaStream_t s)
     // are always taken)
     if (a.min_pts <= 2 && !a.ncount) return cudaSuccess;
     count_phase(1, s);
-#define PRE_RUN(D) run_pre<D>(a, s)
+    cudaError_t e = cudaSuccess;
+#define PRE_RUN(D) e = run_persistent<D>(k_pre<D>, a, s)
     GBD_DIM_SWITCH(a.dim, PRE_RUN)
 #undef PRE_RUN
+    if (e != cudaSuccess) return e;
     note_launches(1);
     return cudaGetLastError();
 }
@@ -2104,9 +2115,11 @@ cudaError_t launch_cluster_pre(const ClusterArgs& a, cudaStream_t s)
 cudaError_t launch_cluster_main(const ClusterArgs& a, cudaStream_t s)
 {
     count_phase(2, s);
-#define MAIN_RUN(D) run_main<D>(a, s)
+    cudaError_t e = cudaSuccess;
+#define MAIN_RUN(D) e = run_main<D>(a, s)
     GBD_DIM_SWITCH(a.dim, MAIN_RUN)
 #undef MAIN_RUN
+    if (e != cudaSuccess) return e;
     note_launches(2);
     return cudaGetLastError();
 }
