@@ -520,7 +520,7 @@ dbscan_status run_batch(Workspace* w, int32_t count, const int64_t* offsets, con
         return set_error(DBSCAN_ERR_INVALID_ARG, "batches take an explicit algorithm (FDBSCAN or DENSEBOX)");
     const int64_t n = offsets[count];
     if (n == 0) return DBSCAN_OK;
-    t_overlap = n <= OVERLAP_POINTS;
+    const OverlapScope overlap(n);
     int max_mp = 1;
     for (int b = 0; b < count; ++b)
         if (min_pts[b] > max_mp) max_mp = min_pts[b];

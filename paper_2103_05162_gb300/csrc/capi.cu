@@ -473,7 +473,6 @@ dbscan_status build_index(Workspace* w, const Plan& p, StageTimer& T, const floa
                           float eps, int dense_mp, int algo, ClusterArgs& a, cudaStream_t s)
 {
     w->last_algo = algo == DBSCAN_ALGO_AUTO ? -2 : algo;  // -2: chosen on the device
-    t_overlap = n <= OVERLAP_POINTS;
     launch_run_begin(p.ctrl, algo, s);
     const float e2 = eps * eps;
     const bool fd = algo != DBSCAN_ALGO_DENSEBOX, db = algo != DBSCAN_ALGO_FDBSCAN;
@@ -620,6 +619,7 @@ dbscan_status build_index(Workspace* w, const Plan& p, StageTimer& T, const floa
 dbscan_status run_pipeline(Workspace* w, const float* points, int64_t n, int dim, float eps, int min_pts, int mode,
                            int algo, int32_t* labels_out, uint8_t* core_out, cudaStream_t s)
 {
+    const OverlapScope overlap(n);
     const int lcap = list_cap(min_pts, mode);
     TRY_CUDA(ensure_arena(w->main, workspace_bytes(n, dim, algo, min_pts, mode), s));
     Plan p;
@@ -655,6 +655,7 @@ dbscan_status run_pipeline(Workspace* w, const float* points, int64_t n, int dim
 dbscan_status run_core_flags(Workspace* w, const float* points, int64_t n, int dim, float eps, int min_pts, int algo,
                              uint8_t* core_out, int32_t* labels_scratch, cudaStream_t s)
 {
+    const OverlapScope overlap(n);
     const int cap_mp = min_pts < 2 ? 2 : min_pts;
     TRY_CUDA(ensure_arena(w->main, workspace_bytes_multi(n, dim, algo, cap_mp, DBSCAN_MODE_DBSCAN_STAR), s));
     Plan p;
@@ -682,6 +683,7 @@ dbscan_status run_core_flags(Workspace* w, const float* points, int64_t n, int d
 dbscan_status run_with_core(Workspace* w, const float* points, int64_t n, int dim, float eps, int min_pts, int mode,
                             int algo, const uint8_t* core_in, int32_t* labels_out, cudaStream_t s)
 {
+    const OverlapScope overlap(n);
     TRY_CUDA(ensure_arena(w->main, workspace_bytes(n, dim, algo, 3, DBSCAN_MODE_DBSCAN_STAR), s));
     Plan p;
     carve_plan(p, w->main.base, n, dim, algo, 0);
@@ -712,6 +714,7 @@ dbscan_status run_with_core(Workspace* w, const float* points, int64_t n, int di
 dbscan_status run_multi(Workspace* w, const float* points, int64_t n, int dim, float eps, const int32_t* min_pts,
                         int count, int mode, int algo, int32_t* labels_out, uint8_t* core_out, cudaStream_t s)
 {
+    const OverlapScope overlap(n);
     int max_mp = 1;
     for (int k = 0; k < count; ++k)
         if (min_pts[k] > max_mp) max_mp = min_pts[k];

@@ -661,8 +661,15 @@ __device__ __forceinline__ void stage_begin(T&... in)
 }
 
 constexpr int64_t OVERLAP_POINTS = 1 << 21;
-// whether this thread's launches overlap (set by the entry points, per call)
+// whether this thread's launches overlap: within the call that opened the scope
 extern thread_local bool t_overlap;
+struct OverlapScope {
+    bool before;
+    explicit OverlapScope(int64_t n) : before(t_overlap) { t_overlap = n <= OVERLAP_POINTS; }
+    ~OverlapScope() { t_overlap = before; }
+    OverlapScope(const OverlapScope&) = delete;
+    OverlapScope& operator=(const OverlapScope&) = delete;
+};
 
 template <typename... Params, typename... Args>
 inline void launch(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, Args&&... args)
