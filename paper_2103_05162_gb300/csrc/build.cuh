@@ -37,14 +37,12 @@ inline int fdbscan_bits(int dim)
 
 // Slots of the per-workspace control block (uint32 words in device memory).
 enum : int {
-    CTRL_NONFINITE = 8,  // nonzero if a coordinate is NaN/Inf (batches)
     CTRL_ERR = 9,        // device error bits (ERR_*) of earlier runs, kept until a host sync point reads them
     CTRL_M = 10,         // number of BVH leaves
     CTRL_NCELLS = 11,    // number of dense cells (DenseBox)
-    CTRL_WORK_PRE = 12,  // work counters of the persistent traversal kernels
+    CTRL_WORK_PRE = 12,  // work counter of the preprocessing kernel
     CTRL_KIND_COUNT = 16,  // 3 words: leaves per kind (0 tile, 1 solid tile, 2 dense cell leaf)
-    CTRL_KIND_FILL = 19,   // 3 words: fill counters of the per-kind leaf lists
-    CTRL_KIND_WORK = 22,   // 3 words: work counters of the per-kind main kernels
+    CTRL_KIND_WORK = 22,   // work counter of the main kernel
     CTRL_WORK_END = 25,    // end of the per-phase counters (cleared before each phase)
     CTRL_ABORT = 26,       // error bits of the current run (ERR_*): set, every later stage does nothing
     CTRL_ALGO = 27,        // the algorithm the current run uses (DBSCAN_ALGO_FDBSCAN / _DENSEBOX)

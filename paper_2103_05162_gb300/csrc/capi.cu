@@ -463,7 +463,7 @@ enum Stage { ST_BOUNDS, ST_KEYS, ST_SORT, ST_GATHER, ST_LEAVES, ST_LBVH, ST_INIT
 // Stages a1-a7: bounds, keys, sort, gather, leaves (DenseBox cells dense for
 // minPts = dense_mp), BVH. Fills the plan-dependent fields of `a`. Nothing
 // here waits for the device: the DenseBox grid is computed from the bounds
-// on the device (k_grid), the sort takes the passes the keys need there, and
+// on the device (k_bounds), the sort takes the passes the keys need there, and
 // the automatic choice (DBSCAN_ALGO_AUTO) enqueues both algorithms' key,
 // sort, gather and leaf stages, of which only the chosen chain runs
 // (CTRL_ALGO). A non-finite coordinate or a sort that gives up sets

@@ -83,30 +83,6 @@ struct __align__(16) PtN {
     float c[8];
 };
 
-// L2-coherent (L1-bypassing) copies of points, for the boxes the refit's
-// threads hand to one another
-__device__ __forceinline__ float4 ld_cg(const float4* p) { return __ldcg(p); }
-__device__ __forceinline__ float2 ld_cg(const float2* p) { return __ldcg(p); }
-__device__ __forceinline__ void st_cg(float4* p, const float4& v) { __stcg(p, v); }
-__device__ __forceinline__ void st_cg(float2* p, const float2& v) { __stcg(p, v); }
-template <int D>
-__device__ __forceinline__ PtN<D> ld_cg(const PtN<D>* p)
-{
-    PtN<D> r;
-    const float4* q = reinterpret_cast<const float4*>(p);
-    const float4 a = __ldcg(q), b = __ldcg(q + 1);
-    r.c[0] = a.x; r.c[1] = a.y; r.c[2] = a.z; r.c[3] = a.w;
-    r.c[4] = b.x; r.c[5] = b.y; r.c[6] = b.z; r.c[7] = b.w;
-    return r;
-}
-template <int D>
-__device__ __forceinline__ void st_cg(PtN<D>* p, const PtN<D>& v)
-{
-    float4* q = reinterpret_cast<float4*>(p);
-    __stcg(q, make_float4(v.c[0], v.c[1], v.c[2], v.c[3]));
-    __stcg(q + 1, make_float4(v.c[4], v.c[5], v.c[6], v.c[7]));
-}
-
 template <int D>
 __device__ __forceinline__ float dist2(const PtN<D>& a, const PtN<D>& b)
 {
@@ -178,14 +154,6 @@ __device__ __forceinline__ f32x2 sqr2(f32x2 a)
     asm("mul.rn.f32x2 %0, %1, %1;" : "=l"(r) : "l"(a));
     return r;
 }
-// gap_rn per half: max(lo - p, p - hi, 0)
-__device__ __forceinline__ f32x2 gap_rn2(f32x2 lo, f32x2 hi, f32x2 p)
-{
-    float a0, a1, b0, b1;
-    unpk2(sub2(lo, p), a0, a1);
-    unpk2(sub2(p, hi), b0, b1);
-    return pk2(fmaxf(fmaxf(a0, b0), 0.0f), fmaxf(fmaxf(a1, b1), 0.0f));
-}
 // gap2_rn per half, interval [alo, ahi] against the pair of intervals [blo, bhi]
 __device__ __forceinline__ f32x2 gap2_rn2(f32x2 alo, f32x2 ahi, f32x2 blo, f32x2 bhi)
 {
@@ -219,7 +187,6 @@ template <int D> struct Traits {
         for (int k = 0; k < 8; ++k) r.c[k] = k < D ? p[D * i + k] : 0.0f;
         return r;
     }
-    __device__ static __forceinline__ float coord(const Point& p, int k) { return p.c[k]; }
     __device__ static __forceinline__ Box point_box(const Point& p) { return Box{p, p}; }
     __device__ static __forceinline__ Box empty_box()
     {
@@ -310,7 +277,6 @@ template <> struct Traits<3> {
     {
         return make_float4(p[3 * i], p[3 * i + 1], p[3 * i + 2], 0.0f);
     }
-    __device__ static __forceinline__ float coord(const Point& p, int k) { return k == 0 ? p.x : (k == 1 ? p.y : p.z); }
     __device__ static __forceinline__ Box point_box(const Point& p) { return Box{p, p}; }
     __device__ static __forceinline__ Box empty_box()
     {
@@ -399,23 +365,6 @@ __device__ __forceinline__ void ld256(const void* p, float4& x, float4& y)
                  : "l"(p));
 }
 
-// The same through L2 (ld.global.cg), for records that other threads of the
-// running kernel write; volatile, so that it stays after the acquire that
-// orders it.
-__device__ __forceinline__ void ldcg256(const void* p, float4& x, float4& y)
-{
-    asm volatile("ld.global.cg.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w), "=f"(y.x), "=f"(y.y), "=f"(y.z), "=f"(y.w)
-                 : "l"(p)
-                 : "memory");
-}
-__device__ __forceinline__ void stcg256(void* p, const float4& x, const float4& y)
-{
-    asm volatile("st.global.cg.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(x.x), "f"(x.y), "f"(x.z),
-                 "f"(x.w), "f"(y.x), "f"(y.y), "f"(y.z), "f"(y.w)
-                 : "memory");
-}
-
 template <> struct Traits<2> {
     using Point = float2;
     struct Box { float4 lo, hi; };  // z unused
@@ -425,7 +374,6 @@ template <> struct Traits<2> {
     {
         return make_float2(p[2 * i], p[2 * i + 1]);
     }
-    __device__ static __forceinline__ float coord(const Point& p, int k) { return k == 0 ? p.x : p.y; }
     __device__ static __forceinline__ Box point_box(const Point& p)
     {
         return Box{make_float4(p.x, p.y, 0.f, 0.f), make_float4(p.x, p.y, 0.f, 0.f)};

@@ -69,29 +69,6 @@ template <int D> struct NB {
         r.m = __ldg(&n[i].m);
         return r;
     }
-    __device__ static __forceinline__ typename T::Box box_l(const typename T::Node& n)
-    {
-        typename T::Box b = T::empty_box();
-#pragma unroll
-        for (int k = 0; k < D; ++k) { b.lo.c[k] = n.ax[k].x; b.hi.c[k] = n.ax[k].z; }
-        return b;
-    }
-    __device__ static __forceinline__ typename T::Box box_r(const typename T::Node& n)
-    {
-        typename T::Box b = T::empty_box();
-#pragma unroll
-        for (int k = 0; k < D; ++k) { b.lo.c[k] = n.ax[k].y; b.hi.c[k] = n.ax[k].w; }
-        return b;
-    }
-    __device__ static __forceinline__ void pd2(const typename T::Node& n, const PP& p, float& dl, float& dr)
-    {
-        GBD_COUNT(CNT_BOX, 2);
-        f32x2 s = sqr2(gap_rn2(pk2(n.ax[0].x, n.ax[0].y), pk2(n.ax[0].z, n.ax[0].w), p.c[0]));
-#pragma unroll
-        for (int k = 1; k < D; ++k)
-            s = add2(s, sqr2(gap_rn2(pk2(n.ax[k].x, n.ax[k].y), pk2(n.ax[k].z, n.ax[k].w), p.c[k])));
-        unpk2(s, dl, dr);
-    }
     __device__ static __forceinline__ void bd2(const typename T::Node& n, const typename T::Box& q, float& dl,
                                                float& dr)
     {
@@ -136,23 +113,6 @@ template <> struct NB<3> {
         r.m = make_int4(__float_as_int(mf.x), __float_as_int(mf.y), __float_as_int(mf.z), __float_as_int(mf.w));
         return r;
     }
-    __device__ static __forceinline__ T::Box box_l(const T::Node& n)
-    {
-        return T::Box{make_float4(n.a.x, n.b.x, n.c.x, 0.f), make_float4(n.a.z, n.b.z, n.c.z, 0.f)};
-    }
-    __device__ static __forceinline__ T::Box box_r(const T::Node& n)
-    {
-        return T::Box{make_float4(n.a.y, n.b.y, n.c.y, 0.f), make_float4(n.a.w, n.b.w, n.c.w, 0.f)};
-    }
-    // squared point-to-box distances of both children (box_dist2's order)
-    __device__ static __forceinline__ void pd2(const T::Node& n, const PP& p, float& dl, float& dr)
-    {
-        GBD_COUNT(CNT_BOX, 2);
-        f32x2 s = sqr2(gap_rn2(pk2(n.a.x, n.a.y), pk2(n.a.z, n.a.w), p.x));
-        s = add2(s, sqr2(gap_rn2(pk2(n.b.x, n.b.y), pk2(n.b.z, n.b.w), p.y)));
-        s = add2(s, sqr2(gap_rn2(pk2(n.c.x, n.c.y), pk2(n.c.z, n.c.w), p.z)));
-        unpk2(s, dl, dr);
-    }
     // squared box-to-box distances of both children from q (box_box_dist2's order)
     __device__ static __forceinline__ void bd2(const T::Node& n, const T::Box& q, float& dl, float& dr)
     {
@@ -186,21 +146,6 @@ template <> struct NB<2> {
         T::Node r;
         r.a = __ldg(&n[i].a); r.b = __ldg(&n[i].b); r.m = __ldg(&n[i].m);
         return r;
-    }
-    __device__ static __forceinline__ T::Box box_l(const T::Node& n)
-    {
-        return T::Box{make_float4(n.a.x, n.b.x, 0.f, 0.f), make_float4(n.a.z, n.b.z, 0.f, 0.f)};
-    }
-    __device__ static __forceinline__ T::Box box_r(const T::Node& n)
-    {
-        return T::Box{make_float4(n.a.y, n.b.y, 0.f, 0.f), make_float4(n.a.w, n.b.w, 0.f, 0.f)};
-    }
-    __device__ static __forceinline__ void pd2(const T::Node& n, const PP& p, float& dl, float& dr)
-    {
-        GBD_COUNT(CNT_BOX, 2);
-        f32x2 s = sqr2(gap_rn2(pk2(n.a.x, n.a.y), pk2(n.a.z, n.a.w), p.x));
-        s = add2(s, sqr2(gap_rn2(pk2(n.b.x, n.b.y), pk2(n.b.z, n.b.w), p.y)));
-        unpk2(s, dl, dr);
     }
     __device__ static __forceinline__ void bd2(const T::Node& n, const T::Box& q, float& dl, float& dr)
     {
@@ -441,22 +386,6 @@ struct DevArgs {
     int32_t* llist;
     int16_t* lcount;
 };
-
-template <int D>
-__device__ __forceinline__ float box_box(const typename Traits<D>::Box& a, const typename Traits<D>::Box& b)
-{
-    return Traits<D>::box_box_dist2(a, b);
-}
-template <>
-__device__ __forceinline__ float box_box<3>(const Traits<3>::Box& a, const Traits<3>::Box& b)
-{
-    return Traits<3>::box_box_dist2(a, b.lo.x, b.lo.y, b.lo.z, b.hi.x, b.hi.y, b.hi.z);
-}
-template <>
-__device__ __forceinline__ float box_box<2>(const Traits<2>::Box& a, const Traits<2>::Box& b)
-{
-    return Traits<2>::box_box_dist2(a, b.lo.x, b.lo.y, b.hi.x, b.hi.y);
-}
 
 // eps^2, minPts and the traversal start of the tile's instance
 struct TileParams {
