@@ -857,7 +857,7 @@ __global__ void k_box_levels(const uint32_t* __restrict__ ctrl, typename Traits<
 // end of its range and the split come from the common-prefix length delta of
 // the sorted leaf keys; equal keys are told apart by the leaf index.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int kdelta(const uint64_t* __restrict__ k, int64_t m, int64_t i, int64_t j)
+__device__ __forceinline__ int kdelta(const uint64_t* k, int64_t m, int64_t i, int64_t j)
 {
     if (j < 0 || j >= m) return -1;
     const uint64_t a = k[i], b = k[j];
@@ -865,7 +865,7 @@ __device__ __forceinline__ int kdelta(const uint64_t* __restrict__ k, int64_t m,
     return 64 + __clz((int)((uint32_t)i ^ (uint32_t)j));
 }
 
-__device__ __forceinline__ void karras(const uint64_t* __restrict__ lkey, int64_t m, int4* __restrict__ nmeta,
+__device__ __forceinline__ void karras(const uint64_t* lkey, int64_t m, int4* __restrict__ nmeta,
                                        int2* __restrict__ child_out, int2* __restrict__ range_out,
                                        int32_t* __restrict__ first_out, unsigned block, unsigned blocks)
 {
@@ -1007,8 +1007,8 @@ __device__ __forceinline__ typename Traits<D>::Box ld_box(const typename Traits<
 
 // union of leaf boxes a..b (inclusive), by the whole warp (all lanes, same a, b)
 template <int D>
-__device__ typename Traits<D>::Box range_box(const typename Traits<D>::Box* __restrict__ leafbox,
-                                             const typename Traits<D>::Box* __restrict__ sum, int64_t m, int64_t a,
+__device__ typename Traits<D>::Box range_box(const typename Traits<D>::Box* leafbox,
+                                             const typename Traits<D>::Box* sum, int64_t m, int64_t a,
                                              int64_t b, int lane)
 {
     using T = Traits<D>;

@@ -584,7 +584,8 @@ __host__ __device__ __forceinline__ float ord2f(uint32_t u)
 // its own wait) and may be read either way. Hence
 //  * every const __restrict__ parameter goes through stage_begin: it comes out
 //    of an empty assembly statement, a pointer of which the compiler knows
-//    nothing, so its loads are ordinary ones and stay after the wait;
+//    nothing, so its loads are ordinary ones and stay after the wait; a device
+//    function that reads what the kernel before wrote takes plain pointers;
 //  * the kernels that take a DevArgs read the control words first and all else
 //    at addresses that depend on them or on what their atomics return;
 //  * __ldg and ldg256 are left to the caller's points and offsets, sorted

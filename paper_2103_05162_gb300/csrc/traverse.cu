@@ -983,7 +983,7 @@ __global__ void __maxnreg__(traversal_regs<D>()) k_pre(const __grid_constant__ D
 // holds all its neighbours outside its tile; it joins the cluster of the first
 // core one (Algorithm 3's claim of a border point, Sec. 3.2, made here from the
 // border's side). Neighbours inside the tile are k_intra's, afterwards.
-__device__ __forceinline__ void list_claim(const int32_t* __restrict__ nlist, int lcap, const uint8_t* __restrict__ nbr,
+__device__ __forceinline__ void list_claim(const int32_t* nlist, int lcap, const uint8_t* nbr,
                                            const uint8_t* core, int32_t* labels, int64_t q)
 {
     const int k = nbr[q];

@@ -46,3 +46,17 @@ def test_read_only_loads_are_of_older_data():
             code = re.sub(r"//.*", "", f.read())
         for m in re.finditer(r"__ldg\([^;]*", code):
             assert re.match(older, m.group(0)), f"{os.path.basename(path)}: {m.group(0)}"
+
+
+def test_device_functions_take_plain_pointers_to_newer_data():
+    # const __restrict__ is left to the caller's points and offsets and to the
+    # traversals' boxes
+    found = set()
+    for path in glob.glob(os.path.join(CSRC, "*.cu*")):
+        with open(path) as f:
+            s = f.read()
+        for m in re.finditer(r"__device__ [^;{}()]*?(\w+)\(([^{};]*?)\)\s*(?:const)?\s*\{", s):
+            names = set(re.findall(r"const\s+[\w:<> ]*?\*\s*__restrict__\s+(\w+)", m.group(2)))
+            assert names <= {"pts", "p", "offs", "boxes"}, f"{os.path.basename(path)}: {m.group(1)}: {sorted(names)}"
+            found |= names
+    assert found == {"pts", "p", "offs", "boxes"}
