@@ -60,8 +60,8 @@ __device__ __forceinline__ float4 load_row(const InstDev& in, int64_t row)
 // searched once per warp and followed from there, so that its parameters are
 // the same for all lanes. (A search per row, nine dependent loads for 512
 // instances, and six atomics per 32 rows were most of the kernels that use
-// this: with 20.6M rows the bounds took 399 us, now 52; keys 203, now 119;
-// gather 238, now 160 (240 where it also splits words).) Sorted positions keep
+// this: with 20.6M rows the bounds took 399 us, now 53; keys 203, now 120;
+// gather 238, now 160 (235 where it also splits words).) Sorted positions keep
 // the instances' rows, so it serves them as well.
 template <int U, typename F>
 __device__ __forceinline__ void rows_by_instance(const int64_t* __restrict__ offs, int count, int64_t n, F f)

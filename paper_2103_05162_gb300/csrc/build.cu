@@ -452,12 +452,12 @@ __global__ void k_gather_packed(const float* __restrict__ pts, const uint64_t* _
 // point, and the box of a cell larger than a tile goes to dbox[first point /
 // 32] (more than 32 points: no two such cells share a slot) for the leaf boxes.
 // Bound by the latency of its loads. Batch of 512 instances (cells of up to
-// 29,000 points): 350 us, one warp walking one run after another 932, a thread
+// 29,000 points): 376 us, one warp walking one run after another 932, a thread
 // per run of up to 64 points 840, groups of 8 lanes 428; 3.9M 2D blob points
-// (few large cells): the leaves stage 215 us instead of 2300; 16.8M halos 121
+// (few large cells): the leaves stage 215 us instead of 2300; 16.8M halos 127
 // instead of 85. The leaf boxes, which walked the large cells again, fell from
-// 511 to 29 us on the batch and from 119 to 60 on the halos. pdense must be
-// zero on entry.
+// 511 to 38 us on the batch and from 119 to 76 on the halos, with the topology
+// that is now in the same launch. pdense must be zero on entry.
 //
 // Batches: the key's bits from lb up are the instance, whose minPts and eps^2
 // are read from mps and e2s (null: min_pts and e2).
@@ -650,7 +650,7 @@ __device__ __forceinline__ K shfl_key(K v, int src)
 // them, k_leaf_records numbers them and writes the leaf records, a leaf's end
 // by the thread that finds the next start. Flags by key probes and ballots, a
 // three-kernel scan, starts and records took 284 us on 16.8M halos in seven
-// launches; these take 111 and 50. (One kernel with a decoupled look-back took 186:
+// launches; these take 112 and 63. (One kernel with a decoupled look-back took 186:
 // the blocks stood at its barrier while their offsets came.)
 constexpr int LEAF_T = TILE;
 static_assert(LEAF_T == 32, "windows of one warp");
@@ -913,7 +913,7 @@ __global__ void k_karras(const uint64_t* __restrict__ lkey, int64_t m, int4* __r
 // The topology (K7) needs nothing of them, nor they of it: the odd blocks of
 // the same launch do it. Both are chains of loads: one after the other in the
 // same threads took 17 us on 16,384 blob points (12 on 1,000, 91 on 16.8M
-// halos), this takes 10 (7.5, 78).
+// halos), this takes 10 (9, 76).
 // ---------------------------------------------------------------------------
 template <int D>
 __global__ void k_leaf_boxes(const typename Traits<D>::Point* __restrict__ sp, const int2* __restrict__ leafr,

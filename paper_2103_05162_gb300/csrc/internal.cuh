@@ -572,9 +572,10 @@ __host__ __device__ __forceinline__ float ord2f(uint32_t u)
 // programmatic dependent of the one before it on the stream, it waits there
 // for that kernel to be complete (and its writes to be visible), and lets the
 // next one be scheduled meanwhile. A small run is a chain of some 20 kernels of
-// 3 to 10 us, and each saves the part of its launch that overlaps (1,000
-// points: 164 -> 117 us per run, 16,384: 245 -> 190). A kernel must not return
-// before stage_begin(): the order would not reach the kernel after it.
+// 3 to 10 us, and each saves the part of its launch that overlaps (16,384
+// halos: 233 -> 179 us per run, 262,144: 372 -> 331; 262,144 road points 246 ->
+// 214). A kernel must not return before stage_begin(): the order would not
+// reach the kernel after it.
 //
 // An overlapped kernel exists while the one before it still writes, so what
 // that one writes may not be read by read-only loads (ld.global.nc: __ldg,
@@ -592,9 +593,13 @@ __host__ __device__ __forceinline__ float ord2f(uint32_t u)
 //    points, leaf records and boxes and nodes, where an older kernel wrote them.
 //
 // Runs of more than OVERLAP_POINTS points are launched one after the other, as
-// without the attribute: their kernels fill the GPU in several waves, and
-// blocks of the next one that wait beside the last wave cost 1 to 3% (8M and
-// 21.6M points) where the launches are 1% of the run.
+// without the attribute: their kernels fill the GPU in several waves, beside the
+// last of which the blocks of the next one take room. Up to that size overlap
+// gains or costs nothing (2,097,152 points: 885 -> 870 us halos, 739 -> 701
+// roads, 705 -> 663 blobs; 1,048,576 halos 607 either way). Above it, it would
+// still gain 1 to 6% at 3M to 6M points and 1% on 8.4M halos, and would lose
+// 0.3% on 8.4M road points and 16.8M halos: the line is a safe one, not the
+// best one.
 // ---------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ void after_wait(T& p)

@@ -330,8 +330,8 @@ __global__ void __launch_bounds__(THREADS, VALS ? 3 : 4)
 // beforehand and nothing is looked up. Its keys stay in registers and shared
 // memory between the passes. A pass of a sort so small is a launch of 4 us and
 // a round trip through L2: six passes and their histogram took 30 us on 1,000
-// points, this takes 7; a full tile 14, and a run of 4,096 points 90 us where
-// one of 4,097, by the general passes, takes 96.
+// points, this takes 7; a full tile 14, and a run of 4,096 3D blob points 124 us
+// where one of 4,097, by the general passes, takes 137 (FDbscan 124 either way).
 template <typename K, bool VALS>
 __global__ void __launch_bounds__(THREADS) k_sort_tile(K* k0, uint32_t* v0, K* k1, uint32_t* v1, int n, int shift0,
                                                        int passes, SortCtl ctl)

@@ -410,7 +410,7 @@ __device__ __forceinline__ TileParams tile_params(const DevArgs<D>& a, int L)
 // says on which side the leaf lies, so a level is one dependent load, and the
 // upper levels are the same for all lanes. Climbing from the leaf took three
 // per level (parent, its children, the sibling's box) and 409 us for the lists
-// of 16.8M halos, where this takes 366: most of it is the walk below the
+// of 16.8M halos, where this takes 363: most of it is the walk below the
 // siblings.
 //
 // Returns the number of siblings (-1: more than SIBCAP); the first SIBCAP go
@@ -563,12 +563,15 @@ __device__ __forceinline__ int walk_take(WarpMem<D>& wm, int& nc, int lane)
 // a walk deeper than LL_STACK gives up its list as well)
 constexpr int LL_THREADS = 256;
 constexpr int LL_STACK = 48;
-// Up to so many leaves per warp of the launch, a warp makes a list: a
-// thread's walk is a chain of one load per node, a warp's of one per level or
-// so (16,384 blob points: 42 us by threads, 19 by warps). With more leaves
-// than the resident threads can take two each, threads do as well (262,144
-// halos, 4 leaves per warp: 57 us either way) or better (524,287 road points,
-// 6 per warp: 25 us by threads, 56 by warps).
+// Up to so many leaves per warp of the launch (of 8 in each of up to 1,216
+// blocks, half of which are resident at once), a warp makes a list: a thread's
+// walk is a chain of one load per node, a warp's of one per level or so (16,384
+// blob points: 42 us by threads, 19 by warps). With more leaves, threads keep
+// more walks in flight. Whole runs by threads and by warps, in us: below the
+// line blobs 349 and 294 (262,144), 500 and 441 (1M), halos 358 and 331
+// (262,144), roads, whose walks are short, 202 and 214 (262,144); above it
+// halos 446 and 433 (524,287), 606 and 666 (1M), 4265 and 6200 (16.8M), roads
+// 278 and 308 (524,287).
 constexpr int LL_ROUNDS = 2;
 
 // Leaf L's list by a whole warp: the same list in the same order (the nearest
@@ -696,9 +699,12 @@ __device__ __forceinline__ int next_leaf(uint32_t* ctr)
     return __shfl_sync(FULL, L, 0);
 }
 
-// Register caps of the preprocessing kernel, the fastest measured: 48 in 3D
-// (16.8M halos 1356 us, 56: 1397), 56 in 2D (4.2M road points 314, 48: 328), 80 in
-// 5D (400K points 239, 96: 252)
+// Register caps of the preprocessing kernel: 48 in 3D (16.8M halos 1356 us when
+// taken, 56: 1397), 56 in 2D (4.2M road points 314, 48: 328), 80 in 5D (400K points
+// 239, 96: 252). Whole runs with this and the main phase's caps 8 to 24 lower or
+// 8 to 32 higher, 2D to 8D, both algorithms: lower -1 to 8% slower; higher 2 to
+// 8% slower from 400,000 points in 4D to 8D and 0.5 to 2% on 4.2M points, up to
+// 1.5% faster in 2D and 3D and at 20,000 points.
 template <int D>
 constexpr int traversal_regs()
 {
@@ -720,10 +726,9 @@ constexpr int main_regs()
 // and every 32 of them (or the last) are tested against the queries, looping
 // over the smaller side. The order of the list and of the points in a leaf is
 // kept, so a query's neighbours are found in the order of the lists.
-// Issue-bound (75% of the slots; 1700 instructions per tile on 16.8M halos,
-// a quarter of them the tile's own pairs): visiting leaf by leaf, with a test
-// of each query against each leaf's box, took 1580 us there and 338 us on 400K
-// 5D points, this takes 1350 and 239 us.
+// Issue-bound (79% of the slots on 4.2M halos): visiting leaf by leaf, with a
+// test of each query against each leaf's box, took 1580 us on 16.8M halos and
+// 338 us on 400K 5D points, this takes 1337 and 235 us.
 constexpr int FEW_QUERIES = 8;
 
 template <int D>
@@ -756,7 +761,7 @@ struct PreWarp {
         if (2 * __popc(am) < n) {
             // lane per staged point, looping over the queries: a step of it
             // costs as much as a step of the other loop, which takes two
-            // staged points (16.8M halos 1397 us, 1461 without the factor)
+            // staged points (16.8M halos, when taken: 1397 us, 1461 without the factor)
             const bool in = lane < n;
             const P rp = wm.soa.get(lane);
             const int ri = wm.idx[lane];
@@ -1001,8 +1006,11 @@ __device__ __forceinline__ void list_claim(const int32_t* nlist, int lcap, const
 // kind, which saves two launches of 5 us each. From SPLIT_INTRA points on both
 // are kernels of their own: a thread per point has more of the lists' scattered
 // reads in flight, and k_intra's warps take their leaves one by one, far apart,
-// instead of consecutive ones of alike cost (16.8M halos: 247 + 80 + 19 us
-// against 415; 512K road points: 36 against 30 + 10 + 11).
+// instead of consecutive ones of alike cost. Whole runs in one and in three
+// kernels, in us: blobs 354 and 367 (524,287), 663 and 708 (2.1M), 962 and 1084
+// (4.2M); halos 870 and 887 (2.1M), 1435 and 1425 (4.2M), 1848 and 1818 (6M), 4335
+// and 4266 (16.8M); roads 278 and 277 (524,287), 701 and 706 (2.1M), 1370 and
+// 1380 (4.2M), 2625 and 2672 (8.4M): the line is where the halos turn.
 constexpr int64_t SPLIT_INTRA = 1 << 22;
 __global__ void k_list_claims(const int32_t* __restrict__ nlist, int lcap, const uint8_t* __restrict__ nbr,
                               const uint8_t* core, int32_t* labels, int64_t n)
@@ -1227,7 +1235,7 @@ __global__ void k_kinds(const int2* __restrict__ leafr, const uint8_t* __restric
 // pair that shared a root at any time needs no test. Testing the pairs first
 // and looking at the sets of those within eps, one leaf after another, took
 // 1241 us on 16.8M halos, 1524 us on 8M halos at minPts 2 and 1243 us on 400K
-// 5D points; this takes 514, 943 and 515 us (kernel times).
+// 5D points; this takes 495, 939 and 480 us (kernel times).
 // ---------------------------------------------------------------------------
 
 // What a point can still do, by its code: the root of its set (core points;
